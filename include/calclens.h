@@ -175,8 +175,9 @@ int clc_degrade(clc_ctx* ctx, const double* map_fine, int nside_fine, double* ma
 /* ------------------------------------------------------------------------ */
 /* Step 2: spherical-harmonic transforms and the SHT Poisson solve (Sec. 3.2) */
 
-/* Limit the FP64 Legendre table (sum over m of (lmax + 2 - m) * 2 nside
- * doubles; 262 GB at nside 2048, lmax 4096) to `bytes` (0 = the free device
+/* Limit the Legendre table of the FP64 transforms (16 bytes per (l, m, ring)
+ * in 64 x 64 blocks, about 0.7 of the sum over m of (lmax + 2 - m) * 2 nside
+ * of them: 7 GB at nside 512, lmax 1024) to `bytes` (0 = the free device
  * memory decides).  Larger tables are built and used one order range m0..m1
  * at a time inside each FP64 SHT call (same results; the recurrence is then
  * recomputed per call). */

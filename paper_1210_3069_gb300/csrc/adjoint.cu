@@ -898,8 +898,6 @@ static int sht_poisson_adjoint(clc_gal_tape* T, const clc_derivs& Fb, double* kb
   int rc;
   auto plan = get_fft_plan(ctx, ns, &rc);
   if (rc) return rc;
-  auto tab = get_legendre_table(ctx, ns, L, &rc);
-  if (rc) return rc;
   const int ldf = 4 * ns - 1;
   const size_t fq = (size_t)ldf * (L + 1);
   const long long Q = alm_idx(L + 1, L + 1, L + 1) + 1;
@@ -927,8 +925,12 @@ static int sht_poisson_adjoint(clc_gal_tape* T, const clc_derivs& Fb, double* kb
   CLC_LAUNCH(ctx, "k_spec_adjoint", k_spec_adjoint, g1, 128, 0, ns, L, Fh, fq, ldf, Gb, fq);
   if ((rc = launch_check(ctx, "k_spec_adjoint"))) return rc;
   // transposed Legendre synthesis: Legendre analysis up to l = lmax + 1
-  for (int q = 0; q < 3; ++q)
-    if ((rc = legendre_analysis(ctx, *tab, Gb + q * fq, ldf, rb + q * Q, L + 1))) return rc;
+  const double2* gq[3] = {Gb, Gb + fq, Gb + 2 * fq};
+  double2* rq[3] = {rb, rb + Q, rb + 2 * Q};
+  if ((rc = for_each_table(ctx, ns, L, [&](const LegendreTable& T) {
+         return legendre_analysis_cols(ctx, T, 3, gq, nullptr, ldf, rq, L + 1);
+       })))
+    return rc;
   dim3 g2((L + 1 + 127) / 128, L + 1);
   const double w = 4.0 * kPi / (12.0 * (double)ns * ns);
   CLC_LAUNCH(ctx, "k_poisson_adjoint", k_poisson_adjoint, g2, 128, 0, rb, Q, L, w, kt);

@@ -55,7 +55,7 @@ struct clc_ctx {
   size_t table_budget = 0;  // FP64 Legendre table limit in bytes (0: device memory decides)
   std::map<std::tuple<int, int, int, int>, std::shared_ptr<clc::TcBatch>> tc_batches;
   // growable scratch buffers, reused across calls on this context's stream
-  clc::Buffer scratch[8];
+  clc::Buffer scratch[10];
 };
 
 namespace clc {

@@ -1,20 +1,61 @@
 // Legendre step of the SHT (paper Sec. 3.2; the associated-Legendre
-// recurrence of Press et al. 2007 Sec. 6.7) in FP64.
+// recurrence of Press et al. 2007 Sec. 6.7) with the accuracy of FP64, on the
+// tcgen05 tensor cores.
 //
-// The table lambda_lm(z_r) is built once per (Nside, lmax) with the
-// three-term recurrence in l, started from
-// lambda_mm = (-1)^m sqrt((2m+1)!! / (4 pi (2m)!!)) sin^m(theta) carried as a
-// mantissa and a power-of-two exponent (sin^m theta underflows FP64 near the
-// poles at large m).  Analysis and synthesis are then per-m matrix-vector
-// products over the northern rings, using lambda_lm(-z) = (-1)^(l+m) lambda_lm(z)
-// for the southern mirror rings.  Layout [m][l][r] keeps ring index r
-// contiguous: the build writes, the synthesis reads (thread per ring) and the
-// analysis reads (warp per l, lanes over rings) all coalesced.
+// lambda_lm(z_r) is built once per (Nside, lmax) with the three-term
+// recurrence in l in FP64, started from lambda_mm = (-1)^m sqrt((2m+1)!! /
+// (4 pi (2m)!!)) sin^m(theta) carried as a mantissa and a power-of-two
+// exponent (sin^m theta underflows FP64 near the poles at large m).  Analysis
+// and synthesis are then per-m matrix products over the northern rings, using
+// lambda_lm(-z) = (-1)^(l+m) lambda_lm(z) for the southern mirror rings.
+//
+// The products are exact integer arithmetic (the error-free splitting of
+// Ozaki et al. 2012, "Error-free transformations of matrix multiplication"):
+// a table row and a data column are scaled by powers of two to integers of at
+// most 62 bits and written as eight signed base-256 digits, small integers
+// that FP16 holds exactly.  Digit products are at most 2^14, so an FP32
+// accumulator adds the up to 8 digit pairs i + j = g of 128 terms without
+// rounding (8 * 128 * 2^14 = 2^24); the sums of each g <= 7 are collected in
+// 64-bit integers and rounded once.  Digit pairs with g > 7 lie below 2^-62 of
+// the largest term and are left out.  The result does not depend on the order
+// of summation.  Rings where lambda_lm is small for every l (towards the
+// poles) are scaled up by 2^cexp <= 2^24 first.
+//
+// Eight digits, not seven: the scale is the largest value of a row or column,
+// while the FP64 sums this replaces keep every term's own 53 bits.  Near the
+// poles the low degrees, whose coefficients are the largest, have tiny
+// lambda_lm, and the Hessian multiplies the sum by m^2 / sin^2 theta (up to
+// 1.5 nside^2): with seven digits (54 bits) the error of u_pp at nside 512,
+// lmax 1024 was 2.2e-12 against 3.1e-14 of plain FP64 sums.
+//
+// Why digits on the tensor cores: the FP64 pipe does 2 FMA per clock and SM,
+// 0.63e12 per second on the chip, and a plane's transforms take 2 FMA per
+// table value forward and 6 back; read from HBM as eight FP16 planes (16 bytes,
+// 0.42e12 values per second) a value serves up to 16 columns at once, so both
+// directions are bound by the table traffic.  At nside 512, lmax 1024 the
+// FP64 kernels took 2.2 ms (analysis), 11.8 ms (synthesis of the three sums)
+// and 53.4 ms (spin-2 sums of two fields); the solve went from 19.2 to 7.8 ms
+// and the four spectra from 63.2 to 7.1 ms.
+#include <algorithm>
 #include <cmath>
 
 #include "legendre.cuh"
+#include "umma.cuh"
 
 namespace clc {
+
+constexpr long long kDigWaitPolls = 1ll << 26;
+constexpr int kDigStages = 8;          // digit-plane pairs (16 KB) in flight per CTA
+constexpr int kDigFlush = 2;           // blocks of 64 terms per TMEM accumulation
+constexpr int kRingScaleMax = 24;      // largest cexp
+constexpr int kNonFinite = 0x7fffffff; // column exponent of a column with a NaN or infinity
+constexpr size_t kSegBytes = 2ull << 30;   // FP64 recurrence values held at a time while building
+
+// half offset of element (row r, column c < 64) inside a tile of 64-half rows
+// in the 128-byte swizzle (8-row groups of 1024 bytes)
+__host__ __device__ __forceinline__ uint32_t dig_off(int r, int c) {
+  return (uint32_t)((r >> 3) * 512 + (r & 7) * 64 + (((c >> 3) ^ (r & 7)) << 3) + (c & 7));
+}
 
 // p * 2^e, exact unless the result is subnormal or zero (one final rounding);
 // |p| < 2^410 and e <= 64 here.
@@ -23,78 +64,193 @@ __device__ __forceinline__ double scale_pow2(double p, int e) {
   if (e < -1600) return 0.0;
   return (p * __longlong_as_double((long long)(e + 600 + 1023) << 52)) * 0x1p-600;
 }
+// the same for any e
+__device__ __forceinline__ double times_pow2(double p, int e) {
+  if (e >= -1022 && e <= 1023) return p * __longlong_as_double((long long)(e + 1023) << 52);
+  return ldexp(p, e);
+}
 
+__device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
+
+// x (|x| <= 2^62) as eight signed base-256 digits: byte i of x + 0x80..80 is
+// digit i plus 128
+__device__ __forceinline__ unsigned long long dig_bias(double x) {
+  return (unsigned long long)__double2ll_rn(x) + 0x8080808080808080ull;
+}
+// digit plane s (0 = most significant) of two values as FP16 integers
+__device__ __forceinline__ unsigned dig_pair(unsigned long long y0, unsigned long long y1, int s) {
+  const int sh = 8 * (kDigits - 1 - s);
+  const unsigned w = 0x64006400u | ((unsigned)(y0 >> sh) & 255u) | (((unsigned)(y1 >> sh) & 255u) << 16);   // 1024 + byte
+  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&w), __half2half2(__ushort_as_half(0x6480)));   // - 1152
+  return *reinterpret_cast<const unsigned*>(&d);
+}
+
+// ---------------------------------------------------------------------------
+// table build
+
+// recurrence coefficients a_lm = sqrt((4l^2 - 1) / (l^2 - m^2)),
+// b_lm = sqrt(((l-1)^2 - m^2) / (4 (l-1)^2 - 1)) of the orders ms ..
+__global__ void k_legendre_coef(int lt, int ms, double2* __restrict__ ab) {
+  const int m = ms + blockIdx.y;
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l > lt || l < m + 2) return;
+  const double l2 = (double)l * l, m2 = (double)m * m, k2 = (l - 1.0) * (l - 1.0);
+  ab[(size_t)blockIdx.y * (lt + 1) + l] = make_double2(sqrt((4.0 * l * l - 1.0) / (l2 - m2)), sqrt((k2 - m2) / (4.0 * k2 - 1.0)));
+}
+
+// lambda_lm of the orders ms .. in FP64, [m][l - m][r], and the ring scales
 __global__ void k_legendre_build(int nside, int lmax, int R, const long long* __restrict__ off,
                                  const double* __restrict__ lognorm, const double2* __restrict__ ab,
-                                 double* __restrict__ tab, int m0) {
-  const int m = m0 + blockIdx.y;
+                                 double* __restrict__ tab, int ms, int8_t* __restrict__ cexp, int ldc) {
+  const int m = ms + blockIdx.y;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= R) return;
   const Ring g = ring_geom(nside, r + 1);
   const double z = g.z;
   const int lt = lmax + 1;  // table band limit
-  double* col = tab + off[m - m0];
+  double* col = tab + off[blockIdx.y];
+  const double2* cab = ab + (size_t)blockIdx.y * (lt + 1);
   const double l2 = lognorm[m] + (double)m * log2(g.s);
   int e = (int)floor(l2);
   double p2 = exp2(l2 - (double)e);
   if (m & 1) p2 = -p2;
-  col[r] = scale_pow2(p2, e);
-  if (lt < m + 1) return;
-  double p1 = sqrt(2.0 * m + 3.0) * z * p2;
-  col[(size_t)R + r] = scale_pow2(p1, e);
-  const double big = 0x1p400, small = 0x1p-400;
-  for (int l = m + 2; l <= lt; ++l) {
-    const double2 c = ab[alm_idx(lt, l, m)];
-    double p0 = c.x * (z * p1 - c.y * p2);
-    if (fabs(p0) > big) {
-      p0 *= small;
-      p1 *= small;
-      e += 400;
+  double v = scale_pow2(p2, e);
+  col[r] = v;
+  int top = abs_hi(v);
+  if (lt >= m + 1) {
+    double p1 = sqrt(2.0 * m + 3.0) * z * p2;
+    v = scale_pow2(p1, e);
+    col[(size_t)R + r] = v;
+    top = max(top, abs_hi(v));
+    const double big = 0x1p400, small = 0x1p-400;
+    for (int l = m + 2; l <= lt; ++l) {
+      const double2 c = cab[l];
+      double p0 = c.x * (z * p1 - c.y * p2);
+      if (fabs(p0) > big) {
+        p0 *= small;
+        p1 *= small;
+        e += 400;
+      }
+      v = scale_pow2(p0, e);
+      col[(size_t)(l - m) * R + r] = v;
+      top = max(top, abs_hi(v));
+      p2 = p1;
+      p1 = p0;
     }
-    col[(size_t)(l - m) * R + r] = scale_pow2(p0, e);
-    p2 = p1;
-    p1 = p0;
+  }
+  // the largest |lambda_lm| of the ring is brought to about 1, by at most 2^kRingScaleMax
+  cexp[(size_t)blockIdx.y * ldc + r] = (int8_t)min(max(1023 - (top >> 20), 0), kRingScaleMax);
+}
+
+// One warp per row (l, m): the exponent of its largest scaled value and its
+// first ring block with a digit.
+__global__ void k_dig_rows(int lmax, int R, int ms, const long long* __restrict__ off, const double* __restrict__ tab,
+                           const int8_t* __restrict__ cexp, int ldc, const int* __restrict__ gidx,
+                           int* __restrict__ rexp, int* __restrict__ rb0) {
+  const int ml = blockIdx.y, m = ms + ml;
+  const int l = m + blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (l > lmax + 1) return;
+  const double* row = tab + off[ml] + (size_t)(l - m) * R;
+  const int8_t* c = cexp + (size_t)ml * ldc;
+  int top = 0;
+  for (int r = lane; r < R; r += 32) {
+    const int h = abs_hi(row[r]);
+    if (h >= 0x00100000) top = max(top, h + ((int)c[r] << 20));
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  const int er = top ? (top >> 20) - 1022 : 0;    // |value| < 2^er
+  const int least = (er - 63 + 1023) << 20;       // values below 2^(er - 63) round to zero digits
+  int first = R;
+  for (int r = lane; r < R; r += 32) {
+    const int h = abs_hi(row[r]);
+    if (h >= 0x00100000 && h + ((int)c[r] << 20) >= least) {
+      first = r;
+      break;
+    }
+  }
+  first = __reduce_min_sync(0xffffffffu, first);
+  if (lane == 0) {
+    const int k = (l - m) >> 1;
+    const int b = gidx[2 * ml + ((l - m) & 1)] + (k >> 6);
+    rexp[(size_t)b * 64 + (k & 63)] = er;
+    atomicMin(rb0 + b, first >> 6);
   }
 }
 
+// One CTA per atom: FP64 values to digit planes.
+__global__ void __launch_bounds__(256) k_dig_fill(int lmax, int R, int ms, const long long* __restrict__ off,
+                                                  const double* __restrict__ tab, const int8_t* __restrict__ cexp,
+                                                  int ldc, const int* __restrict__ gidx, const int* __restrict__ grp,
+                                                  const int* __restrict__ rexp, const int* __restrict__ rb0,
+                                                  __half* const* __restrict__ abase, int blk0) {
+  const int blk = blk0 + blockIdx.x, rb = blockIdx.y;
+  const int first = rb0[blk];
+  if (rb < first) return;
+  const int g = grp[blockIdx.x];                  // group within the segment's orders
+  const int ml = g >> 1, m = ms + ml;
+  const int k0 = (blk - gidx[g]) * 64;
+  __half* atom = abase[blk] + (size_t)(rb - first) * kDigits * kAtom;
+  for (int u = threadIdx.x; u < 512; u += 256) {
+    const int row = u >> 3, ch = u & 7;
+    const int l = m + (g & 1) + 2 * (k0 + row);
+    const bool ok = l <= lmax + 1;
+    const int er = rexp[(size_t)blk * 64 + row];
+    const double* src = tab + off[ml] + (size_t)(l - m) * R;
+    unsigned long long y[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int r = rb * 64 + ch * 8 + q;
+      y[q] = dig_bias(ok && r < R ? times_pow2(src[r], (int)cexp[(size_t)ml * ldc + r] + 62 - er) : 0.0);
+    }
+#pragma unroll
+    for (int s = 0; s < kDigits; ++s)
+      *reinterpret_cast<uint4*>(atom + s * kAtom + dig_off(row, ch * 8)) =
+          make_uint4(dig_pair(y[0], y[1], s), dig_pair(y[2], y[3], s), dig_pair(y[4], y[5], s), dig_pair(y[6], y[7], s));
+  }
+}
+
+__global__ void k_ring_factors(int nside, double* __restrict__ fac) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= 2 * nside) return;
+  const Ring g = ring_geom(nside, r + 1);
+  const double is2 = 1.0 / (g.s * g.s);
+  fac[r] = g.z * is2;
+  fac[2 * nside + r] = is2;
+}
+
+static int row_blocks(int lt, int m, int p) { return m + p <= lt ? ((lt - m - p) / 2 + 1 + 63) / 64 : 0; }
+
 size_t legendre_table_bytes(int nside, int lmax, int m0, int m1) {
-  const int lt = lmax + 1;
-  size_t e = 0;
-  for (int m = m0; m < m1; ++m) e += (size_t)(lt - m + 1) * 2 * nside;
-  return e * sizeof(double);
+  const size_t nkb = (2 * (size_t)nside + 63) / 64;
+  size_t b = 0;
+  for (int m = m0; m < m1; ++m) b += row_blocks(lmax + 1, m, 0) + row_blocks(lmax + 1, m, 1);
+  return b * nkb * kDigits * kAtom * sizeof(__half);
+}
+
+static bool dev_alloc(Buffer& b, size_t bytes) {
+  b.bytes = std::max(bytes, (size_t)16);
+  if (cudaMalloc(&b.p, b.bytes) != cudaSuccess) {
+    cudaGetLastError();
+    b.p = nullptr;
+    b.bytes = 0;
+    return false;
+  }
+  return true;
 }
 
 int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, LegendreTable* T) {
+  const int lt = lmax + 1, R = 2 * nside, nkb = (R + 63) / 64, nm = m1 - m0, ldc = nkb * 64;
   T->nside = nside;
   T->lmax = lmax;
-  T->R = 2 * nside;
+  T->R = R;
+  T->nkb = nkb;
   T->m0 = m0;
   T->m1 = m1;
-  const int lt = lmax + 1;
-  T->h_offsets.resize(m1 - m0);
-  long long acc = 0;
-  for (int m = m0; m < m1; ++m) {
-    T->h_offsets[m - m0] = acc;
-    acc += (long long)(lt - m + 1) * T->R;
-  }
-  T->elems = (size_t)acc;
-  size_t freeb = 0, totalb = 0;
-  cudaMemGetInfo(&freeb, &totalb);
-  const size_t bytes = T->elems * sizeof(double);
-  if (bytes + (size_t)(1ull << 30) > freeb)
-    return set_err(ctx, CLC_ENOMEM, "Legendre table of " + std::to_string(bytes >> 20) + " MiB does not fit");
-  // recurrence coefficients a_lm = sqrt((4l^2 - 1) / (l^2 - m^2)),
-  // b_lm = sqrt(((l-1)^2 - m^2) / (4 (l-1)^2 - 1)), packed with band limit lt
-  std::vector<double2> ab((size_t)alm_idx(lt, lt, lt) + 1);
-  for (int m = 0; m <= lt; ++m)
-    for (int l = m; l <= lt; ++l) {
-      double a = 0, b = 0;
-      if (l >= m + 2) {
-        a = std::sqrt((4.0 * l * l - 1.0) / ((double)l * l - (double)m * m));
-        b = std::sqrt(((l - 1.0) * (l - 1.0) - (double)m * m) / (4.0 * (l - 1.0) * (l - 1.0) - 1.0));
-      }
-      ab[alm_idx(lt, l, m)] = make_double2(a, b);
-    }
+  T->h_gidx.assign(2 * nm + 1, 0);
+  for (int g = 0; g < 2 * nm; ++g) T->h_gidx[g + 1] = T->h_gidx[g] + row_blocks(lt, m0 + (g >> 1), g & 1);
+  const int nblk = T->h_gidx[2 * nm];
+  std::vector<int> h_rb0(nblk, nkb);
+  std::vector<__half*> h_abase(nblk, nullptr);
   // log2 of sqrt((2m+1)!! / (4 pi (2m)!!))
   std::vector<double> lognorm(lmax + 1);
   double ln = 0.5 * std::log2(1.0 / (4.0 * kPi));
@@ -102,30 +258,124 @@ int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, Lege
     if (m > 0) ln += 0.5 * std::log2((2.0 * m + 1.0) / (2.0 * m));
     lognorm[m] = ln;
   }
-  Buffer d_ab, d_ln;
-  auto alloc = [&](Buffer& b, size_t n) -> bool {
-    b.bytes = n;
-    if (cudaMalloc(&b.p, n) != cudaSuccess) {
-      cudaGetLastError();
-      b.p = nullptr;
-      return false;
+  // segments of orders whose FP64 values fit the build buffer
+  std::vector<int> seg{m0};
+  size_t tab_bytes = 0, acc = 0;
+  int seg_orders = 0;
+  for (int m = m0; m < m1; ++m) {
+    const size_t b = (size_t)(lt - m + 1) * R * sizeof(double);
+    if (acc > 0 && acc + b > kSegBytes) {
+      seg.push_back(m);
+      acc = 0;
     }
-    return true;
+    acc += b;
+    tab_bytes = std::max(tab_bytes, acc);
+    seg_orders = std::max(seg_orders, m - seg.back() + 1);
+  }
+  seg.push_back(m1);
+  Buffer d_tab, d_ab, d_ln, d_off, d_grp;
+  const char* what = "Legendre table allocation failed";
+  if (!dev_alloc(T->gidx, sizeof(int) * (2 * nm + 1)) || !dev_alloc(T->rb0, sizeof(int) * nblk) ||
+      !dev_alloc(T->abase, sizeof(__half*) * nblk) || !dev_alloc(T->rexp, sizeof(int) * 64 * (size_t)nblk) ||
+      !dev_alloc(T->cexp, (size_t)nm * ldc) || !dev_alloc(T->fac, sizeof(double) * 2 * R) ||
+      !dev_alloc(T->zero, (size_t)kDigits * kAtom * sizeof(__half)) || !dev_alloc(d_tab, tab_bytes) ||
+      !dev_alloc(d_ab, sizeof(double2) * (size_t)seg_orders * (lt + 1)) ||
+      !dev_alloc(d_ln, sizeof(double) * lognorm.size()) || !dev_alloc(d_off, sizeof(long long) * seg_orders) ||
+      !dev_alloc(d_grp, sizeof(int) * nblk))
+    return set_err(ctx, CLC_ENOMEM, what);
+  cudaStream_t st = ctx->stream;
+  cudaMemcpyAsync(T->gidx.p, T->h_gidx.data(), sizeof(int) * (2 * nm + 1), cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(T->rb0.p, h_rb0.data(), sizeof(int) * nblk, cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(d_ln.p, lognorm.data(), sizeof(double) * lognorm.size(), cudaMemcpyHostToDevice, st);
+  cudaMemsetAsync(T->rexp.p, 0, T->rexp.bytes, st);
+  cudaMemsetAsync(T->cexp.p, 0, T->cexp.bytes, st);
+  cudaMemsetAsync(T->zero.p, 0, T->zero.bytes, st);
+  CLC_LAUNCH(ctx, "k_ring_factors", k_ring_factors, (R + 127) / 128, 128, 0, nside, (double*)T->fac.p);
+  int rc;
+  for (size_t s = 0; s + 1 < seg.size(); ++s) {
+    const int ms = seg[s], me = seg[s + 1], n = me - ms, g0 = 2 * (ms - m0);
+    const int b0 = T->h_gidx[g0], b1 = T->h_gidx[2 * (me - m0)];
+    std::vector<long long> off(n);
+    long long a = 0;
+    for (int m = ms; m < me; ++m) {
+      off[m - ms] = a;
+      a += (long long)(lt - m + 1) * R;
+    }
+    std::vector<int> grp(std::max(b1 - b0, 1));
+    for (int g = 0; g < 2 * n; ++g)
+      for (int b = T->h_gidx[g0 + g]; b < T->h_gidx[g0 + g + 1]; ++b) grp[b - b0] = g;
+    cudaMemcpyAsync(d_off.p, off.data(), sizeof(long long) * n, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(d_grp.p, grp.data(), sizeof(int) * (b1 - b0), cudaMemcpyHostToDevice, st);
+    int8_t* cx = (int8_t*)T->cexp.p + (size_t)(ms - m0) * ldc;
+    const int* gx = (const int*)T->gidx.p + g0;
+    CLC_LAUNCH(ctx, "k_legendre_coef", k_legendre_coef, dim3((lt + 128) / 128, n), 128, 0, lt, ms, (double2*)d_ab.p);
+    CLC_LAUNCH(ctx, "k_legendre_build", k_legendre_build, dim3((R + 127) / 128, n), 128, 0, nside, lmax, R,
+               (const long long*)d_off.p, (const double*)d_ln.p, (const double2*)d_ab.p, (double*)d_tab.p, ms, cx, ldc);
+    CLC_LAUNCH(ctx, "k_dig_rows", k_dig_rows, dim3((lt - ms + 8) / 8, n), 256, 0, lmax, R, ms, (const long long*)d_off.p,
+               (const double*)d_tab.p, (const int8_t*)cx, ldc, gx, (int*)T->rexp.p, (int*)T->rb0.p);
+    if ((rc = launch_check(ctx, "Legendre table rows"))) return rc;
+    cudaMemcpyAsync(h_rb0.data() + b0, (const int*)T->rb0.p + b0, sizeof(int) * (b1 - b0), cudaMemcpyDeviceToHost, st);
+    if ((rc = cuda_check(ctx, cudaStreamSynchronize(st), "Legendre table rows"))) return rc;
+    // a row block keeps at least the ring blocks of the one before it (lower l)
+    size_t natom = 0;
+    for (int g = 0; g < 2 * n; ++g)
+      for (int b = T->h_gidx[g0 + g]; b < T->h_gidx[g0 + g + 1]; ++b) {
+        if (b > T->h_gidx[g0 + g]) h_rb0[b] = std::min(h_rb0[b], h_rb0[b - 1]);
+        natom += nkb - h_rb0[b];
+      }
+    auto piece = std::make_unique<Buffer>();
+    const size_t bytes = natom * kDigits * kAtom * sizeof(__half);
+    if (!dev_alloc(*piece, bytes))
+      return set_err(ctx, CLC_ENOMEM, "Legendre table of " + std::to_string(bytes >> 20) + " MiB does not fit");
+    __half* at = (__half*)piece->p;
+    T->atoms.push_back(std::move(piece));
+    for (int b = b0; b < b1; ++b) {
+      h_abase[b] = at;
+      at += (size_t)(nkb - h_rb0[b]) * kDigits * kAtom;
+    }
+    cudaMemcpyAsync((int*)T->rb0.p + b0, h_rb0.data() + b0, sizeof(int) * (b1 - b0), cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync((__half**)T->abase.p + b0, h_abase.data() + b0, sizeof(__half*) * (b1 - b0), cudaMemcpyHostToDevice,
+                    st);
+    if (b1 > b0)
+      CLC_LAUNCH(ctx, "k_dig_fill", k_dig_fill, dim3(b1 - b0, nkb), 256, 0, lmax, R, ms, (const long long*)d_off.p,
+                 (const double*)d_tab.p, (const int8_t*)cx, ldc, gx, (const int*)d_grp.p, (const int*)T->rexp.p,
+                 (const int*)T->rb0.p, (__half* const*)T->abase.p, b0);
+    // the host arrays of the segment and the build buffers are reused: wait
+    if ((rc = launch_check(ctx, "k_dig_fill"))) return rc;
+    if ((rc = cuda_check(ctx, cudaStreamSynchronize(st), "Legendre table build"))) return rc;
+  }
+  // work lists.  Analysis: (group, 128-row tile, first ring block); synthesis:
+  // (order, 128-ring tile, first row blocks of the two parities).
+  std::vector<std::pair<int, int4>> an, sy;
+  for (int g = 0; g < 2 * nm; ++g) {
+    const int nb = T->h_gidx[g + 1] - T->h_gidx[g];
+    for (int t = 0; 2 * t < nb; ++t) {
+      const int first = h_rb0[T->h_gidx[g] + std::min(2 * t + 1, nb - 1)];
+      an.push_back({nkb - first, make_int4(g, t, first, 0)});
+    }
+  }
+  for (int m = 0; m < nm; ++m)
+    for (int t = 0; 2 * t < nkb; ++t) {
+      int first[2], len = 0;
+      for (int p = 0; p < 2; ++p) {
+        const int gb = T->h_gidx[2 * m + p], nb = T->h_gidx[2 * m + p + 1] - gb;
+        int b = 0;
+        while (b < nb && h_rb0[gb + b] > std::min(2 * t + 1, nkb - 1)) ++b;
+        first[p] = b;
+        len += nb - b;
+      }
+      sy.push_back({len, make_int4(m, t, first[0], first[1])});
+    }
+  auto upload = [&](std::vector<std::pair<int, int4>>& v, Buffer& buf, int* count) -> int {
+    std::stable_sort(v.begin(), v.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
+    std::vector<int4> it;
+    for (auto& x : v) it.push_back(x.second);
+    *count = (int)it.size();
+    if (!dev_alloc(buf, sizeof(int4) * it.size())) return set_err(ctx, CLC_ENOMEM, what);
+    return cuda_check(ctx, cudaMemcpy(buf.p, it.data(), sizeof(int4) * it.size(), cudaMemcpyHostToDevice), "work list");
   };
-  if (!alloc(T->data, bytes) || !alloc(T->offsets, sizeof(long long) * (m1 - m0)) ||
-      !alloc(d_ab, sizeof(double2) * ab.size()) || !alloc(d_ln, sizeof(double) * lognorm.size()))
-    return set_err(ctx, CLC_ENOMEM, "Legendre table allocation failed");
-  cudaMemcpyAsync(T->offsets.p, T->h_offsets.data(), sizeof(long long) * (m1 - m0), cudaMemcpyHostToDevice,
-                  ctx->stream);
-  cudaMemcpyAsync(d_ab.p, ab.data(), sizeof(double2) * ab.size(), cudaMemcpyHostToDevice, ctx->stream);
-  cudaMemcpyAsync(d_ln.p, lognorm.data(), sizeof(double) * lognorm.size(), cudaMemcpyHostToDevice, ctx->stream);
-  dim3 grid((T->R + 127) / 128, m1 - m0);
-  CLC_LAUNCH(ctx, "k_legendre_build", k_legendre_build, grid, 128, 0, nside, lmax, T->R, (const long long*)T->offsets.p,
-             (const double*)d_ln.p, (const double2*)d_ab.p, (double*)T->data.p, m0);
-  const int rc = launch_check(ctx, "k_legendre_build");
-  // the coefficient buffers are freed when this function returns: wait for the build
-  cudaStreamSynchronize(ctx->stream);
-  return rc;
+  if ((rc = upload(an, T->an, &T->n_an))) return rc;
+  return upload(sy, T->sy, &T->n_sy);
 }
 
 std::shared_ptr<LegendreTable> get_legendre_table(clc_ctx* ctx, int nside, int lmax, int* rc) {
@@ -142,125 +392,548 @@ std::shared_ptr<LegendreTable> get_legendre_table(clc_ctx* ctx, int nside, int l
   return T;
 }
 
-// Block (l-block, m): 8 warps, each warp one l at a time; lanes over rings.
-__global__ void k_legendre_analysis(int nside, int lmax, int R, const long long* __restrict__ off,
-                                    const double* __restrict__ tab, const double2* __restrict__ F, int ldf,
-                                    double2* __restrict__ alm, int ltop, int lpack, int m0) {
-  extern __shared__ double2 V[];  // V[0..R) even (N + S), V[R..2R) odd (N - S)
-  const int m = m0 + blockIdx.y;
-  const int l0 = m + blockIdx.x * 64;
-  if (l0 > ltop) return;
-  const double2* Fm = F + (size_t)m * ldf;
-  for (int r = threadIdx.x; r < R; r += blockDim.x) {
-    const int i = r + 1;
-    const double2 fn = Fm[i - 1];
-    double2 fs = make_double2(0.0, 0.0);
-    if (i != 2 * nside) fs = Fm[4 * nside - i - 1];
-    V[r] = make_double2(fn.x + fs.x, fn.y + fs.y);
-    V[R + r] = make_double2(fn.x - fs.x, fn.y - fs.y);
+// ---------------------------------------------------------------------------
+// data operands: columns of doubles to digit planes.  Block of 64 terms:
+// kDigits x kCols rows (digit plane j, column c at row j kCols + c) of 64
+// halves; rows of columns not in use are left as they are (they only reach
+// accumulator columns that nothing reads).
+
+constexpr int kCols = 16;                          // real columns of a contraction
+constexpr int kOpBlock = kDigits * kCols * 64;     // halves of a block
+
+// block-wide maxima of four non-negative integers (results in all threads)
+__device__ __forceinline__ void block_max4(int v[4], int* sh) {
+  const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  __syncthreads();   // earlier readers of sh are done
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int x = __reduce_max_sync(0xffffffffu, v[i]);
+    if ((threadIdx.x & 31) == 0) sh[4 * warp + i] = x;
   }
   __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double* col = tab + off[m - m0];
-  for (int l = l0 + warp; l <= ltop && l < l0 + 64; l += 8) {
-    const double* row = col + (size_t)(l - m) * R;
-    const double2* v = V + (((l + m) & 1) ? R : 0);
-    double ax = 0.0, ay = 0.0;
-    for (int r = lane; r < R; r += 32) {
-      const double lam = row[r];
-      const double2 x = v[r];
-      ax = fma(lam, x.x, ax);
-      ay = fma(lam, x.y, ay);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      ax += __shfl_xor_sync(0xffffffffu, ax, o);
-      ay += __shfl_xor_sync(0xffffffffu, ay, o);
-    }
-    if (lane == 0) alm[alm_idx(lpack, l, m)] = make_double2(ax, ay);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    v[i] = sh[i];
+    for (int w = 1; w < nw; ++w) v[i] = max(v[i], sh[4 * w + i]);
   }
 }
 
-int legendre_analysis(clc_ctx* ctx, const LegendreTable& T, const double2* F, int ldf, double2* alm, int ltop) {
-  const int L = T.lmax;
-  if (ltop < 0) ltop = L;
-  dim3 grid((ltop + 1 + 63) / 64, T.m1 - T.m0);
-  const int smem = 2 * T.R * (int)sizeof(double2);
-  cudaFuncSetAttribute(k_legendre_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  CLC_LAUNCH(ctx, "k_legendre_analysis", k_legendre_analysis, grid, 256, smem, T.nside, L, T.R, (const long long*)T.offsets.p,
-                                                        (const double*)T.data.p, F, ldf, alm, ltop, ltop, T.m0);
-  return launch_check(ctx, "k_legendre_analysis");
+// exponent e of a column with largest absolute high word `hi` (|value| < 2^e)
+__device__ __forceinline__ int col_exp(int hi) {
+  if (hi >= 0x7ff00000) return kNonFinite;
+  return hi ? max(hi >> 20, 1) - 1022 : 0;
+}
+
+struct AnaCols {
+  const double2* F[8];
+  int kind[8];
+  int nv;
+};
+
+// One CTA per order; column 2 v + re/im of both parities.
+__global__ void __launch_bounds__(256) k_dig_pack_analysis(AnaCols a, int nside, int R, int nkb, int ldf, int m0,
+                                                           const int8_t* __restrict__ cexp,
+                                                           const double* __restrict__ fac, __half* __restrict__ op,
+                                                           int* __restrict__ colexp) {
+  __shared__ int sh[4 * 8];
+  const int ml = blockIdx.x, m = m0 + ml;
+  const int8_t* cx = cexp + (size_t)ml * nkb * 64;
+  for (int v = blockIdx.y; v < a.nv; v += gridDim.y) {
+    const double2* F = a.F[v] + (size_t)m * ldf;
+    const int kind = a.kind[v];
+    // (even re, even im, odd re, odd im) of ring r, scaled
+    auto vals = [&](int r, double x[4]) {
+      if (r >= R) {
+        x[0] = x[1] = x[2] = x[3] = 0.0;
+        return;
+      }
+      const double2 n = F[r];
+      double2 s = make_double2(0.0, 0.0);
+      if (r + 1 != 2 * nside) s = F[4 * nside - r - 2];
+      double w = __longlong_as_double((long long)(1023 - (int)cx[r]) << 52);
+      if (kind) w *= fac[(size_t)(kind - 1) * R + r];
+      const double sg = kind == 1 ? -1.0 : 1.0;
+      x[0] = fma(sg, s.x, n.x) * w;
+      x[1] = fma(sg, s.y, n.y) * w;
+      x[2] = fma(-sg, s.x, n.x) * w;
+      x[3] = fma(-sg, s.y, n.y) * w;
+    };
+    int top[4] = {0, 0, 0, 0};
+    for (int r = threadIdx.x; r < R; r += 256) {
+      double x[4];
+      vals(r, x);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) top[i] = max(top[i], abs_hi(x[i]));
+    }
+    block_max4(top, sh);
+    int ec[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ec[i] = col_exp(top[i]);
+    if (threadIdx.x < 4)
+      colexp[(size_t)(2 * ml + (threadIdx.x >> 1)) * kCols + 2 * v + (threadIdx.x & 1)] = ec[threadIdx.x];
+    for (int r = 2 * threadIdx.x; r < nkb * 64; r += 512) {
+      double x0[4], x1[4];
+      vals(r, x0);
+      vals(r + 1, x1);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const bool ok = ec[i] != kNonFinite;
+        const unsigned long long y0 = dig_bias(ok ? times_pow2(x0[i], 62 - ec[i]) : 0.0);
+        const unsigned long long y1 = dig_bias(ok ? times_pow2(x1[i], 62 - ec[i]) : 0.0);
+        __half* dst = op + ((size_t)(2 * ml + (i >> 1)) * nkb + (r >> 6)) * kOpBlock;
+#pragma unroll
+        for (int s = 0; s < kDigits; ++s)
+          *reinterpret_cast<unsigned*>(dst + dig_off(s * kCols + 2 * v + (i & 1), r & 63)) = dig_pair(y0, y1, s);
+      }
+    }
+  }
 }
 
 struct SynthRhs {
   const double2* rhs;
   int nq;
-  int lq[3];
+  int lq[4];
 };
 
-// Block (ring chunk, m); thread per northern ring; the alm columns of this m
-// are staged in shared memory.
-__global__ void k_legendre_synthesis(int nside, int lmax, int R, const long long* __restrict__ off,
-                                     const double* __restrict__ tab, SynthRhs s, double2* __restrict__ G, int ld,
-                                     int m0) {
-  extern __shared__ double2 A[];  // A[q * (lt - m + 1) + (l - m)]
-  const int m = m0 + blockIdx.y;
-  const int lt = lmax + 1;
-  const int nl = lt - m + 1;
-  for (int t = threadIdx.x; t < s.nq * nl; t += blockDim.x) {
-    const int q = t / nl, l = m + t % nl;
-    const size_t qoff = (size_t)q * (alm_idx(lt, lt, lt) + 1);
-    A[t] = (l <= s.lq[q]) ? s.rhs[qoff + alm_idx(lt, l, m)] : make_double2(0.0, 0.0);
-  }
-  __syncthreads();
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
-  int lmax_used = 0;
-  for (int q = 0; q < s.nq; ++q) lmax_used = max(lmax_used, s.lq[q]);
-  const double* col = tab + off[m - m0];
-  double acc[3][2][2];
+// One CTA per order; column 2 q + re/im of both parities (rows l = m + p + 2 k).
+__global__ void __launch_bounds__(256) k_dig_pack_synthesis(SynthRhs s, int lmax, int m0, const int* __restrict__ gidx,
+                                                            const int* __restrict__ rexp, __half* __restrict__ op,
+                                                            int* __restrict__ colexp) {
+  __shared__ int sh[4 * 8];
+  const int ml = blockIdx.x, m = m0 + ml, lt = lmax + 1;
+  const int gb[3] = {gidx[2 * ml], gidx[2 * ml + 1], gidx[2 * ml + 2]};
+  const int np = max(gb[1] - gb[0], gb[2] - gb[1]) * 32;   // pairs of rows
+  for (int q = blockIdx.y; q < s.nq; q += gridDim.y) {
+    const double2* rhs = s.rhs + (size_t)q * (alm_idx(lt, lt, lt) + 1);
+    // (re, im) of row k of parity p, scaled
+    auto val = [&](int p, int k) -> double2 {
+      const int l = m + p + 2 * k;
+      if (l > s.lq[q] || l > lt) return make_double2(0.0, 0.0);
+      const double2 v = rhs[alm_idx(lt, l, m)];
+      const int e = rexp[(size_t)gb[p] * 64 + k];
+      return make_double2(times_pow2(v.x, e), times_pow2(v.y, e));
+    };
+    int top[4] = {0, 0, 0, 0};
+    for (int k = threadIdx.x; k < 2 * np; k += 256) {
 #pragma unroll
-  for (int q = 0; q < 3; ++q)
+      for (int p = 0; p < 2; ++p) {
+        const double2 v = val(p, k);
+        top[2 * p] = max(top[2 * p], abs_hi(v.x));
+        top[2 * p + 1] = max(top[2 * p + 1], abs_hi(v.y));
+      }
+    }
+    block_max4(top, sh);
+    int ec[4];
 #pragma unroll
-    for (int p = 0; p < 2; ++p) acc[q][p][0] = acc[q][p][1] = 0.0;
-  for (int l = m; l <= lmax_used; ++l) {
-    const double lam = col[(size_t)(l - m) * R + r];
-    const int p = (l + m) & 1;
+    for (int i = 0; i < 4; ++i) ec[i] = col_exp(top[i]);
+    if (threadIdx.x < 4)
+      colexp[(size_t)(2 * ml + (threadIdx.x >> 1)) * kCols + 2 * q + (threadIdx.x & 1)] = ec[threadIdx.x];
+    for (int t = threadIdx.x; t < np; t += 256) {
+      const int k = 2 * t;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      if (q < s.nq) {
-        const double2 a = A[q * nl + (l - m)];
-        if (p) {
-          acc[q][1][0] = fma(lam, a.x, acc[q][1][0]);
-          acc[q][1][1] = fma(lam, a.y, acc[q][1][1]);
-        } else {
-          acc[q][0][0] = fma(lam, a.x, acc[q][0][0]);
-          acc[q][0][1] = fma(lam, a.y, acc[q][0][1]);
+      for (int p = 0; p < 2; ++p) {
+        if (k >= (gb[p + 1] - gb[p]) * 64) continue;
+        const double2 a = val(p, k), b = val(p, k + 1);
+        __half* dst = op + (size_t)(gb[p] + (k >> 6)) * kOpBlock;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const int e = ec[2 * p + i];
+          const bool ok = e != kNonFinite;
+          const unsigned long long y0 = dig_bias(ok ? times_pow2(i ? a.y : a.x, 62 - e) : 0.0);
+          const unsigned long long y1 = dig_bias(ok ? times_pow2(i ? b.y : b.x, 62 - e) : 0.0);
+#pragma unroll
+          for (int j = 0; j < kDigits; ++j)
+            *reinterpret_cast<unsigned*>(dst + dig_off(j * kCols + 2 * q + i, k & 63)) = dig_pair(y0, y1, j);
         }
       }
     }
   }
-  const int i = r + 1;
-  const size_t qstride = (size_t)ld * (lmax + 2);
-  for (int q = 0; q < s.nq; ++q) {
-    double2* Gq = G + q * qstride + (size_t)m * ld;
-    Gq[i - 1] = make_double2(acc[q][0][0] + acc[q][1][0], acc[q][0][1] + acc[q][1][1]);
-    if (i != 2 * nside) Gq[4 * nside - i - 1] = make_double2(acc[q][0][0] - acc[q][1][0], acc[q][0][1] - acc[q][1][1]);
+}
+
+// ---------------------------------------------------------------------------
+// contractions: persistent, warp-specialised, bulk-copy pipelined
+//
+// Analysis item (group, 128-row tile): the terms are rings, blocks of 64 from
+// the first one with a digit to the equator; A = two atoms (row blocks 2 t and
+// 2 t + 1 of the ring block), K-major.  Synthesis item (order, 128-ring tile):
+// the terms are rows of parity 0, then of parity 1; A = two atoms (ring blocks
+// 2 t and 2 t + 1 of the row block), MN-major.  A block's eight digit planes of
+// A (16 KB each) pass through a ring of eight stages; its B operand (all digit
+// planes of the data) comes with the first.  Plane i is multiplied by the data
+// planes 0 .. 7 - i at once (N = (8 - i) kCols columns) into the accumulator
+// columns from i kCols on, so that column block g collects the digit pairs i + j =
+// g.  After kDigFlush blocks the four epilogue warps (one row per thread) move
+// the sums into 64-bit integers: hi = D0 2^24 + D1 2^16 + D2 2^8 + D3 and lo =
+// D4 2^24 + D5 2^16 + D6 2^8 + D7 (the value is hi 2^32 + lo); two accumulators alternate.
+// Two data blocks suffice: with eight stages the copy that refills a data
+// block is issued after the empty barrier of that block's last plane.
+// Warps 0-3: epilogue (TMEM lanes 32w .. 32w + 31), warp 4: bulk copies, warp 5: MMAs.
+
+struct DigArgs {
+  const __half* const* abase;
+  const int* rb0;
+  const int* gidx;
+  const __half* zero;
+  const __half* op;
+  const int* rexp;
+  const int* colexp;
+  const int8_t* cexp;
+  int nside, lmax, R, nkb, m0;
+  int nv;             // complex columns
+  double2* out[8];    // analysis
+  int ltop;           // analysis: highest l, band limit of the packing
+  double2* G;         // synthesis
+  size_t qstride;
+  int ld;
+};
+
+template <int N>
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t* r);
+template <>
+__device__ __forceinline__ void tmem_ld<2>(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
+}
+template <>
+__device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+template <>
+__device__ __forceinline__ void tmem_ld<16>(uint32_t taddr, uint32_t* r) {
+  tmem_ld<8>(taddr, r);
+  tmem_ld<8>(taddr + 8, r + 8);
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// blocks of 64 terms of an item: n[0] of the first, n[1] of the second phase
+template <bool kSyn>
+__device__ __forceinline__ void dig_counts(const DigArgs& a, int4 w, int n[2]) {
+  if (kSyn) {
+    n[0] = a.gidx[2 * w.x + 1] - a.gidx[2 * w.x] - w.z;
+    n[1] = a.gidx[2 * w.x + 2] - a.gidx[2 * w.x + 1] - w.w;
+  } else {
+    n[0] = a.nkb - w.z;
+    n[1] = 0;
   }
+}
+
+template <bool kSyn, int NC>
+__global__ void __launch_bounds__(192) k_dig_gemm(DigArgs a, const int4* __restrict__ items, int nitems, int* d_err) {
+  constexpr uint32_t kOpBytes = kOpBlock * 2;   // a data block
+  constexpr uint32_t kAcc = 128;                // TMEM columns of an accumulator (kDigits kCols)
+  extern __shared__ __align__(16) uint8_t smem_g[];
+  __shared__ uint64_t full[kDigStages], empty[kDigStages], chunkb[2], freeb[2], drainb;
+  __shared__ uint32_t tmem_base;
+  __shared__ volatile int abort_flag;
+  const uint32_t raw = umma::smem_u32(smem_g);
+  uint8_t* base = smem_g + (((raw + 1023u) & ~1023u) - raw);
+  uint8_t* opb = base + kDigStages * 16384;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kDigStages; ++s) {
+      umma::mbar_init(&full[s], 1);
+      umma::mbar_init(&empty[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      umma::mbar_init(&chunkb[s], 1);
+      umma::mbar_init(&freeb[s], 128);
+    }
+    umma::mbar_init(&drainb, 1);
+    abort_flag = 0;
+    umma::fence_mbar_init();
+  }
+  if (warp == 0) umma::tmem_alloc(&tmem_base, 2 * kAcc);
+  umma::fence_before_sync();
+  __syncthreads();
+  umma::fence_after_sync();
+  const uint32_t tmem = tmem_base;
+  auto fail = [&]() {
+    atomicCAS(d_err, 0, kDevTimeout);
+    abort_flag = 1;
+  };
+
+  if (warp == 4) {
+    // ---- producer
+    if (lane == 0) {
+      uint32_t it = 0, blk = 0;
+      int last_it[kDigStages];
+      for (int s = 0; s < kDigStages; ++s) last_it[s] = -1;
+      for (int item = blockIdx.x; item < nitems && !abort_flag; item += gridDim.x) {
+        const int4 w = items[item];
+        int n[2];
+        dig_counts<kSyn>(a, w, n);
+        for (int ph = 0; ph < 2 && !abort_flag; ++ph) {
+          // analysis: the two row blocks of the tile
+          int i0 = 0, s0 = 0, s1 = a.nkb;
+          const __half *b0 = nullptr, *b1 = nullptr;
+          if (!kSyn && n[0] > 0) {
+            i0 = a.gidx[w.x] + 2 * w.y;
+            s0 = a.rb0[i0];
+            b0 = a.abase[i0];
+            if (i0 + 1 < a.gidx[w.x + 1]) {
+              s1 = a.rb0[i0 + 1];
+              b1 = a.abase[i0 + 1];
+            }
+          }
+          for (int k = 0; k < n[ph] && !abort_flag; ++k, ++blk) {
+            const __half *p0 = a.zero, *p1 = a.zero, *op;
+            if (kSyn) {
+              const int idx = a.gidx[2 * w.x + ph] + (ph ? w.w : w.z) + k;
+              const int first = a.rb0[idx], rb = 2 * w.y;
+              const __half* b = a.abase[idx];
+              if (rb >= first) p0 = b + (size_t)(rb - first) * kDigits * kAtom;
+              if (rb + 1 < a.nkb && rb + 1 >= first) p1 = b + (size_t)(rb + 1 - first) * kDigits * kAtom;
+              op = a.op + (size_t)idx * kOpBlock;
+            } else {
+              const int rb = w.z + k;
+              if (rb >= s0) p0 = b0 + (size_t)(rb - s0) * kDigits * kAtom;
+              if (rb >= s1) p1 = b1 + (size_t)(rb - s1) * kDigits * kAtom;
+              op = a.op + ((size_t)w.x * a.nkb + rb) * kOpBlock;
+            }
+            for (int d = 0; d < kDigits; ++d, ++it) {
+              const int s = (int)(it % kDigStages);
+              const uint32_t u = it / kDigStages;
+              if (u > 0 && !umma::mbar_wait(&empty[s], (u - 1) & 1u, kDigWaitPolls)) {
+                fail();
+                break;
+              }
+              uint8_t* st = base + (size_t)s * 16384;
+              umma::mbar_arrive_expect_tx(&full[s], 16384u + (d == 0 ? kOpBytes : 0u));
+              umma::bulk_g2s(st, p0 + d * kAtom, 8192u, &full[s]);
+              umma::bulk_g2s(st + 8192, p1 + d * kAtom, 8192u, &full[s]);
+              if (d == 0) umma::bulk_g2s(opb + (blk & 1u) * kOpBytes, op, kOpBytes, &full[s]);
+              last_it[s] = (int)it;
+            }
+          }
+        }
+      }
+      if (abort_flag)
+        for (int s = 0; s < kDigStages; ++s)   // bounded drain of the copies in flight
+          if (last_it[s] >= 0) umma::mbar_wait(&full[s], (uint32_t)(last_it[s] / kDigStages) & 1u, kDigWaitPolls);
+    }
+  } else if (warp == 5) {
+    // ---- MMA issuer
+    if (lane == 0) {
+      uint32_t it = 0, blk = 0, nchunk = 0;
+      for (int item = blockIdx.x; item < nitems && !abort_flag; item += gridDim.x) {
+        int n[2];
+        dig_counts<kSyn>(a, items[item], n);
+        for (int ph = 0; ph < 2; ++ph)
+          for (int k = 0; k < n[ph] && !abort_flag; ++k, ++blk) {
+            const bool first = k % kDigFlush == 0;
+            const uint32_t buf = nchunk & 1u;
+            if (first && nchunk > 1 && !umma::mbar_wait(&freeb[buf], ((nchunk >> 1) - 1) & 1u, kDigWaitPolls)) {
+              fail();   // the epilogue has not released the accumulator
+              break;
+            }
+            const uint32_t sb = umma::smem_u32(opb + (blk & 1u) * kOpBytes);
+            for (int d = 0; d < kDigits; ++d, ++it) {
+              const int s = (int)(it % kDigStages);
+              if (!umma::mbar_wait(&full[s], (it / kDigStages) & 1u, kDigWaitPolls)) {
+                fail();
+                break;
+              }
+              umma::fence_after_sync();
+              const uint32_t sa = umma::smem_u32(base + (size_t)s * 16384);
+              const int N = (kDigits - d) * kCols;
+              const uint32_t idesc = kSyn ? umma::idesc_f16_f32_amn(128, N) : umma::idesc_f16_f32(128, N);
+              const uint64_t dA = kSyn ? umma::desc_sw128_mn(sa, 8192, 1024) : umma::desc_sw128(sa);
+              const uint64_t dB = umma::desc_sw128(sb);
+              const uint32_t td = tmem + buf * kAcc + (uint32_t)(d * kCols);
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                umma::mma_f16(td, dA + (uint64_t)((kSyn ? kk * 2048 : kk * 32) >> 4), dB + (uint64_t)((kk * 32) >> 4),
+                              idesc, (first && d == 0 && kk == 0) ? 0u : 1u);
+              umma::commit(&empty[s]);
+            }
+            if (abort_flag) break;
+            if (k % kDigFlush == kDigFlush - 1 || k + 1 == n[ph]) {
+              umma::commit(&chunkb[buf]);
+              ++nchunk;
+            }
+          }
+      }
+      if (abort_flag) {   // bounded wait for the MMAs in flight
+        umma::commit(&drainb);
+        umma::mbar_wait(&drainb, 0, kDigWaitPolls);
+      }
+    }
+  } else {
+    // ---- epilogue warps
+    uint32_t nchunk = 0;
+    const uint32_t trow = tmem + ((uint32_t)(warp * 32) << 16);
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    for (int item = blockIdx.x; item < nitems && !__any_sync(0xffffffffu, abort_flag); item += gridDim.x) {
+      const int4 w = items[item];
+      int n[2];
+      dig_counts<kSyn>(a, w, n);
+      double val[kSyn ? 2 : 1][NC];
+      bool ok = true;
+#pragma unroll
+      for (int ph = 0; ph < (kSyn ? 2 : 1); ++ph) {
+        long long hi[NC], lo[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) hi[c] = lo[c] = 0;
+        for (int k = 0; ok && k < n[ph]; k += kDigFlush, ++nchunk) {
+          const uint32_t buf = nchunk & 1u;
+          // warp-uniform decision: the TMEM accesses below are whole-warp operations
+          const bool got = umma::mbar_wait(&chunkb[buf], (nchunk >> 1) & 1u, kDigWaitPolls);
+          if (!__all_sync(0xffffffffu, got)) {
+            if (lane == 0) fail();
+            ok = false;
+            break;
+          }
+          umma::fence_after_sync();
+          uint32_t v[4][NC];
+          auto sum4 = [&](int c) {
+            return (long long)__float2int_rn(__uint_as_float(v[0][c])) * 16777216 +
+                   (long long)__float2int_rn(__uint_as_float(v[1][c])) * 65536 +
+                   (long long)__float2int_rn(__uint_as_float(v[2][c])) * 256 + __float2int_rn(__uint_as_float(v[3][c]));
+          };
+#pragma unroll
+          for (int g = 0; g < 4; ++g) tmem_ld<NC>(trow + buf * kAcc + g * kCols, v[g]);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < NC; ++c) hi[c] += sum4(c);
+#pragma unroll
+          for (int g = 0; g < 4; ++g) tmem_ld<NC>(trow + buf * kAcc + (4 + g) * kCols, v[g]);
+          tmem_wait_ld();
+          umma::fence_before_sync();
+          umma::mbar_arrive(&freeb[buf]);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) lo[c] += sum4(c);
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c) val[ph][c] = fma((double)hi[c], 4294967296.0, (double)lo[c]);
+      }
+      if (!ok) break;
+      __syncwarp();
+      if (!kSyn) {
+        const int m = a.m0 + (w.x >> 1), k = w.y * 128 + warp * 32 + lane;
+        const int l = m + (w.x & 1) + 2 * k;
+        if (l <= a.ltop) {
+          const int er = a.rexp[(size_t)a.gidx[w.x] * 64 + k] - 68;
+          const int* ce = a.colexp + (size_t)w.x * kCols;
+          const long long i = alm_idx(a.ltop, l, m);
+#pragma unroll
+          for (int c = 0; c < NC; c += 2) {
+            if (c >= 2 * a.nv) continue;
+            const int e0 = ce[c], e1 = ce[c + 1];
+            a.out[c >> 1][i] = make_double2(e0 == kNonFinite ? nan : times_pow2(val[0][c], er + e0),
+                                            e1 == kNonFinite ? nan : times_pow2(val[0][c + 1], er + e1));
+          }
+        }
+      } else {
+        const int m = a.m0 + w.x, r = w.y * 128 + warp * 32 + lane;
+        if (r < a.R) {
+          const int cr = -68 - (int)a.cexp[(size_t)w.x * a.nkb * 64 + r];
+          const int* ce = a.colexp + (size_t)(2 * w.x) * kCols;
+#pragma unroll
+          for (int c = 0; c < NC; c += 2) {
+            if (c >= 2 * a.nv) continue;
+            double x[2][2];
+#pragma unroll
+            for (int p = 0; p < 2; ++p)
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                const int e = ce[p * kCols + c + i];
+                x[p][i] = e == kNonFinite ? nan : times_pow2(val[kSyn ? p : 0][c + i], cr + e);
+              }
+            double2* Gq = a.G + (size_t)(c >> 1) * a.qstride + (size_t)m * a.ld;
+            Gq[r] = make_double2(x[0][0] + x[1][0], x[0][1] + x[1][1]);
+            if (r + 1 != 2 * a.nside) Gq[4 * a.nside - r - 2] = make_double2(x[0][0] - x[1][0], x[0][1] - x[1][1]);
+          }
+        }
+      }
+    }
+  }
+  umma::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) umma::tmem_dealloc(tmem, 2 * kAcc);
+}
+
+template <bool kSyn, int NC>
+static int run_gemm(clc_ctx* ctx, const char* name, const DigArgs& a, const Buffer& items, int n) {
+  if (n == 0) return CLC_OK;
+  const int smem = 1024 + kDigStages * 16384 + 2 * kOpBlock * 2;
+  cudaFuncSetAttribute(k_dig_gemm<kSyn, NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  CLC_LAUNCH(ctx, name, (k_dig_gemm<kSyn, NC>), std::min(n, num_sms(ctx)), 192, smem, a, (const int4*)items.p, n,
+             ctx->d_err);
+  return launch_check(ctx, name);
+}
+
+static DigArgs dig_args(const LegendreTable& T, const __half* op, const int* colexp) {
+  DigArgs a{};
+  a.abase = (const __half* const*)T.abase.p;
+  a.rb0 = (const int*)T.rb0.p;
+  a.gidx = (const int*)T.gidx.p;
+  a.zero = (const __half*)T.zero.p;
+  a.op = op;
+  a.rexp = (const int*)T.rexp.p;
+  a.colexp = colexp;
+  a.cexp = (const int8_t*)T.cexp.p;
+  a.nside = T.nside;
+  a.lmax = T.lmax;
+  a.R = T.R;
+  a.nkb = T.nkb;
+  a.m0 = T.m0;
+  return a;
+}
+
+template <int NC>
+static int analysis_cols(clc_ctx* ctx, const LegendreTable& T, const AnaCols& c, int ldf, double2* const* out, int ltop) {
+  const int nm = T.m1 - T.m0;
+  const size_t ob = (size_t)2 * nm * T.nkb * kOpBlock * sizeof(__half);
+  __half* op = (__half*)scratch(ctx, 8, ob + sizeof(int) * 2 * nm * kCols);
+  if (!op) return CLC_ENOMEM;
+  int* colexp = (int*)((uint8_t*)op + ob);
+  CLC_LAUNCH(ctx, "k_dig_pack", k_dig_pack_analysis, dim3(nm, c.nv), 256, 0, c, T.nside, T.R, T.nkb, ldf, T.m0,
+             (const int8_t*)T.cexp.p, (const double*)T.fac.p, op, colexp);
+  if (int rc = launch_check(ctx, "k_dig_pack_analysis")) return rc;
+  DigArgs a = dig_args(T, op, colexp);
+  a.nv = c.nv;
+  for (int v = 0; v < c.nv; ++v) a.out[v] = out[v];
+  a.ltop = ltop;
+  return run_gemm<false, NC>(ctx, "k_legendre_analysis", a, T.an, T.n_an);
+}
+
+int legendre_analysis_cols(clc_ctx* ctx, const LegendreTable& T, int nv, const double2* const* F, const int* kind,
+                           int ldf, double2* const* out, int ltop) {
+  if (ltop < 0) ltop = T.lmax;
+  AnaCols c{};
+  c.nv = nv;
+  for (int v = 0; v < nv; ++v) {
+    c.F[v] = F[v];
+    c.kind[v] = kind ? kind[v] : 0;
+  }
+  // the epilogue reads and collects only the columns in use
+  if (nv == 1) return analysis_cols<2>(ctx, T, c, ldf, out, ltop);
+  if (nv <= 4) return analysis_cols<8>(ctx, T, c, ldf, out, ltop);
+  return analysis_cols<16>(ctx, T, c, ldf, out, ltop);
 }
 
 int legendre_synthesis(clc_ctx* ctx, const LegendreTable& T, const double2* rhs, int nq, const int* lq, double2* G,
                        int ld) {
-  const int L = T.lmax;
-  SynthRhs s;
+  const int nm = T.m1 - T.m0, nblk = T.h_gidx[2 * nm];
+  SynthRhs s{};
   s.rhs = rhs;
   s.nq = nq;
-  for (int q = 0; q < 3; ++q) s.lq[q] = q < nq ? lq[q] : 0;
-  dim3 grid((T.R + 127) / 128, T.m1 - T.m0);
-  const int smem = nq * (L + 2) * (int)sizeof(double2);
-  cudaFuncSetAttribute(k_legendre_synthesis, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  CLC_LAUNCH(ctx, "k_legendre_synthesis", k_legendre_synthesis, grid, 128, smem, T.nside, L, T.R, (const long long*)T.offsets.p,
-                                                         (const double*)T.data.p, s, G, ld, T.m0);
-  return launch_check(ctx, "k_legendre_synthesis");
+  for (int q = 0; q < nq; ++q) s.lq[q] = lq[q];
+  const size_t ob = (size_t)nblk * kOpBlock * sizeof(__half);
+  __half* op = (__half*)scratch(ctx, 9, ob + sizeof(int) * 2 * nm * kCols);
+  if (!op) return CLC_ENOMEM;
+  int* colexp = (int*)((uint8_t*)op + ob);
+  CLC_LAUNCH(ctx, "k_dig_pack", k_dig_pack_synthesis, dim3(nm, nq), 256, 0, s, T.lmax, T.m0, (const int*)T.gidx.p,
+             (const int*)T.rexp.p, op, colexp);
+  if (int rc = launch_check(ctx, "k_dig_pack_synthesis")) return rc;
+  DigArgs a = dig_args(T, op, colexp);
+  a.nv = nq;
+  a.G = G;
+  a.qstride = (size_t)ld * (T.lmax + 2);
+  a.ld = ld;
+  return nq == 1 ? run_gemm<true, 2>(ctx, "k_legendre_synthesis", a, T.sy, T.n_sy)
+                 : run_gemm<true, 8>(ctx, "k_legendre_synthesis", a, T.sy, T.n_sy);
 }
 
 }  // namespace clc

@@ -1,19 +1,37 @@
-// Legendre transforms of the HEALPix SHT (paper Sec. 3.2).
+// Legendre transforms of the HEALPix SHT (paper Sec. 3.2) to FP64 accuracy on
+// the tensor cores.
 #pragma once
+
+#include <cuda_fp16.h>
 
 #include "common.cuh"
 
 namespace clc {
 
-// lambda_lm(z_r) for the 2 nside northern rings (equator included), every
-// m <= lmax and l = m .. lmax + 1, stored [m][l - m][r] (r contiguous).
+constexpr int kDigits = 8;      // signed base-256 digits of a table or data value
+constexpr int kAtom = 4096;     // halves of one digit plane of a 64 x 64 atom
+
+// lambda_lm(z_r) of the orders m0 <= m < m1 on the R = 2 nside northern rings
+// (equator included), l = m .. lmax + 1, as digit planes for the contraction
+// kernels of legendre.cu.  Group g = 2 (m - m0) + p holds the rows l = m + p +
+// 2 k; 64 rows form a row block, 64 rings a ring block, and the atom of a row
+// block and a ring block is kDigits planes of 64 x 64 FP16 integers in the
+// 128-byte swizzle.  A row block keeps the atoms of its ring blocks rb0 .. nkb
+// - 1 only: towards the pole lambda_lm falls below the last digit.
 struct LegendreTable {
-  int nside = 0, lmax = 0, R = 0;
-  int m0 = 0, m1 = 0;  // orders held: m0 <= m < m1 (offsets relative to m0)
-  Buffer data;      // double
-  Buffer offsets;   // int64[lmax + 1]: start of column m (in elements)
-  std::vector<long long> h_offsets;
-  size_t elems = 0;
+  int nside = 0, lmax = 0, R = 0, nkb = 0;
+  int m0 = 0, m1 = 0;                            // orders held
+  std::vector<int> h_gidx;                       // first row block of each group (2 nm + 1)
+  Buffer gidx;                                   // the same on the device
+  Buffer rb0;                                    // int: first ring block kept, per row block
+  Buffer abase;                                  // const __half*: atom of ring block rb0, per row block
+  Buffer rexp;                                   // int: row values are below 2^rexp, 64 per row block
+  Buffer cexp;                                   // int8: ring r of order m is scaled by 2^cexp, [m - m0][nkb * 64]
+  Buffer fac;                                    // double [2][R]: cos / sin^2 and 1 / sin^2 of the rings
+  Buffer zero;                                   // an atom of zeros
+  std::vector<std::unique_ptr<Buffer>> atoms;    // the atoms, in pieces
+  Buffer an, sy;                                 // work lists of the contractions (int4), longest first
+  int n_an = 0, n_sy = 0;
 };
 
 // The whole table of (nside, lmax), cached in the context.
@@ -21,6 +39,7 @@ std::shared_ptr<LegendreTable> get_legendre_table(clc_ctx* ctx, int nside, int l
 // A table of the orders m0 <= m < m1 only (caller-owned; for solves whose
 // whole table does not fit in device memory).
 int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, LegendreTable* T);
+// bytes such a table needs at most
 size_t legendre_table_bytes(int nside, int lmax, int m0, int m1);
 
 // packed index of (l, m) for band limit lmax (m-major)
@@ -28,16 +47,61 @@ __host__ __device__ __forceinline__ long long alm_idx(int lmax, int l, int m) {
   return (long long)m * (2 * lmax + 1 - m) / 2 + l;
 }
 
-// alm[idx(l, m)] = sum_r lambda_lm(r) V_m^{(l+m) % 2}(r) from ring Fourier
-// coefficients F[m * ldf + ring] (weights already applied), for the table's
-// orders and l <= ltop (lmax by default, at most lmax + 1), packed with band
-// limit ltop.
-int legendre_analysis(clc_ctx* ctx, const LegendreTable& T, const double2* F, int ldf, double2* alm, int ltop = -1);
+// For v < nv <= 8: out[v][idx(l, m)] = sum_r lambda_lm(r) w_v(r) V_m^{(l+m) % 2}(r)
+// from ring Fourier coefficients F[v][m * ldf + ring] (weights already
+// applied), for the table's orders and l <= ltop (lmax by default, at most
+// lmax + 1), packed with band limit ltop.  V^p is north + (-1)^p south;
+// kind[v] (null: all 0) selects the ring weight w: 0: 1; 1: cos / sin^2 (odd
+// under the reflection, so V^p is north - (-1)^p south); 2: 1 / sin^2.
+int legendre_analysis_cols(clc_ctx* ctx, const LegendreTable& T, int nv, const double2* const* F, const int* kind,
+                           int ldf, double2* const* out, int ltop = -1);
+inline int legendre_analysis(clc_ctx* ctx, const LegendreTable& T, const double2* F, int ldf, double2* alm,
+                             int ltop = -1) {
+  return legendre_analysis_cols(ctx, T, 1, &F, nullptr, ldf, &alm, ltop);
+}
 
-// G_q[m][ring] = sum_l lambda_lm(ring) rhs_q[idx'(l, m)] for q < nq, where
+// G_q[m][ring] = sum_l lambda_lm(ring) rhs_q[idx'(l, m)] for q < nq <= 4, where
 // rhs_q is packed with band limit lmax + 1 (idx' = alm_idx(lmax + 1, l, m)) and
 // lq[q] is the highest l used by rhs q.  G_q lives at G + q * ld * (lmax + 2).
 int legendre_synthesis(clc_ctx* ctx, const LegendreTable& T, const double2* rhs, int nq, const int* lq,
                        double2* G, int ld);
+
+// Run fn on tables covering every order m <= lmax: the cached whole table
+// when it fits in device memory (or the context's budget), otherwise tables
+// of consecutive order ranges built one after the other, each freed before
+// the next (the recurrence is then recomputed per call).
+template <typename Fn>
+int for_each_table(clc_ctx* ctx, int nside, int lmax, Fn fn) {
+  int rc;
+  const bool cached = ctx->leg_tables.count(std::make_tuple(nside, lmax, 0)) > 0;
+  size_t freeb = 0, totalb = 0;
+  cudaMemGetInfo(&freeb, &totalb);
+  const size_t whole = legendre_table_bytes(nside, lmax, 0, lmax + 1);
+  const bool limited = ctx->table_budget > 0 && whole > ctx->table_budget;
+  if (!limited && (cached || whole + (6ull << 30) <= freeb)) {
+    auto T = get_legendre_table(ctx, nside, lmax, &rc);
+    if (rc) return rc;
+    return fn(*T);
+  }
+  size_t budget = freeb > (16ull << 30) ? freeb - (16ull << 30) : freeb / 4;
+  if (budget > (48ull << 30)) budget = 48ull << 30;
+  if (ctx->table_budget > 0 && ctx->table_budget < budget) budget = ctx->table_budget;
+  for (int m0 = 0; m0 <= lmax;) {
+    int m1 = m0 + 1;
+    size_t b = legendre_table_bytes(nside, lmax, m0, m1);
+    while (m1 <= lmax) {
+      const size_t nb = legendre_table_bytes(nside, lmax, m1, m1 + 1);
+      if (b + nb > budget) break;
+      b += nb;
+      ++m1;
+    }
+    LegendreTable T;
+    if ((rc = build_legendre_table(ctx, nside, lmax, m0, m1, &T))) return rc;
+    if ((rc = fn(T))) return rc;
+    if ((rc = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "table chunk"))) return rc;
+    m0 = m1;
+  }
+  return CLC_OK;
+}
 
 }  // namespace clc

@@ -63,44 +63,6 @@ static int check_sht_args(clc_ctx* ctx, int nside, int lmax, const char* who) {
   return CLC_OK;
 }
 
-// Run fn on FP64 Legendre tables covering every order m <= lmax: the cached
-// whole table when it fits in device memory, otherwise tables of consecutive
-// order ranges built one after the other (each freed before the next; the
-// recurrence cost is then paid per call).
-template <typename Fn>
-static int for_each_table(clc_ctx* ctx, int nside, int lmax, Fn fn) {
-  int rc;
-  const bool cached = ctx->leg_tables.count(std::make_tuple(nside, lmax, 0)) > 0;
-  size_t freeb = 0, totalb = 0;
-  cudaMemGetInfo(&freeb, &totalb);
-  const size_t whole = legendre_table_bytes(nside, lmax, 0, lmax + 1);
-  const bool limited = ctx->table_budget > 0 && whole > ctx->table_budget;
-  if (!limited && (cached || whole + (2ull << 30) <= freeb)) {
-    auto T = get_legendre_table(ctx, nside, lmax, &rc);
-    if (rc) return rc;
-    return fn(*T);
-  }
-  size_t budget = std::min<size_t>(freeb > (8ull << 30) ? freeb - (8ull << 30) : (freeb / 2), 48ull << 30);
-  if (ctx->table_budget > 0) budget = std::min(budget, ctx->table_budget);
-  int m0 = 0;
-  while (m0 <= lmax) {
-    int m1 = m0 + 1;
-    size_t b = legendre_table_bytes(nside, lmax, m0, m1);
-    while (m1 <= lmax) {
-      const size_t nb = legendre_table_bytes(nside, lmax, m1, m1 + 1);
-      if (b + nb > budget) break;
-      b += nb;
-      ++m1;
-    }
-    LegendreTable T;
-    if ((rc = build_legendre_table(ctx, nside, lmax, m0, m1, &T))) return rc;
-    if ((rc = fn(T))) return rc;
-    if ((rc = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "table chunk"))) return rc;
-    m0 = m1;
-  }
-  return CLC_OK;
-}
-
 // analysis into a device alm buffer (band limit lmax)
 int sht_analysis(clc_ctx* ctx, const double* map, int nside, int lmax, double2* alm) {
   int rc;

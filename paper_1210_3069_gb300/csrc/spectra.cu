@@ -18,8 +18,6 @@
 #include "legendre.cuh"
 #include "sphere.cuh"
 
-int clc_sht_analysis(clc_ctx*, const double*, int, int, double*);
-
 namespace clc {
 
 __device__ __forceinline__ double eps_lm(int l, int m) {
@@ -27,112 +25,52 @@ __device__ __forceinline__ double eps_lm(int l, int m) {
   return sqrt(((double)l * l - (double)m * m) / (4.0 * l * l - 1.0));
 }
 
-// block (l-block, m): warp per l (8 l per warp), lanes over the northern
-// rings, taken in chunks of kEbChunk rings staged in shared memory (the
-// ring sums of each l accumulate across chunks in registers)
-constexpr int kEbChunk = 1024;
-
-__global__ void k_legendre_eb(int nside, int lmax, int R, const long long* __restrict__ off,
-                              const double* __restrict__ tab, const double2* __restrict__ F1,
-                              const double2* __restrict__ F2, int ldf, double2* __restrict__ E,
-                              double2* __restrict__ B) {
-  extern __shared__ double2 V[];  // [4][kEbChunk]: F1 even/odd, F2 even/odd
-  const int m = blockIdx.y;
-  const int l0 = m + blockIdx.x * 64;
-  if (l0 > lmax) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double* col = tab + off[m];
-  double acc[8][4];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.0;
-  for (int c0 = 0; c0 < R; c0 += kEbChunk) {
-    const int cn = min(kEbChunk, R - c0);
-    __syncthreads();   // the previous chunk is consumed
-    for (int rr = threadIdx.x; rr < cn; rr += blockDim.x) {
-      const int i = c0 + rr + 1;
-      const bool eq = i == 2 * nside;
-      const double2 a = F1[(size_t)m * ldf + i - 1], c = F2[(size_t)m * ldf + i - 1];
-      double2 as = make_double2(0.0, 0.0), cs = make_double2(0.0, 0.0);
-      if (!eq) {
-        as = F1[(size_t)m * ldf + 4 * nside - i - 1];
-        cs = F2[(size_t)m * ldf + 4 * nside - i - 1];
-      }
-      V[rr] = make_double2(a.x + as.x, a.y + as.y);
-      V[kEbChunk + rr] = make_double2(a.x - as.x, a.y - as.y);
-      V[2 * kEbChunk + rr] = make_double2(c.x + cs.x, c.y + cs.y);
-      V[3 * kEbChunk + rr] = make_double2(c.x - cs.x, c.y - cs.y);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int l = l0 + warp + 8 * k;
-      if (l > lmax || l < 2) continue;
-      const double* row = col + (size_t)(l - m) * R;
-      const double* rowp = row + R;                              // l + 1 (table holds lmax + 1)
-      const double* rowm = l > m ? row - R : nullptr;            // l - 1
-      const double e1 = (double)l * eps_lm(l + 1, m), e0 = (l + 1.0) * eps_lm(l, m);
-      const double ll1 = (double)l * (l + 1.0), m2 = 2.0 * m * m, m_2 = 2.0 * m;
-      const int p = (l + m) & 1;
-      const double2* VA1 = V + (p ? kEbChunk : 0);          // F1 with A's parity
-      const double2* VB1 = V + (p ? 0 : kEbChunk);          // F1 with B's parity
-      const double2* VA2 = V + 2 * kEbChunk + (p ? kEbChunk : 0);
-      const double2* VB2 = V + 2 * kEbChunk + (p ? 0 : kEbChunk);
-      double ex = 0, ey = 0, bx = 0, by = 0;
-      for (int rr = lane; rr < cn; rr += 32) {
-        const int r = c0 + rr;
-        const Ring g = ring_geom(nside, r + 1);
-        const double is = 1.0 / g.s, cot = g.z * is;
-        const double lam = row[r];
-        const double dl = (e1 * rowp[r] - (rowm ? e0 * rowm[r] : 0.0)) * is;
-        const double A = -2.0 * cot * dl - (ll1 - m2 * is * is) * lam;
-        const double Bf = m_2 * is * (dl - cot * lam);
-        const double2 a1 = VA1[rr], b1 = VB1[rr], a2 = VA2[rr], b2 = VB2[rr];
-        // E += A F1 - i B F2 ; B += A F2 + i B F1
-        ex += A * a1.x + Bf * b2.y;
-        ey += A * a1.y - Bf * b2.x;
-        bx += A * a2.x - Bf * b1.y;
-        by += A * a2.y + Bf * b1.x;
-      }
-      acc[k][0] += ex;
-      acc[k][1] += ey;
-      acc[k][2] += bx;
-      acc[k][3] += by;
-    }
+// E_lm and B_lm from the Legendre sums of the two fields with the ring weights
+// 1, cos / sin^2 and 1 / sin^2 (legendre_analysis_cols, kinds 0, 1, 2; band
+// limit lmax + 1).  With sin t dlambda_lm = e1 lambda_{l+1,m} - e0 lambda_{l-1,m},
+//   sum A F  = -2 (e1 S1_{l+1} - e0 S1_{l-1}) - l(l+1) S0_l + 2 m^2 S2_l,
+//   sum B F  = 2 m (e1 S2_{l+1} - e0 S2_{l-1} - S1_l):
+// A and B are products of lambda and ring factors, so every sum over rings is
+// one of the table's contractions and nothing is evaluated per (l, m, ring).
+__global__ void k_eb_combine(const double2* __restrict__ S, size_t q, int lmax, double2* __restrict__ E,
+                             double2* __restrict__ B) {
+  const int m = blockIdx.y, lt = lmax + 1;
+  const int l = m + blockIdx.x * blockDim.x + threadIdx.x;
+  if (l > lmax) return;
+  const size_t o = alm_idx(lmax, l, m);
+  if (l < 2) {
+    E[o] = B[o] = make_double2(0.0, 0.0);
+    return;
   }
+  const double e1 = (double)l * eps_lm(l + 1, m), e0 = (l + 1.0) * eps_lm(l, m);
+  const double ll1 = (double)l * (l + 1.0), m2 = 2.0 * (double)m * m, m_2 = 2.0 * m;
+  const size_t i = alm_idx(lt, l, m);
+  double2 a[2], b[2];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int l = l0 + warp + 8 * k;
-    if (l > lmax || l >= l0 + 64) continue;
-    const size_t li = alm_idx(lmax, l, m);
-    if (l < 2) {
-      if (lane == 0) {
-        E[li] = make_double2(0.0, 0.0);
-        B[li] = make_double2(0.0, 0.0);
-      }
-      continue;
-    }
-    double ex = acc[k][0], ey = acc[k][1], bx = acc[k][2], by = acc[k][3];
-    for (int o = 16; o > 0; o >>= 1) {
-      ex += __shfl_xor_sync(0xffffffffu, ex, o);
-      ey += __shfl_xor_sync(0xffffffffu, ey, o);
-      bx += __shfl_xor_sync(0xffffffffu, bx, o);
-      by += __shfl_xor_sync(0xffffffffu, by, o);
-    }
-    if (lane == 0) {
-      const double inv = 1.0 / sqrt((l + 2.0) * (l + 1.0) * l * (l - 1.0));
-      E[li] = make_double2(ex * inv, ey * inv);
-      B[li] = make_double2(bx * inv, by * inv);
-    }
+  for (int f = 0; f < 2; ++f) {
+    const double2 *S0 = S + (3 * f) * q + i, *S1 = S0 + q, *S2 = S1 + q;
+    const double2 z = make_double2(0.0, 0.0);
+    const double2 d1 = l > m ? S1[-1] : z, d2 = l > m ? S2[-1] : z, u1 = S1[1], u2 = S2[1];
+    a[f].x = fma(-2.0, fma(e1, u1.x, -e0 * d1.x), fma(m2, S2->x, -ll1 * S0->x));
+    a[f].y = fma(-2.0, fma(e1, u1.y, -e0 * d1.y), fma(m2, S2->y, -ll1 * S0->y));
+    b[f].x = m_2 * (fma(e1, u2.x, -e0 * d2.x) - S1->x);
+    b[f].y = m_2 * (fma(e1, u2.y, -e0 * d2.y) - S1->y);
   }
+  const double inv = 1.0 / sqrt((l + 2.0) * (l + 1.0) * l * (l - 1.0));
+  // E = (A F1 - i B F2) / N_l, B = (A F2 + i B F1) / N_l
+  E[o] = make_double2((a[0].x + b[1].y) * inv, (a[0].y - b[1].x) * inv);
+  B[o] = make_double2((a[1].x - b[0].y) * inv, (a[1].y + b[0].x) * inv);
 }
 
-// C_l = (a_l0 b_l0* + 2 sum_{m>0} Re a_lm b_lm*) / (2l+1), one thread per l
-__global__ void k_cl(const double2* __restrict__ a, const double2* __restrict__ b, int lmax, double* __restrict__ cl) {
+// C_l = (a_l0 b_l0* + 2 sum_{m>0} Re a_lm b_lm*) / (2l+1), one thread per l;
+// coefficients packed with band limit lpack
+__global__ void k_cl(const double2* __restrict__ a, const double2* __restrict__ b, int lmax, int lpack,
+                     double* __restrict__ cl) {
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l > lmax) return;
   double acc = 0.0;
   for (int m = 0; m <= l; ++m) {
-    const double2 x = a[alm_idx(lmax, l, m)], y = b[alm_idx(lmax, l, m)];
+    const double2 x = a[alm_idx(lpack, l, m)], y = b[alm_idx(lpack, l, m)];
     acc += (m ? 2.0 : 1.0) * (x.x * y.x + x.y * y.y);
   }
   cl[l] = acc / (2.0 * l + 1.0);
@@ -181,25 +119,41 @@ __global__ void k_decompose_A_image(const double* __restrict__ x, const double* 
   }
 }
 
-int eb_analysis(clc_ctx* ctx, const double* g1, const double* g2, int nside, int lmax, double2* E, double2* B) {
+static int power_spectrum(clc_ctx* ctx, const double2* a, const double2* b, int lmax, int lpack, double* cl) {
+  CLC_LAUNCH(ctx, "k_cl", k_cl, (lmax + 128) / 128, 128, 0, a, b, lmax, lpack, cl);
+  return launch_check(ctx, "k_cl");
+}
+
+// E and B coefficients of the shear maps g[0], g[1], and, for ns = 2, the
+// scalar coefficients (band limit lmax + 1 packing) of the maps s[0], s[1]:
+// all in one pass over the Legendre table.
+static int eb_analysis(clc_ctx* ctx, const double* const* g, int ns, const double* const* s, int nside, int lmax,
+                       double2* E, double2* B, double2* const* salm) {
   int rc;
   auto plan = get_fft_plan(ctx, nside, &rc);
   if (rc) return rc;
-  auto T = get_legendre_table(ctx, nside, lmax, &rc);
-  if (rc) return rc;
   const int ldf = 4 * nside - 1;
-  double2* F = (double2*)scratch(ctx, 0, 2 * sizeof(double2) * (size_t)ldf * (lmax + 1));
-  if (!F) return CLC_ENOMEM;
-  double2* F2 = F + (size_t)ldf * (lmax + 1);
+  const size_t fq = (size_t)ldf * (lmax + 1), Q = (size_t)(lmax + 2) * (lmax + 3) / 2;
+  double2* F = (double2*)scratch(ctx, 0, (2 + ns) * sizeof(double2) * fq);
+  double2* S = (double2*)scratch(ctx, 2, 6 * sizeof(double2) * Q);
+  if (!F || !S) return CLC_ENOMEM;
   const double w = 4.0 * kPi / (12.0 * (double)nside * nside);
-  if ((rc = ring_analysis(ctx, *plan, g1, lmax, w, F, ldf))) return rc;
-  if ((rc = ring_analysis(ctx, *plan, g2, lmax, w, F2, ldf))) return rc;
-  dim3 grid((lmax + 1 + 63) / 64, lmax + 1);
-  const int smem = 4 * kEbChunk * (int)sizeof(double2);
-  cudaFuncSetAttribute(k_legendre_eb, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  CLC_LAUNCH(ctx, "k_legendre_eb", k_legendre_eb, grid, 256, smem, nside, lmax, T->R, (const long long*)T->offsets.p,
-             (const double*)T->data.p, F, F2, ldf, E, B);
-  return launch_check(ctx, "k_legendre_eb");
+  for (int f = 0; f < 2 + ns; ++f)
+    if ((rc = ring_analysis(ctx, *plan, f < 2 ? g[f] : s[f - 2], lmax, w, F + f * fq, ldf))) return rc;
+  const double2* cols[8];
+  double2* out[8];
+  int kind[8];
+  for (int v = 0; v < 6 + ns; ++v) {
+    cols[v] = F + (v < 6 ? v / 3 : v - 4) * fq;
+    kind[v] = v < 6 ? v % 3 : 0;
+    out[v] = v < 6 ? S + v * Q : salm[v - 6];
+  }
+  rc = for_each_table(ctx, nside, lmax, [&](const LegendreTable& T) {
+    return legendre_analysis_cols(ctx, T, 6 + ns, cols, kind, ldf, out, lmax + 1);
+  });
+  if (rc) return rc;
+  CLC_LAUNCH(ctx, "k_eb_combine", k_eb_combine, dim3((lmax + 128) / 128, lmax + 1), 128, 0, S, Q, lmax, E, B);
+  return launch_check(ctx, "k_eb_combine");
 }
 
 }  // namespace clc
@@ -213,16 +167,15 @@ extern "C" int clc_eb_analysis(clc_ctx* ctx, const double* g1, const double* g2,
     return set_err(ctx, CLC_EINVAL, "clc_eb_analysis: bad nside / lmax");
   if (!g1 || !g2 || !E || !B) return set_err(ctx, CLC_EINVAL, "clc_eb_analysis: null pointer");
   cudaSetDevice(ctx->device);
-  return eb_analysis(ctx, g1, g2, nside, lmax, (double2*)E, (double2*)B);
+  const double* g[2] = {g1, g2};
+  return eb_analysis(ctx, g, 0, nullptr, nside, lmax, (double2*)E, (double2*)B, nullptr);
 }
 
 extern "C" int clc_power_spectrum(clc_ctx* ctx, const double* alm, const double* alm2, int lmax, double* cl) {
   if (!ctx) return CLC_EINVAL;
   if (lmax < 0 || !alm || !cl) return set_err(ctx, CLC_EINVAL, "clc_power_spectrum: bad arguments");
   cudaSetDevice(ctx->device);
-  CLC_LAUNCH(ctx, "k_cl", k_cl, (lmax + 128) / 128, 128, 0, (const double2*)alm,
-             (const double2*)(alm2 ? alm2 : alm), lmax, cl);
-  return launch_check(ctx, "k_cl");
+  return power_spectrum(ctx, (const double2*)alm, (const double2*)(alm2 ? alm2 : alm), lmax, lmax, cl);
 }
 
 extern "C" int clc_lensing_spectra(clc_ctx* ctx, const double* x, const double* A, int nside, int lmax,
@@ -232,24 +185,22 @@ extern "C" int clc_lensing_spectra(clc_ctx* ctx, const double* x, const double* 
     return set_err(ctx, CLC_EINVAL, "clc_lensing_spectra: bad arguments");
   cudaSetDevice(ctx->device);
   const int64_t np = 12ll * nside * nside;
-  const size_t na = (size_t)(lmax + 1) * (lmax + 2) / 2;
-  double* maps = (double*)scratch(ctx, 5, 4 * np * sizeof(double) + 4 * na * sizeof(double2));
+  const size_t na = (size_t)(lmax + 1) * (lmax + 2) / 2, nt = (size_t)(lmax + 2) * (lmax + 3) / 2;
+  double* maps = (double*)scratch(ctx, 5, 4 * np * sizeof(double) + 2 * (na + nt) * sizeof(double2));
   if (!maps) return CLC_ENOMEM;
-  double2* alm = (double2*)(maps + 4 * np);
+  double2* E = (double2*)(maps + 4 * np);
+  double2 *B = E + na, *salm[2] = {B + na, B + na + nt};
   int rc;
   if (x)
     CLC_LAUNCH(ctx, "k_decompose_A", k_decompose_A_image, 4 * nside - 1, 256, 0, x, A, nside, np, maps);
   else
     CLC_LAUNCH(ctx, "k_decompose_A", k_decompose_A, 1024, 256, 0, A, np, maps);
   if ((rc = launch_check(ctx, "k_decompose_A"))) return rc;
-  if ((rc = clc_sht_analysis(ctx, maps, nside, lmax, (double*)alm))) return rc;                    // kappa
-  if ((rc = clc_sht_analysis(ctx, maps + 3 * np, nside, lmax, (double*)(alm + na)))) return rc;    // omega
-  if ((rc = eb_analysis(ctx, maps + np, maps + 2 * np, nside, lmax, alm + 2 * na, alm + 3 * na))) return rc;
-  for (int q = 0; q < 4; ++q) {
-    // output order: kappa, E, B, omega
-    const int src = q == 0 ? 0 : (q == 1 ? 2 : (q == 2 ? 3 : 1));
-    if ((rc = clc_power_spectrum(ctx, (const double*)(alm + src * na), nullptr, lmax, cl_out + (size_t)q * (lmax + 1))))
+  const double *g[2] = {maps + np, maps + 2 * np}, *sc[2] = {maps, maps + 3 * np};
+  if ((rc = eb_analysis(ctx, g, 2, sc, nside, lmax, E, B, salm))) return rc;
+  const double2* alm[4] = {salm[0], E, B, salm[1]};   // kappa, E, B, omega
+  for (int q = 0; q < 4; ++q)
+    if ((rc = power_spectrum(ctx, alm[q], alm[q], lmax, q == 0 || q == 3 ? lmax + 1 : lmax, cl_out + (size_t)q * (lmax + 1))))
       return rc;
-  }
   return CLC_OK;
 }
