@@ -2,7 +2,7 @@
 // along iso-latitude rings, Press et al. 2007 Sec. 6.7).  The plan of one
 // Nside holds the twiddles, the Bluestein chirps and filter spectra of the
 // non-power-of-two polar rings (FP64, plus FP32 copies for the mixed path);
-// the per-ring device code is in ring_fft.cuh.  One CTA per ring.
+// the per-ring device code is in ring_fft.cuh.
 #include <algorithm>
 
 #include "ring_fft.cuh"
@@ -45,23 +45,42 @@ __global__ void k_bluestein_tables(int nside, PlanDevT<double> P, C2<double>* ch
   for (int j = threadIdx.x; j < M; j += blockDim.x) filter[c.w + j] = s[pidx<double>(j)];
 }
 
+__global__ void k_ring_table(int nside, RingS* __restrict__ rings) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= 4 * nside - 1) return;
+  RingS o;
+  o.r = ring_geom(nside, r + 1);
+  o.is = 1.0 / o.r.s;
+  rings[r] = o;
+}
+
+// phases e^{i pi b / (4 k)}, b <= k, of ring class k = blockIdx.x + 1
+__global__ void k_phase_table(C2<double>* __restrict__ phase) {
+  const int k = blockIdx.x + 1;
+  for (int b = threadIdx.x; b <= k; b += blockDim.x)
+    phase[phase_offset(k) + b] = expi_pi<double>((double)b / (double)(4 * k));
+}
+
 __global__ void k_round_to_float(const double2* __restrict__ in, size_t n, float2* __restrict__ out) {
   for (size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (size_t)gridDim.x * blockDim.x)
     out[j] = make_float2((float)in[j].x, (float)in[j].y);
 }
 
+// one CTA per ring
 template <typename T>
-__global__ void k_ring_analysis(const double* __restrict__ map, int nside, int lmax, double weight,
-                                C2<T>* __restrict__ F, int ldf, PlanDevT<T> P) {
+__global__ void __launch_bounds__(512) k_ring_analysis(const double* __restrict__ map, int nside, int lmax,
+                                                       double weight, C2<T>* __restrict__ F, int ldf, PlanDevT<T> P) {
   extern __shared__ __align__(16) unsigned char smem_fft[];
   ring_analysis_ring<T>(map, nside, lmax, weight, F, ldf, P, blockIdx.x + 1, reinterpret_cast<C2<T>*>(smem_fft));
 }
 
+// one CTA per (field, ring)
 template <typename T>
-__global__ void k_ring_synthesis(SynthArgsT<T> a, int nside, int lmax, int mode, int mmax_fft, PlanDevT<T> P) {
+__global__ void __launch_bounds__(512) k_ring_synthesis(SynthArgsT<T> a, int nside, int lmax, int mode, PlanDevT<T> P,
+                                                        int buf_len) {
   extern __shared__ __align__(16) unsigned char smem_fft[];
-  C2<T>* s = reinterpret_cast<C2<T>*>(smem_fft);
-  ring_synthesis_ring<T>(a, nside, lmax, mode, P, blockIdx.x + 1, s, s + fft_buf_len<T>(mmax_fft));
+  ring_synthesis_ring<T>(a, nside, lmax, mode, P, blockIdx.y + 1, blockIdx.x, reinterpret_cast<C2<T>*>(smem_fft),
+                         buf_len);
 }
 
 template <>
@@ -71,6 +90,8 @@ PlanDevT<double> plan_dev<double>(const FftPlan& p) {
   d.cls = (const int4*)p.cls.p;
   d.chirp = (const C2<double>*)p.chirp.p;
   d.filter = (const C2<double>*)p.filter.p;
+  d.rings = (const RingS*)p.rings.p;
+  d.phase = (const C2<double>*)p.phase.p;
   d.logmmax = 0;
   while ((1 << d.logmmax) < p.mmax_fft) ++d.logmmax;
   return d;
@@ -83,6 +104,8 @@ PlanDevT<float> plan_dev<float>(const FftPlan& p) {
   d.cls = (const int4*)p.cls.p;
   d.chirp = (const C2<float>*)p.chirp32.p;
   d.filter = (const C2<float>*)p.filter32.p;
+  d.rings = (const RingS*)p.rings.p;
+  d.phase = (const C2<double>*)p.phase.p;
   d.logmmax = 0;
   while ((1 << d.logmmax) < p.mmax_fft) ++d.logmmax;
   return d;
@@ -131,7 +154,8 @@ std::shared_ptr<FftPlan> get_fft_plan(clc_ctx* ctx, int nside, int* rc) {
   if (!alloc(p->twiddle, sizeof(double2) * std::max(mmax / 2, 1)) || !alloc(p->cls, sizeof(int4) * cls.size()) ||
       !alloc(p->chirp, sizeof(double2) * chirp_n) || !alloc(p->filter, sizeof(double2) * filt_n) ||
       !alloc(p->twiddle32, sizeof(float2) * std::max(mmax / 2, 1)) || !alloc(p->chirp32, sizeof(float2) * chirp_n) ||
-      !alloc(p->filter32, sizeof(float2) * filt_n)) {
+      !alloc(p->filter32, sizeof(float2) * filt_n) || !alloc(p->rings, sizeof(RingS) * (4 * (size_t)nside - 1)) ||
+      !alloc(p->phase, sizeof(double2) * phase_offset(nside + 1))) {
     *rc = set_err(ctx, CLC_ENOMEM, "FFT plan allocation failed");
     return nullptr;
   }
@@ -139,6 +163,8 @@ std::shared_ptr<FftPlan> get_fft_plan(clc_ctx* ctx, int nside, int* rc) {
                                         ctx->stream), "plan upload");
   if (*rc) return nullptr;
   CLC_LAUNCH(ctx, "k_twiddle", k_twiddle, 64, 256, 0, (double2*)p->twiddle.p, mmax);
+  CLC_LAUNCH(ctx, "k_ring_table", k_ring_table, (4 * nside + 126) / 128, 128, 0, nside, (RingS*)p->rings.p);
+  CLC_LAUNCH(ctx, "k_phase_table", k_phase_table, nside, 256, 0, (C2<double>*)p->phase.p);
   PlanDevT<double> d = plan_dev<double>(*p);
   if (nside > 1 && chirp_n > 0) {
     const int smem = fft_buf_len<double>(mmax) * (int)sizeof(double2);
@@ -164,9 +190,9 @@ template <typename T>
 int ring_analysis_t(clc_ctx* ctx, const FftPlan& plan, const double* map, int lmax, double weight, C2<T>* F,
                     int ldf) {
   const int nside = plan.nside;
-  const int smem = ring_analysis_smem<T>(plan);
+  const int smem = ring_fft_smem<T>(plan);
   cudaFuncSetAttribute(k_ring_analysis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  CLC_LAUNCH(ctx, "k_ring_analysis", (k_ring_analysis<T>), 4 * nside - 1, 256, smem, map, nside, lmax, weight, F, ldf,
+  CLC_LAUNCH(ctx, "k_ring_analysis", (k_ring_analysis<T>), 4 * nside - 1, std::max(128, ring_fft_threads(plan.mmax_fft)), smem, map, nside, lmax, weight, F, ldf,
              plan_dev<T>(plan));
   return launch_check(ctx, "k_ring_analysis");
 }
@@ -187,10 +213,11 @@ int ring_synthesis_t(clc_ctx* ctx, const FftPlan& plan, const C2<T>* G, int ld, 
   a.p01q = a.p01m = 0;
   a.ncap = a.nring = 0;
   for (int f = 0; f < 6; ++f) a.out[f] = out[f];
-  const int smem = ring_synthesis_smem<T>(plan);
+  const int smem = ring_fft_smem<T>(plan);
   cudaFuncSetAttribute(k_ring_synthesis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  CLC_LAUNCH(ctx, "k_ring_synthesis", (k_ring_synthesis<T>), 4 * nside - 1, 256, smem, a, nside, lmax, mode,
-             plan.mmax_fft, plan_dev<T>(plan));
+  CLC_LAUNCH(ctx, "k_ring_synthesis", (k_ring_synthesis<T>), dim3(mode ? 6 : 1, 4 * nside - 1),
+             ring_fft_threads(plan.mmax_fft), smem, a, nside, lmax, mode, plan_dev<T>(plan),
+             smem / (int)sizeof(C2<T>));
   return launch_check(ctx, "k_ring_synthesis");
 }
 

@@ -11,6 +11,17 @@ struct alignas(2 * sizeof(T)) C2 {
   T x, y;
 };
 
+// Geometry of a ring with 1 / sin(theta)
+struct RingS {
+  Ring r;
+  double is;
+};
+
+// The phase table of ring class k (1 .. nside - 1: the polar rings of 4 k
+// pixels; nside: the equatorial rings) holds e^{i pi b / n}, b <= n / 4 = k, at
+// phase_offset(k) + b.
+__host__ __device__ constexpr int phase_offset(int k) { return (k - 1) * (k + 2) / 2; }
+
 struct FftPlan {
   int nside = 0;
   int mmax_fft = 0;        // largest complex FFT size used by any ring
@@ -19,6 +30,8 @@ struct FftPlan {
   Buffer chirp;            // double2: e^{i pi j^2 / N} per Bluestein class
   Buffer filter;           // double2: FFT_M of the Bluestein filter per class
   Buffer twiddle32, chirp32, filter32;   // the same tables rounded to FP32
+  Buffer rings;            // RingS[4 nside - 1]
+  Buffer phase;            // double2: phase_offset(nside + 1) phases
   size_t chirp_n = 0, filt_n = 0;
 };
 
@@ -28,6 +41,8 @@ struct PlanDevT {
   const int4* cls;
   const C2<T>* chirp;
   const C2<T>* filter;
+  const RingS* rings;
+  const C2<double>* phase;
   int logmmax;
 };
 
@@ -42,12 +57,11 @@ template <typename T>
 __host__ __device__ constexpr int fft_buf_len(int m) { return m + (m >> fft_pad_shift<T>()) + 1; }
 template <typename T>
 PlanDevT<T> plan_dev(const FftPlan& p);
-// dynamic shared memory of the ring kernels (analysis: FFT buffer; synthesis:
-// FFT buffer + N + 1 spectrum points)
+// dynamic shared memory of the ring kernels: the FFT buffer
 template <typename T>
-int ring_analysis_smem(const FftPlan& p) { return fft_buf_len<T>(p.mmax_fft) * (int)sizeof(C2<T>); }
-template <typename T>
-int ring_synthesis_smem(const FftPlan& p) { return (fft_buf_len<T>(p.mmax_fft) + 2 * p.nside + 1) * (int)sizeof(C2<T>); }
+int ring_fft_smem(const FftPlan& p) { return fft_buf_len<T>(p.mmax_fft) * (int)sizeof(C2<T>); }
+// threads of a ring block: one per 16 points of the longest FFT
+inline int ring_fft_threads(int mmax) { return mmax / 16 < 64 ? 64 : mmax / 16 > 512 ? 512 : mmax / 16; }
 
 // F[m * ldf + (i - 1)] = sum_j map_j e^{-i m phi_j} over ring i, m = 0 .. lmax,
 // times `weight` (all 4 nside - 1 rings; ldf >= 4 nside - 1).

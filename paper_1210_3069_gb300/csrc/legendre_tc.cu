@@ -210,12 +210,12 @@ __device__ __forceinline__ int find_class(const TcBatchDev& b, long long idx, lo
 }
 
 // ---------------------------------------------------------------------------
-// ring FFTs (FP32) of every plane of every class; one ring per CTA at a time
-// (512 threads for the six-field synthesis, 256 for the analysis)
+// ring FFTs (FP32) of every plane of every class: a block takes one ring
+// (analysis) or one field of one ring (synthesis) at a time
 
-constexpr int kRingThreads = 512;
+constexpr int kRingThreads = 512;   // most threads of a block (ring_fft_threads)
 
-__global__ void k_tc_ring_analysis(TcBatchDev b) {
+__global__ void __launch_bounds__(kRingThreads) k_tc_ring_analysis(TcBatchDev b) {
   extern __shared__ __align__(16) unsigned char smem_ra[];
   C2<float>* s = reinterpret_cast<C2<float>*>(smem_ra);
   for (long long it = blockIdx.x; it < b.n_ring; it += gridDim.x) {
@@ -228,10 +228,13 @@ __global__ void k_tc_ring_analysis(TcBatchDev b) {
   }
 }
 
-__global__ void __launch_bounds__(kRingThreads, 2) k_tc_ring_synthesis(TcBatchDev b) {
+__global__ void __launch_bounds__(kRingThreads) k_tc_ring_synthesis(TcBatchDev b, int buf_len) {
   extern __shared__ __align__(16) unsigned char smem_rs[];
   C2<float>* s = reinterpret_cast<C2<float>*>(smem_rs);
-  for (long long it = blockIdx.x; it < b.n_ring; it += gridDim.x) {
+  const int nf = b.mode ? 6 : 1;
+  for (long long u = blockIdx.x; u < b.n_ring * nf; u += gridDim.x) {
+    const long long it = u / nf;
+    const int f = (int)(u - it * nf);
     const TcClass& C = b.cls[find_class(b, it, &TcClass::ring0)];
     const long long loc = it - C.ring0;
     const int nr = 4 * C.nside - 1;
@@ -250,8 +253,8 @@ __global__ void __launch_bounds__(kRingThreads, 2) k_tc_ring_synthesis(TcBatchDe
     a.ncap = C.ncap;
     a.nring = C.ldf;
     double* const* o = b.out + (size_t)(C.plane0 + pl) * 6;
-    for (int f = 0; f < 6; ++f) a.out[f] = o[f];
-    ring_synthesis_ring<float>(a, C.nside, C.lmax, b.mode, C.fft, i, s, s + fft_buf_len<float>(C.mmax));
+    for (int k = 0; k < 6; ++k) a.out[k] = o[k];
+    ring_synthesis_ring<float>(a, C.nside, C.lmax, b.mode, C.fft, i, f, s, buf_len);
   }
 }
 
@@ -755,14 +758,14 @@ int tc_build_items(clc_ctx* ctx, const TcBatchDev& b, const std::vector<std::sha
   std::vector<std::pair<int, int4>> an, sy;   // (stages, item): longer items first
   it->na_max = 16;
   it->ns_max = 16;
-  it->fft_an_smem = it->fft_sy_smem = it->pack_s_smem = 0;
+  it->fft_smem = it->fft_threads = it->pack_s_smem = 0;
   for (int c = 0; c < b.ncls; ++c) {
     const TcClass& C = b.cls[c];
     const TcTable& T = *tabs[c];
     it->na_max = std::max(it->na_max, C.Na);
     it->ns_max = std::max(it->ns_max, C.Ns);
-    it->fft_an_smem = std::max(it->fft_an_smem, fft_buf_len<float>(C.mmax) * (int)sizeof(float2));
-    it->fft_sy_smem = std::max(it->fft_sy_smem, (fft_buf_len<float>(C.mmax) + 2 * C.nside + 1) * (int)sizeof(float2));
+    it->fft_smem = std::max(it->fft_smem, fft_buf_len<float>(C.mmax) * (int)sizeof(float2));
+    it->fft_threads = std::max(it->fft_threads, ring_fft_threads(C.mmax));
     it->pack_s_smem = std::max(it->pack_s_smem, 3 * T.h_pad[0] * (int)sizeof(float));
     for (int m = 0; m <= C.lmax; ++m)
       for (int p = 0; p < 2; ++p)
@@ -811,9 +814,9 @@ static int grid_of(clc_ctx* ctx, K kern, int threads, int smem, long long items,
 int tc_run_stage(clc_ctx* ctx, const TcBatchDev& b, const TcItems& it, const TcLaunch& L, int stage) {
   switch (stage) {
     case 0: {
-      cudaFuncSetAttribute(k_tc_ring_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, it.fft_an_smem);
-      const int g = grid_of(ctx, k_tc_ring_analysis, 256, it.fft_an_smem, b.n_ring, L.fft_ctas);
-      CLC_LAUNCH(ctx, "k_tc_ring_analysis", k_tc_ring_analysis, g, 256, it.fft_an_smem, b);
+      cudaFuncSetAttribute(k_tc_ring_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, it.fft_smem);
+      const int g = grid_of(ctx, k_tc_ring_analysis, it.fft_threads, it.fft_smem, b.n_ring, L.fft_ctas);
+      CLC_LAUNCH(ctx, "k_tc_ring_analysis", k_tc_ring_analysis, g, it.fft_threads, it.fft_smem, b);
       return launch_check(ctx, "k_tc_ring_analysis");
     }
     case 1: {
@@ -854,9 +857,10 @@ int tc_run_stage(clc_ctx* ctx, const TcBatchDev& b, const TcItems& it, const TcL
       return launch_check(ctx, "k_tc_synthesis");
     }
     default: {
-      cudaFuncSetAttribute(k_tc_ring_synthesis, cudaFuncAttributeMaxDynamicSharedMemorySize, it.fft_sy_smem);
-      const int g = grid_of(ctx, k_tc_ring_synthesis, kRingThreads, it.fft_sy_smem, b.n_ring, L.fft_ctas);
-      CLC_LAUNCH(ctx, "k_tc_ring_synthesis", k_tc_ring_synthesis, g, kRingThreads, it.fft_sy_smem, b);
+      cudaFuncSetAttribute(k_tc_ring_synthesis, cudaFuncAttributeMaxDynamicSharedMemorySize, it.fft_smem);
+      const int g = grid_of(ctx, k_tc_ring_synthesis, it.fft_threads, it.fft_smem, b.n_ring * (b.mode ? 6 : 1), L.fft_ctas);
+      CLC_LAUNCH(ctx, "k_tc_ring_synthesis", k_tc_ring_synthesis, g, it.fft_threads, it.fft_smem, b,
+                 it.fft_smem / (int)sizeof(float2));
       return launch_check(ctx, "k_tc_ring_synthesis");
     }
   }

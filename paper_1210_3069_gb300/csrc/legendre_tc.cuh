@@ -76,7 +76,7 @@ struct TcBatchDev {
 struct TcLaunch {
   int an_stages = 2, an_ctas = 2;     // analysis pipeline depth, resident CTAs per SM
   int sy_stages = 2, sy_ctas = 2;     // synthesis
-  int fft_ctas = 4;                   // ring FFT kernels, resident CTAs per SM
+  int fft_ctas = 8;                   // ring FFT kernels, resident CTAs per SM
 };
 
 // Device-side work lists of a batch (built once per batch layout).
@@ -84,7 +84,7 @@ struct TcItems {
   Buffer an, sy;                      // int4 items: analysis (cls, grp, tile, 0), synthesis (cls, m, ring tile, 0)
   int n_an = 0, n_sy = 0;
   int na_max = 16, ns_max = 16;       // widest operands (TMEM columns, stage sizes)
-  int fft_an_smem = 0, fft_sy_smem = 0, pack_s_smem = 0;
+  int fft_smem = 0, fft_threads = 64, pack_s_smem = 0;
 };
 
 int tc_build_items(clc_ctx* ctx, const TcBatchDev& b, const std::vector<std::shared_ptr<TcTable>>& tabs,

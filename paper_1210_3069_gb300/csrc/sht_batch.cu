@@ -301,7 +301,7 @@ static int tc_autotune(TcBatch* B) {
     TcLaunch pick = L;
     std::vector<TcLaunch> cand;
     if (stage == 0 || stage == 5) {
-      for (int c : {2, 4, 8}) {
+      for (int c : {4, 8, 16}) {
         TcLaunch x = L;
         x.fft_ctas = c;
         cand.push_back(x);
