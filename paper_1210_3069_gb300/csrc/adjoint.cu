@@ -11,12 +11,12 @@
 // The ray state entering every plane is checkpointed.
 //
 // Reverse: planes from last to first.  Each plane's lens maps are recomputed
-// from its convergence map; each ray's step is re-run from its checkpoint
-// with forward-mode dual numbers, which give the vector-Jacobian product of
-// the step with respect to the entering state (including the dependence of
-// the lens lookup on the ray position) and to the five lens values at the
-// ray; the latter are scattered through the interpolation weights into
-// adjoint lens maps, and the adjoint SHT Poisson solve (transposed ring
+// from its convergence map; each ray's step is re-run from its checkpoint and
+// reversed formula by formula, which gives the adjoints of the entering state
+// and of the five lens values at the ray; the dependence of the lens lookup on
+// the ray position comes from dual numbers in the two tangent directions at
+// the ray.  The lens adjoints are scattered through the interpolation weights
+// into adjoint lens maps, and the adjoint SHT Poisson solve (transposed ring
 // FFTs, transposed derivative combinations, transposed Legendre synthesis,
 // transposed Poisson and analysis) turns them into the gradient map.
 #include "fft.cuh"
@@ -196,237 +196,332 @@ __device__ __forceinline__ void basis_s(const S n[3], S t[3], S p[3]) {
   p[1] = n[0] / rho;
   p[2] = Lift<S>::of(0.0);
 }
-// rotate v about unit axis k by the angle with cosine c, sine s
-template <typename S>
-__device__ __forceinline__ void rodrigues_s(const S v[3], const S k[3], const S& c, const S& s, S o[3]) {
-  S kv[3];
-  cross3s(k, v, kv);
-  const S kd = dot3s(k, v) * (1.0 - c);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) o[i] = v[i] * c + kv[i] * s + k[i] * kd;
-}
-// transport matrix Q (2x2) from the tangent basis at n0 to the one at n1 (Appendix B)
-template <typename S>
-__device__ void transport_q_s(const S n0[3], const S n1[3], S Q[4]) {
-  S cr[3];
-  cross3s(n0, n1, cr);
-  const S s = sqrt(dot3s(cr, cr));
-  const S c = dot3s(n0, n1);
-  S t0[3], p0[3], t1[3], p1[3], tr[3], pr[3];
-  basis_s(n0, t0, p0);
-  basis_s(n1, t1, p1);
-  if (val(s) > 0.0) {
-    const S k[3] = {cr[0] / s, cr[1] / s, cr[2] / s};
-    rodrigues_s(t0, k, c, s, tr);
-    rodrigues_s(p0, k, c, s, pr);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      tr[i] = t0[i];
-      pr[i] = p0[i];
-    }
-  }
-  Q[0] = dot3s(t1, tr);
-  Q[1] = dot3s(t1, pr);
-  Q[2] = dot3s(p1, tr);
-  Q[3] = dot3s(p1, pr);
-}
-template <typename S>
-__device__ __forceinline__ void qaqt_s(const S Q[4], const S A[4], S o[4]) {
-  const S m0 = Q[0] * A[0] + Q[1] * A[2], m1 = Q[0] * A[1] + Q[1] * A[3];
-  const S m2 = Q[2] * A[0] + Q[3] * A[2], m3 = Q[2] * A[1] + Q[3] * A[3];
-  o[0] = m0 * Q[0] + m1 * Q[1];
-  o[1] = m0 * Q[2] + m1 * Q[3];
-  o[2] = m2 * Q[0] + m3 * Q[1];
-  o[3] = m2 * Q[2] + m3 * Q[3];
-}
-
 struct StepC {
   double c, d, dchi2;
 };
 
-// One plane (Eq. Atraj, Eq. betaprop, Eq. posprop, Appendix B) given the
-// lens values L = (alpha_t, alpha_p, U_tt, U_pp, U_tp) at the ray:
-// out = x1[3], beta1[3], A^(n+1)[4], A^(n)[4] (both in the basis at x1).
-template <typename S>
-__device__ void step_eval(const S x[3], const S be[3], const S A[4], const S Ap[4], const S L[5], const StepC& sc,
-                          S out[14]) {
-  const S xn = sqrt(dot3s(x, x));
-  const S nv[3] = {x[0] / xn, x[1] / xn, x[2] / xn};
-  S An[4];
-  An[0] = (1.0 - sc.c) * Ap[0] + sc.c * A[0] - sc.d * (L[2] * A[0] + L[4] * A[2]);
-  An[1] = (1.0 - sc.c) * Ap[1] + sc.c * A[1] - sc.d * (L[2] * A[1] + L[4] * A[3]);
-  An[2] = (1.0 - sc.c) * Ap[2] + sc.c * A[2] - sc.d * (L[4] * A[0] + L[3] * A[2]);
-  An[3] = (1.0 - sc.c) * Ap[3] + sc.c * A[3] - sc.d * (L[4] * A[1] + L[3] * A[3]);
-  S t[3], q[3];
-  basis_s(nv, t, q);
-  const S av[3] = {L[0] * t[0] + L[1] * q[0], L[0] * t[1] + L[1] * q[1], L[0] * t[2] + L[1] * q[2]};
-  const S am = sqrt(dot3s(av, av));
-  S bn[3] = {be[0], be[1], be[2]};
-  if (val(am) > 0.0) {
-    S kx[3];
-    cross3s(nv, av, kx);
-    const S kk[3] = {kx[0] / am, kx[1] / am, kx[2] / am};
-    S sn, cs;
-    sincos(am, &sn, &cs);
-    rodrigues_s(be, kk, cs, sn, bn);
-  }
-  const S xb = dot3s(x, bn);
-  const S lam = sc.dchi2 / (xb + sqrt(xb * xb + sc.dchi2));
-  S x1[3];
+// One plane (Eq. Atraj, Eq. betaprop, Eq. posprop, Appendix B) with what its
+// reverse needs.  The deflection rotates beta about kk = n x alpha (unnormalised)
+// by a = |alpha|: bn = beta cos a + (kk x beta) sin(a) / a + kk (kk . beta)
+// (1 - cos a) / a^2, coefficients even in a; the transport is the plane
+// rotation q0, q1 of Appendix B (rays.cu).
+struct StepFwd {
+  double xn, n[3], t[3], q[3];            // at the plane
+  double An[4];                           // A^(n+1) in the basis at n
+  double av[3], kk[3], cs, sc, vc, dsc, dvc;   // rotation: coefficients and d sc, d vc / d a^2
+  bool turned;
+  double bn[3], sq, lam;
+  double x1[3], x1n, n1[3], t1[3], p1[3];
+  double w, ic, q0, q1;                   // transport; ic = 1 / (1 + n . n1)
+};
+
+__device__ __forceinline__ void step_basis(const double x[3], StepFwd& f) {
+  f.xn = ::sqrt(dot3s(x, x));
+  const double ix = 1.0 / f.xn;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) x1[c] = x[c] + lam * bn[c];
-  const S x1n = sqrt(dot3s(x1, x1));
-  const S n1[3] = {x1[0] / x1n, x1[1] / x1n, x1[2] / x1n};
-  S Q[4];
-  transport_q_s(nv, n1, Q);
-  qaqt_s(Q, An, out + 6);
-  qaqt_s(Q, A, out + 10);
+  for (int c = 0; c < 3; ++c) f.n[c] = x[c] * ix;
+  basis_s(f.n, f.t, f.q);
+}
+
+// o = Q A Q^T for Q = [[q0, -q1], [q1, q0]]
+__device__ __forceinline__ void turn_2x2(double q0, double q1, const double A[4], double o[4]) {
+  const double m0 = q0 * A[0] - q1 * A[2], m1 = q0 * A[1] - q1 * A[3];
+  const double m2 = q1 * A[0] + q0 * A[2], m3 = q1 * A[1] + q0 * A[3];
+  o[0] = m0 * q0 - m1 * q1;
+  o[1] = m0 * q1 + m1 * q0;
+  o[2] = m2 * q0 - m3 * q1;
+  o[3] = m2 * q1 + m3 * q0;
+}
+
+// f.xn .. f.q set by step_basis
+__device__ void step_forward(const double x[3], const double be[3], const double A[4], const double Ap[4],
+                             const double L[5], const StepC& sc, StepFwd& f) {
+  f.An[0] = (1.0 - sc.c) * Ap[0] + sc.c * A[0] - sc.d * (L[2] * A[0] + L[4] * A[2]);
+  f.An[1] = (1.0 - sc.c) * Ap[1] + sc.c * A[1] - sc.d * (L[2] * A[1] + L[4] * A[3]);
+  f.An[2] = (1.0 - sc.c) * Ap[2] + sc.c * A[2] - sc.d * (L[4] * A[0] + L[3] * A[2]);
+  f.An[3] = (1.0 - sc.c) * Ap[3] + sc.c * A[3] - sc.d * (L[4] * A[1] + L[3] * A[3]);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    out[c] = x1[c];
-    out[3 + c] = bn[c];
+    f.av[c] = L[0] * f.t[c] + L[1] * f.q[c];
+    f.bn[c] = be[c];
+  }
+  const double a2 = dot3s(f.av, f.av);
+  f.turned = a2 > 0.0;
+  if (f.turned) {
+    cross3s(f.n, f.av, f.kk);
+    if (a2 < 0.0009765625) {   // Maclaurin series in a^2, first omitted terms below 1e-19
+      f.cs = 1.0 - a2 * (0.5 - a2 * ((1.0 / 24.0) - a2 * ((1.0 / 720.0) - a2 * (1.0 / 40320.0))));
+      f.sc = 1.0 - a2 * ((1.0 / 6.0) - a2 * ((1.0 / 120.0) - a2 * ((1.0 / 5040.0) - a2 * (1.0 / 362880.0))));
+      f.vc = 0.5 - a2 * ((1.0 / 24.0) - a2 * ((1.0 / 720.0) - a2 * ((1.0 / 40320.0) - a2 * (1.0 / 3628800.0))));
+      f.dsc = -(1.0 / 6.0) + a2 * ((1.0 / 60.0) - a2 * ((1.0 / 1680.0) - a2 * ((1.0 / 90720.0) - a2 * (1.0 / 7983360.0))));
+      f.dvc = -(1.0 / 24.0) + a2 * ((1.0 / 360.0) - a2 * ((1.0 / 13440.0) - a2 * ((1.0 / 907200.0) - a2 * (1.0 / 95800320.0))));
+    } else {
+      const double a = ::sqrt(a2);
+      double sn;
+      ::sincos(a, &sn, &f.cs);
+      f.sc = sn / a;
+      f.vc = (1.0 - f.cs) / a2;
+      f.dsc = 0.5 * (f.cs - f.sc) / a2;
+      f.dvc = (0.5 * f.sc - f.vc) / a2;
+    }
+    double kb[3];
+    cross3s(f.kk, be, kb);
+    const double kd = dot3s(f.kk, be) * f.vc;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f.bn[c] = be[c] * f.cs + kb[c] * f.sc + f.kk[c] * kd;
+  }
+  const double xb = dot3s(x, f.bn);
+  f.sq = ::sqrt(xb * xb + sc.dchi2);
+  f.lam = sc.dchi2 / (xb + f.sq);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) f.x1[c] = x[c] + f.lam * f.bn[c];
+  f.x1n = ::sqrt(dot3s(f.x1, f.x1));
+  const double i1 = 1.0 / f.x1n;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) f.n1[c] = f.x1[c] * i1;
+  basis_s(f.n1, f.t1, f.p1);
+  f.ic = 1.0 / (1.0 + dot3s(f.n, f.n1));
+  f.w = dot3s(f.n1, f.t) * f.ic;
+  f.q0 = dot3s(f.t1, f.t) - f.w * dot3s(f.t1, f.n);
+  f.q1 = dot3s(f.p1, f.t) - f.w * dot3s(f.p1, f.n);
+}
+
+// out = x1[3], beta1[3], A^(n+1)[4], A^(n)[4] (both in the basis at x1)
+__device__ __forceinline__ void step_out(const StepFwd& f, const double A[4], double out[14]) {
+  turn_2x2(f.q0, f.q1, f.An, out + 6);
+  turn_2x2(f.q0, f.q1, A, out + 10);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    out[c] = f.x1[c];
+    out[3 + c] = f.bn[c];
   }
 }
 
-// ring pair bracketing phi on ring i with the fraction f (templated in phi)
-template <typename S>
-__device__ __forceinline__ void ring_pair_s(int nside, int i, const S& phi, int64_t* p0, int64_t* p1, S* f) {
-  const Ring r = ring_geom(nside, i);
-  const S t = (phi - r.phi0) * ((double)r.npix / (2.0 * kPi));
-  const double j0 = floor(val(t));
-  *f = t - j0;
-  int64_t j = imod((int64_t)j0, r.npix);
-  *p0 = r.first + j;
-  *p1 = r.first + (j + 1 == r.npix ? 0 : j + 1);
+// nb += adjoint of basis_s at n for the adjoints tb, pb of (theta-hat, phi-hat)
+__device__ __forceinline__ void basis_reverse(const double n[3], const double tb[3], const double pb[3], double nb[3]) {
+  const double ir = 1.0 / ::sqrt(n[0] * n[0] + n[1] * n[1]);
+  const double ux = n[0] * ir, uy = n[1] * ir;   // theta-hat = (z u, -rho), phi-hat = (-u_y, u_x)
+  const double ubx = n[2] * tb[0] + pb[1], uby = n[2] * tb[1] - pb[0];
+  const double ru = (ux * ubx + uy * uby) * ir + tb[2];   // radial part of u's adjoint and rho's
+  nb[0] += ubx * ir - ux * ru;
+  nb[1] += uby * ir - uy * ru;
+  nb[2] += ux * tb[0] + uy * tb[1];
 }
 
-// Ring-bilinear interpolation weights (with the polar blend) at (theta, phi),
-// templated in the position: the pixels follow the values, the weights carry
-// the tangents.
+// o = Q M Q^T: adjoint of M into mb (set), of (q0, q1) added
+__device__ __forceinline__ void turn_reverse(double q0, double q1, const double M[4], const double ob[4], double mb[4],
+                                             double& q0b, double& q1b) {
+  turn_2x2(q0, -q1, ob, mb);   // Q^T ob Q
+  // dQ = q0' I + q1' J, J = [[0, -1], [1, 0]]: ob . (dQ M Q^T + Q M dQ^T)
+  const double Q[4] = {q0, -q1, q1, q0};
+  double P[4], R[4];   // P = M Q^T, R = Q M
+  P[0] = M[0] * Q[0] + M[1] * Q[1];
+  P[1] = M[0] * Q[2] + M[1] * Q[3];
+  P[2] = M[2] * Q[0] + M[3] * Q[1];
+  P[3] = M[2] * Q[2] + M[3] * Q[3];
+  R[0] = Q[0] * M[0] + Q[1] * M[2];
+  R[1] = Q[0] * M[1] + Q[1] * M[3];
+  R[2] = Q[2] * M[0] + Q[3] * M[2];
+  R[3] = Q[2] * M[1] + Q[3] * M[3];
+  q0b += ob[0] * (P[0] + R[0]) + ob[1] * (P[1] + R[1]) + ob[2] * (P[2] + R[2]) + ob[3] * (P[3] + R[3]);
+  q1b += -ob[0] * P[2] - ob[1] * P[3] + ob[2] * P[0] + ob[3] * P[1]         // J P
+         - ob[0] * R[1] + ob[1] * R[0] - ob[2] * R[3] + ob[3] * R[2];       // R J^T
+}
+
+// Reverse of step_forward + step_out: from the adjoints v[14] of the outputs
+// to those of the entering state ib[14], of the lens values Lb[5] and of the
+// direction n (without its part through x / |x|) nb[3].  ib[0..2] lacks n's
+// share, which the caller adds once the lookup's is in nb.
+__device__ void step_reverse(const double x[3], const double be[3], const double A[4], const double L[5],
+                             const StepC& sc, const StepFwd& f, const double v[14], double ib[14], double Lb[5],
+                             double nb[3]) {
+  double q0b = 0.0, q1b = 0.0, Anb[4], Ab[4];
+  turn_reverse(f.q0, f.q1, f.An, v + 6, Anb, q0b, q1b);
+  turn_reverse(f.q0, f.q1, A, v + 10, Ab, q0b, q1b);
+  // transport
+  const double wb = -(q0b * dot3s(f.t1, f.n) + q1b * dot3s(f.p1, f.n));
+  const double sb = wb * f.ic, cb = -wb * f.w * f.ic;
+  double t1b[3], p1b[3], tb[3], n1b[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const double e = f.t[c] - f.w * f.n[c], g = q0b * f.t1[c] + q1b * f.p1[c];
+    t1b[c] = q0b * e;
+    p1b[c] = q1b * e;
+    tb[c] = g + sb * f.n1[c];
+    nb[c] = cb * f.n1[c] - f.w * g;
+    n1b[c] = sb * f.t[c] + cb * f.n[c];
+  }
+  basis_reverse(f.n1, t1b, p1b, n1b);
+  // x1 = x + lam bn, lam = sq - x . bn
+  const double r1 = dot3s(f.n1, n1b), i1 = 1.0 / f.x1n;
+  double xb[3], bb[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) xb[c] = v[c] + (n1b[c] - f.n1[c] * r1) * i1;
+  const double sl = -dot3s(xb, f.bn) * f.lam / f.sq;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    bb[c] = v[3 + c] + f.lam * xb[c] + sl * x[c];
+    xb[c] += sl * f.bn[c];
+  }
+  double qb[3] = {0.0, 0.0, 0.0};
+  Lb[0] = Lb[1] = 0.0;
+  if (f.turned) {
+    double kb[3], g1[3], g2[3], kkb[3], avb[3], h[3];
+    cross3s(f.kk, be, kb);
+    cross3s(bb, f.kk, g1);
+    cross3s(be, bb, g2);
+    const double kd = dot3s(f.kk, be), kv = dot3s(f.kk, bb);
+    const double a2b = -0.5 * f.sc * dot3s(be, bb) + f.dsc * dot3s(kb, bb) + f.dvc * kd * kv;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      kkb[c] = f.sc * g2[c] + f.vc * (kd * bb[c] + kv * be[c]);
+      ib[3 + c] = f.cs * bb[c] + f.sc * g1[c] + f.vc * kv * f.kk[c];
+    }
+    cross3s(kkb, f.n, avb);
+    cross3s(f.av, kkb, h);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      avb[c] += 2.0 * a2b * f.av[c];
+      nb[c] += h[c];
+      tb[c] += L[0] * avb[c];
+      qb[c] = L[1] * avb[c];
+    }
+    Lb[0] = dot3s(f.t, avb);
+    Lb[1] = dot3s(f.q, avb);
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ib[3 + c] = bb[c];
+  }
+  basis_reverse(f.n, tb, qb, nb);
+  // Eq. Atraj
+  Lb[2] = -sc.d * (Anb[0] * A[0] + Anb[1] * A[1]);
+  Lb[3] = -sc.d * (Anb[2] * A[2] + Anb[3] * A[3]);
+  Lb[4] = -sc.d * (Anb[0] * A[2] + Anb[1] * A[3] + Anb[2] * A[0] + Anb[3] * A[1]);
+  ib[6] = Ab[0] + sc.c * Anb[0] - sc.d * (L[2] * Anb[0] + L[4] * Anb[2]);
+  ib[7] = Ab[1] + sc.c * Anb[1] - sc.d * (L[2] * Anb[1] + L[4] * Anb[3]);
+  ib[8] = Ab[2] + sc.c * Anb[2] - sc.d * (L[4] * Anb[0] + L[3] * Anb[2]);
+  ib[9] = Ab[3] + sc.c * Anb[3] - sc.d * (L[4] * Anb[1] + L[3] * Anb[3]);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) ib[10 + c] = (1.0 - sc.c) * Anb[c];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) ib[c] = xb[c];
+}
+
+// Lens lookup from RING maps: ring-bilinear interpolation (with the polar
+// blend) at the unit vector nv of alpha as a tangent 3-vector and U as a
+// symmetric tangent 3x3 tensor.  Per pixel k: index p, weight w (templated in
+// the position: the pixels follow the values, the weights carry the tangents)
+// and the pixel's basis.  Ring colatitudes and geometry come from the plan's
+// table: computing them here (an FP64 division, square root and atan2 per
+// ring) was most of the lookup.
 template <typename S>
 struct InterpS {
-  int64_t p[8];
-  S w[8];
+  int64_t p[6];
+  S w[6];
+  double t[6][3], q[6][2];   // theta-hat, phi-hat (third component 0)
   int n;
 };
 
 template <typename S>
-__device__ void interp_weights_s(int nside, const S& theta, const S& phi, InterpS<S>& o) {
+__device__ __forceinline__ void interp_pixel(const Ring& r, int64_t j, const S& w, InterpS<S>& o, int k) {
+  o.p[k] = r.first + j;
+  o.w[k] = w;
+  double sp, cp;
+  sincospi((double)(2 * j + (r.phi0 != 0.0 ? 1 : 0)) / (double)r.npix, &sp, &cp);
+  o.t[k][0] = r.z * cp;
+  o.t[k][1] = r.z * sp;
+  o.t[k][2] = -r.s;
+  o.q[k][0] = -sp;
+  o.q[k][1] = cp;
+}
+
+// the two pixels of ring r bracketing phi, weights w (1 - f), w f
+template <typename S>
+__device__ __forceinline__ void interp_ring(const Ring& r, const S& phi, const S& w, InterpS<S>& o, int k) {
+  const S t = (phi - r.phi0) * ((double)r.npix / (2.0 * kPi));
+  const double j0 = floor(val(t));
+  const S f = t - j0;
+  const int64_t j = imod((int64_t)j0, r.npix);
+  interp_pixel<S>(r, j, w * (1.0 - f), o, k);
+  interp_pixel<S>(r, j + 1 == r.npix ? 0 : j + 1, w * f, o, k + 1);
+}
+
+template <typename S>
+__device__ void interp_weights_s(int nside, const RingS* __restrict__ rings, const S nv[3], InterpS<S>& o) {
+  const S rho = sqrt(nv[0] * nv[0] + nv[1] * nv[1]);
+  const S theta = atan2(rho, nv[2]);
+  S phi = atan2(nv[1], nv[0]);
+  if (val(phi) < 0) phi = phi + 2.0 * kPi;
   const double th = val(theta);
-  int i1 = ring_above(nside, cos(th), 0.0);
+  int i1 = ring_above(nside, val(nv[2]), 0.0);
   const int nr = 4 * nside - 1;
-  while (i1 >= 1 && ring_theta(nside, i1) > th) --i1;
-  while (i1 + 1 <= nr && ring_theta(nside, i1 + 1) <= th) ++i1;
+  while (i1 >= 1 && rings[i1 - 1].th > th) --i1;
+  while (i1 + 1 <= nr && rings[i1].th <= th) ++i1;
   if (i1 == 0 || i1 == nr) {
     const int ir = (i1 == 0) ? 1 : nr;
-    const double tr = ring_theta(nside, ir);
-    const S w = (i1 == 0) ? theta / tr : (kPi - theta) / (kPi - tr);
-    S fa;
-    ring_pair_s(nside, ir, phi, &o.p[0], &o.p[1], &fa);
-    o.w[0] = w * (1.0 - fa);
-    o.w[1] = w * fa;
-    const Ring r = ring_geom(nside, ir);
-    for (int k = 0; k < 4; ++k) {
-      o.p[2 + k] = r.first + k;
-      o.w[2 + k] = (1.0 - w) * 0.25;
-    }
+    const RingS r = rings[ir - 1];
+    const S w = (i1 == 0) ? theta / r.th : (kPi - theta) / (kPi - r.th);
+    // the ring's four pixels in the polar mean, two of them also by longitude
+    interp_ring<S>(r.r, phi, w, o, 0);
+    for (int k = 0; k < 4; ++k) interp_pixel<S>(r.r, k, (1.0 - w) * 0.25, o, 2 + k);
     o.n = 6;
     return;
   }
-  const double ta = ring_theta(nside, i1), tb = ring_theta(nside, i1 + 1);
-  const S w = (theta - ta) / (tb - ta);
-  S fa, fb;
-  ring_pair_s(nside, i1, phi, &o.p[0], &o.p[1], &fa);
-  ring_pair_s(nside, i1 + 1, phi, &o.p[2], &o.p[3], &fb);
-  o.w[0] = (1.0 - w) * (1.0 - fa);
-  o.w[1] = (1.0 - w) * fa;
-  o.w[2] = w * (1.0 - fb);
-  o.w[3] = w * fb;
+  const RingS ra = rings[i1 - 1], rb = rings[i1];
+  const S w = (theta - ra.th) / (rb.th - ra.th);
+  interp_ring<S>(ra.r, phi, 1.0 - w, o, 0);
+  interp_ring<S>(rb.r, phi, w, o, 2);
   o.n = 4;
 }
 
-// tangent basis at a RING pixel centre
-__device__ __forceinline__ void pixel_basis(int nside, int64_t p, double t[3], double q[3]) {
-  int64_t j;
-  const int i = pix2ring(nside, p, &j);
-  const Ring r = ring_geom(nside, i);
-  const double phi = r.phi0 + (2.0 * kPi) * (double)j / (double)r.npix;
-  const double cp = cos(phi), sp = sin(phi);
-  t[0] = r.z * cp;
-  t[1] = r.z * sp;
-  t[2] = -r.s;
-  q[0] = -sp;
-  q[1] = cp;
-  q[2] = 0.0;
-}
-
-// Lens values at unit vector nv from the five RING maps: alpha as a tangent
-// 3-vector and U as a tangent 3x3 tensor, interpolated and projected on the
-// basis at nv (the ray step's lookup).
+// Lens values at nv in its basis (et, ep): the interpolated tensors projected.
 template <typename S>
-__device__ void lens_eval(const clc_derivs& M, int nside, const S nv[3], S out[5]) {
-  const S rho = sqrt(nv[0] * nv[0] + nv[1] * nv[1]);
-  const S th = atan2(rho, nv[2]);
-  S ph = atan2(nv[1], nv[0]);
-  if (val(ph) < 0) ph = ph + 2.0 * kPi;
-  InterpS<S> w;
-  interp_weights_s(nside, th, ph, w);
-  S a3[3], U3[3][3];
+__device__ void lens_eval(const clc_derivs& M, const InterpS<S>& w, const S et[3], const S ep[3], S out[5]) {
+  S a3[3], U[6];   // U: xx, yy, zz, xy, xz, yz
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    a3[a] = Lift<S>::of(0.0);
+  for (int a = 0; a < 3; ++a) a3[a] = Lift<S>::of(0.0);
 #pragma unroll
-    for (int b = 0; b < 3; ++b) U3[a][b] = Lift<S>::of(0.0);
-  }
+  for (int a = 0; a < 6; ++a) U[a] = Lift<S>::of(0.0);
   for (int k = 0; k < w.n; ++k) {
     const int64_t p = w.p[k];
-    double t[3], q[3];
-    pixel_basis(nside, p, t, q);
+    const double *t = w.t[k], *q = w.q[k];
     const double at = M.a_th[p], ap = M.a_ph[p], utt = M.u_tt[p], upp = M.u_pp[p], utp = M.u_tp[p];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      a3[a] = a3[a] + w.w[k] * (at * t[a] + ap * q[a]);
-#pragma unroll
-      for (int b = 0; b < 3; ++b)
-        U3[a][b] = U3[a][b] + w.w[k] * (utt * t[a] * t[b] + upp * q[a] * q[b] + utp * (t[a] * q[b] + q[a] * t[b]));
-    }
+    // U = t (utt t + utp q)^T + q (utp t + upp q)^T
+    const double b0 = utt * t[0] + utp * q[0], b1 = utt * t[1] + utp * q[1], b2 = utt * t[2];
+    const double c0 = utp * t[0] + upp * q[0], c1 = utp * t[1] + upp * q[1], c2 = utp * t[2];
+    a3[0] = a3[0] + w.w[k] * (at * t[0] + ap * q[0]);
+    a3[1] = a3[1] + w.w[k] * (at * t[1] + ap * q[1]);
+    a3[2] = a3[2] + w.w[k] * (at * t[2]);
+    U[0] = U[0] + w.w[k] * (t[0] * b0 + q[0] * c0);
+    U[1] = U[1] + w.w[k] * (t[1] * b1 + q[1] * c1);
+    U[2] = U[2] + w.w[k] * (t[2] * b2);
+    U[3] = U[3] + w.w[k] * (t[0] * b1 + q[0] * c1);
+    U[4] = U[4] + w.w[k] * (t[0] * b2 + q[0] * c2);
+    U[5] = U[5] + w.w[k] * (t[1] * b2 + q[1] * c2);
   }
-  S t[3], q[3];
-  basis_s(nv, t, q);
-  out[0] = dot3s(a3, t);
-  out[1] = dot3s(a3, q);
-  S Ut[3], Uq[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    Ut[a] = U3[a][0] * t[0] + U3[a][1] * t[1] + U3[a][2] * t[2];
-    Uq[a] = U3[a][0] * q[0] + U3[a][1] * q[1] + U3[a][2] * q[2];
-  }
-  out[2] = dot3s(t, Ut);
-  out[3] = dot3s(q, Uq);
-  out[4] = dot3s(t, Uq);
+  out[0] = dot3s(a3, et);
+  out[1] = a3[0] * ep[0] + a3[1] * ep[1];
+  const S Ut[3] = {U[0] * et[0] + U[3] * et[1] + U[4] * et[2], U[3] * et[0] + U[1] * et[1] + U[5] * et[2],
+                   U[4] * et[0] + U[5] * et[1] + U[2] * et[2]};
+  const S Uq[2] = {U[0] * ep[0] + U[3] * ep[1], U[3] * ep[0] + U[1] * ep[1]};
+  out[2] = dot3s(et, Ut);
+  out[3] = ep[0] * Uq[0] + ep[1] * Uq[1];
+  out[4] = ep[0] * Ut[0] + ep[1] * Ut[1];
 }
 
 // Adjoint of the lookup's linear dependence on the maps: the five adjoint
 // maps receive, at each interpolation pixel, w_k P_k^T Lbar.
-__device__ void lens_scatter(const clc_derivs& Mbar, int nside, const double nv[3], const double Lb[5]) {
-  const double rho = ::sqrt(nv[0] * nv[0] + nv[1] * nv[1]);
-  const double th = ::atan2(rho, nv[2]);
-  double ph = ::atan2(nv[1], nv[0]);
-  if (ph < 0) ph += 2.0 * kPi;
-  InterpS<double> w;
-  interp_weights_s(nside, th, ph, w);
-  double t[3], q[3];
-  basis_s(nv, t, q);
+template <typename S>
+__device__ void lens_scatter(const clc_derivs& Mbar, const InterpS<S>& w, const double t[3], const double q[3],
+                             const double Lb[5]) {
   for (int k = 0; k < w.n; ++k) {
     const int64_t p = w.p[k];
-    double tk[3], qk[3];
-    pixel_basis(nside, p, tk, qk);
+    const double *tk = w.t[k], *qk = w.q[k];
     const double a = tk[0] * t[0] + tk[1] * t[1] + tk[2] * t[2];
-    const double b = qk[0] * t[0] + qk[1] * t[1] + qk[2] * t[2];
-    const double c = tk[0] * q[0] + tk[1] * q[1] + tk[2] * q[2];
-    const double e = qk[0] * q[0] + qk[1] * q[1] + qk[2] * q[2];
-    const double ww = w.w[k];
+    const double b = qk[0] * t[0] + qk[1] * t[1];
+    const double c = tk[0] * q[0] + tk[1] * q[1];
+    const double e = qk[0] * q[0] + qk[1] * q[1];
+    const double ww = val(w.w[k]);
     atomicAdd(&Mbar.a_th[p], ww * (a * Lb[0] + c * Lb[1]));
     atomicAdd(&Mbar.a_ph[p], ww * (b * Lb[0] + e * Lb[1]));
     atomicAdd(&Mbar.u_tt[p], ww * (a * a * Lb[2] + c * c * Lb[3] + a * c * Lb[4]));
@@ -667,12 +762,16 @@ __global__ void k_gal_init(const double* __restrict__ z, const double* __restric
 struct LensSrc {
   clc_derivs M;
   int nside;
+  const RingS* rings;
   MGView V;
   const int32_t* bundle;
 };
 
+// lens values at unit vector nv with its basis; iw keeps the interpolation of
+// the pure-SHT lookup
 template <bool kMG, typename S>
-__device__ __forceinline__ void lens_at(const LensSrc& src, int64_t k, const S nv[3], S L[5]) {
+__device__ __forceinline__ void lens_at(const LensSrc& src, int64_t k, const S nv[3], const S et[3], const S ep[3],
+                                        InterpS<S>& iw, S L[5]) {
   if (kMG) {
     const int slot = mg_slot(src.V, src.bundle[k]);
     if (slot >= 0) {
@@ -682,22 +781,27 @@ __device__ __forceinline__ void lens_at(const LensSrc& src, int64_t k, const S n
       for (int c = 0; c < 5; ++c) L[c] = Lift<S>::of(0.0);   // outside a partial sky's domain
     }
   } else {
-    lens_eval<S>(src.M, src.nside, nv, L);
+    interp_weights_s<S>(src.nside, src.rings, nv, iw);
+    lens_eval<S>(src.M, iw, et, ep, L);
   }
 }
 
 template <bool kMG>
-__global__ void k_gal_step(double* st, int64_t n, LensSrc src, StepC sc, const int* __restrict__ bin,
-                           const double* __restrict__ tw, int plane, double* __restrict__ gamma) {
+__global__ void __launch_bounds__(128) k_gal_step(double* st, int64_t n, LensSrc src, StepC sc,
+                                                  const int* __restrict__ bin, const double* __restrict__ tw, int plane,
+                                                  double* __restrict__ gamma) {
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-    double in[14], o[14];
+    double in[14], o[14], L[5];
 #pragma unroll
     for (int c = 0; c < 14; ++c) in[c] = st[c * n + k];
-    const double xn = ::sqrt(in[0] * in[0] + in[1] * in[1] + in[2] * in[2]);
-    const double nv[3] = {in[0] / xn, in[1] / xn, in[2] / xn};
-    double L[5];
-    lens_at<kMG, double>(src, k, nv, L);
-    step_eval<double>(in, in + 3, in + 6, in + 10, L, sc, o);
+    StepFwd f;
+    step_basis(in, f);
+    {
+      InterpS<double> iw;
+      lens_at<kMG, double>(src, k, f.n, f.t, f.q, iw, L);
+    }
+    step_forward(in, in + 3, in + 6, in + 10, L, sc, f);
+    step_out(f, in + 6, o);
 #pragma unroll
     for (int c = 0; c < 14; ++c) st[c * n + k] = o[c];
     if (bin[k] == plane) {
@@ -712,15 +816,15 @@ __global__ void k_gal_step(double* st, int64_t n, LensSrc src, StepC sc, const i
 }
 
 // Reverse of one plane.  adj[14][n] holds the adjoint of the state leaving
-// the plane on entry and of the state entering it on return.
-constexpr int kDualK = 5;
-
+// the plane on entry and of the state entering it on return.  FP64-pipe bound;
+// the whole step in dual numbers of 19 directions (four passes of five) took
+// 4.07 ms for 1e5 rays.
 template <bool kMG>
 __global__ void __launch_bounds__(128) k_gal_step_adjoint(const double* __restrict__ ck, double* adj, int64_t n,
                                                           LensSrc src, clc_derivs Mbar, double* ubar, StepC sc,
                                                           const int* __restrict__ bin, const double* __restrict__ tw,
                                                           int plane, const double* __restrict__ gbar) {
-  typedef Dual<kDualK> D;
+  typedef Dual<2> D;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
     double v[14];
 #pragma unroll
@@ -735,50 +839,46 @@ __global__ void __launch_bounds__(128) k_gal_step_adjoint(const double* __restri
         v[10 + c] += (1.0 - t) * Ab[c];
       }
     }
-    double in0[14];
+    double in[14];
 #pragma unroll
-    for (int c = 0; c < 14; ++c) in0[c] = ck[c * n + k];
-    double ib[14], Lb[5];
-    // directions 0..13: entering state; 14..18: the five lens values
-    for (int d0 = 0; d0 < 19; d0 += kDualK) {
-      D in[14];
+    for (int c = 0; c < 14; ++c) in[c] = ck[c * n + k];
+    StepFwd f;
+    step_basis(in, f);
+    // the lookup with its derivatives along theta-hat and phi-hat at the ray
+    InterpS<D> iw;
+    D nd[3], et[3], ep[3], Ld[5];
 #pragma unroll
-      for (int c = 0; c < 14; ++c) {
-        in[c] = dual_const<kDualK>(in0[c]);
+    for (int c = 0; c < 3; ++c) {
+      nd[c].v = f.n[c];
+      nd[c].d[0] = f.t[c];
+      nd[c].d[1] = f.q[c];
+    }
+    basis_s(nd, et, ep);
+    lens_at<kMG, D>(src, k, nd, et, ep, iw, Ld);
+    double L[5], Lb[5], ib[14], nb[3];
 #pragma unroll
-        for (int j = 0; j < kDualK; ++j) in[c].d[j] = (d0 + j == c) ? 1.0 : 0.0;
-      }
-      const D xn = sqrt(in[0] * in[0] + in[1] * in[1] + in[2] * in[2]);
-      const D nv[3] = {in[0] / xn, in[1] / xn, in[2] / xn};
-      D L[5];
-      lens_at<kMG, D>(src, k, nv, L);
+    for (int c = 0; c < 5; ++c) L[c] = Ld[c].v;
+    step_forward(in, in + 3, in + 6, in + 10, L, sc, f);
+    step_reverse(in, in + 3, in + 6, L, sc, f, v, ib, Lb, nb);
+    double d0 = 0.0, d1 = 0.0;
 #pragma unroll
-      for (int c = 0; c < 5; ++c)
-#pragma unroll
-        for (int j = 0; j < kDualK; ++j)
-          if (d0 + j == 14 + c) L[c].d[j] += 1.0;
-      D o[14];
-      step_eval<D>(in, in + 3, in + 6, in + 10, L, sc, o);
-#pragma unroll
-      for (int j = 0; j < kDualK; ++j) {
-        const int dir = d0 + j;
-        if (dir >= 19) break;
-        double acc = 0.0;
-#pragma unroll
-        for (int c = 0; c < 14; ++c) acc += v[c] * o[c].d[j];
-        if (dir < 14) ib[dir] = acc;
-        else Lb[dir - 14] = acc;
-      }
+    for (int c = 0; c < 5; ++c) {
+      d0 += Lb[c] * Ld[c].d[0];
+      d1 += Lb[c] * Ld[c].d[1];
     }
 #pragma unroll
+    for (int c = 0; c < 3; ++c) nb[c] += d0 * f.t[c] + d1 * f.q[c];
+    // n = x / |x|
+    const double rn = dot3s(f.n, nb), ix = 1.0 / f.xn;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ib[c] += (nb[c] - f.n[c] * rn) * ix;
+#pragma unroll
     for (int c = 0; c < 14; ++c) adj[c * n + k] = ib[c];
-    const double xn = ::sqrt(in0[0] * in0[0] + in0[1] * in0[1] + in0[2] * in0[2]);
-    const double nv[3] = {in0[0] / xn, in0[1] / xn, in0[2] / xn};
     if (kMG) {
       const int slot = src.V.slot ? src.V.slot[src.bundle[k]] : src.bundle[k];
-      if (slot >= 0) patch_scatter(src.V, slot, nv, Lb, ubar);
+      if (slot >= 0) patch_scatter(src.V, slot, f.n, Lb, ubar);
     } else {
-      lens_scatter(Mbar, src.nside, nv, Lb);
+      lens_scatter<D>(Mbar, iw, f.t, f.q, Lb);
     }
   }
 }
@@ -968,12 +1068,17 @@ static int plane_lens(clc_gal_tape* T, int m, LensSrc* src) {
     src->M = clc_derivs{mp, mp + np, mp + 2 * np, mp + 3 * np, mp + 4 * np};
     src->nside = T->nside;
     src->bundle = nullptr;
+    int rc;
+    auto plan = get_fft_plan(ctx, T->nside, &rc);
+    if (rc) return rc;
+    src->rings = (const RingS*)plan->rings.p;
     return clc_poisson_sht(ctx, T->kappa[m], T->nside, T->lmax, T->precision, nullptr, &src->M);
   }
   int rc = clc_poisson_shtmg(ctx, T->kappa[m], T->nside, &T->mg, T->sol, nullptr);
   if (rc != CLC_OK && rc != CLC_ENOTCONVERGED) return rc;
   src->M = clc_derivs{};
   src->nside = 0;
+  src->rings = nullptr;
   src->V = mg_view(T->sol);
   src->bundle = (const int32_t*)T->bundle.p;
   return CLC_OK;

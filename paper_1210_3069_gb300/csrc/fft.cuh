@@ -11,10 +11,10 @@ struct alignas(2 * sizeof(T)) C2 {
   T x, y;
 };
 
-// Geometry of a ring with 1 / sin(theta)
+// Geometry of a ring with 1 / sin(theta) and its colatitude
 struct RingS {
   Ring r;
-  double is;
+  double is, th;
 };
 
 // The phase table of ring class k (1 .. nside - 1: the polar rings of 4 k
