@@ -1069,9 +1069,8 @@ static int plane_lens(clc_gal_tape* T, int m, LensSrc* src) {
     src->nside = T->nside;
     src->bundle = nullptr;
     int rc;
-    auto plan = get_fft_plan(ctx, T->nside, &rc);
+    src->rings = get_ring_table(ctx, T->nside, &rc);
     if (rc) return rc;
-    src->rings = (const RingS*)plan->rings.p;
     return clc_poisson_sht(ctx, T->kappa[m], T->nside, T->lmax, T->precision, nullptr, &src->M);
   }
   int rc = clc_poisson_shtmg(ctx, T->kappa[m], T->nside, &T->mg, T->sol, nullptr);

@@ -50,6 +50,7 @@ struct clc_ctx {
   std::map<std::string, std::vector<std::pair<cudaEvent_t, cudaEvent_t>>> prof_ev;
   std::vector<cudaEvent_t> ev_pool;
   std::map<int, std::shared_ptr<clc::FftPlan>> fft_plans;
+  std::map<int, std::shared_ptr<clc::Buffer>> ring_tables;   // RingS[4 nside - 1] by nside
   std::map<std::tuple<int, int, int>, std::shared_ptr<clc::LegendreTable>> leg_tables;
   std::map<std::pair<int, int>, std::shared_ptr<clc::TcTable>> tc_tables;
   size_t table_budget = 0;  // FP64 Legendre table limit in bytes (0: device memory decides)
@@ -106,6 +107,9 @@ int cuda_check(clc_ctx* ctx, cudaError_t e, const char* what);
 void* scratch(clc_ctx* ctx, int slot, size_t bytes);
 int launch_check(clc_ctx* ctx, const char* what);
 bool valid_nside(int nside);
+struct RingS;
+// Geometry of the 4 nside - 1 rings on the device, kept by the context.
+const RingS* get_ring_table(clc_ctx* ctx, int nside, int* rc);
 int num_sms(clc_ctx* ctx);
 
 // ---------------------------------------------------------------------------
@@ -305,12 +309,12 @@ __device__ __host__ __forceinline__ Ring ring_geom(int nside, int i) {
   return r;
 }
 
-// Ring (1-based) of a RING pixel index
+// Ring (1-based) of a RING pixel index (FP32 estimate, settled in integers)
 __device__ __forceinline__ int pix2ring(int nside, int64_t p, int64_t* j) {
   const int64_t n = nside;
   const int64_t ncap = 2 * n * (n - 1), np = 12 * n * n;
   if (p < ncap) {
-    int64_t i = (int64_t)((1.0 + sqrt(1.0 + 2.0 * (double)p)) * 0.5);
+    int64_t i = (int64_t)((1.f + sqrtf(1.f + 2.f * (float)p)) * 0.5f);
     while (2 * i * (i - 1) > p) --i;
     while (2 * (i + 1) * i <= p) ++i;
     *j = p - 2 * i * (i - 1);
@@ -322,12 +326,18 @@ __device__ __forceinline__ int pix2ring(int nside, int64_t p, int64_t* j) {
     return (int)(q / (4 * n) + n);
   }
   const int64_t q = np - p;
-  int64_t i = (int64_t)((1.0 + sqrt(2.0 * (double)q - 1.0)) * 0.5);
+  int64_t i = (int64_t)((1.f + sqrtf(2.f * (float)q - 1.f)) * 0.5f);
   while (i > 1 && 2 * i * (i - 1) >= q) --i;
   while (2 * i * (i + 1) < q) ++i;
   *j = p - (np - 2 * i * (i + 1));
   return (int)(4 * n - i);
 }
+
+// Geometry of a ring with 1 / sin(theta) and its colatitude
+struct RingS {
+  Ring r;
+  double is, th;
+};
 
 // continuous ring coordinate of z (ring i at z_i gives i)
 __device__ __forceinline__ double ring_coord(int nside, double z) {
@@ -358,18 +368,6 @@ __device__ __forceinline__ int ring_above(int nside, double z, double s) {
   return i;  // ring index with theta_i <= theta (0 = above the first ring)
 }
 
-// Two pixels of ring i bracketing phi and the weight of the second
-__device__ __forceinline__ void ring_pair(int nside, int i, double phi, int64_t* p0, int64_t* p1, double* f) {
-  const Ring r = ring_geom(nside, i);
-  const double t = (phi - r.phi0) * (double)r.npix / (2.0 * kPi);
-  const double j0 = floor(t);
-  *f = t - j0;
-  int64_t j = (int64_t)j0;
-  j = imod(j, r.npix);
-  *p0 = r.first + j;
-  *p1 = r.first + (j + 1 == r.npix ? 0 : j + 1);
-}
-
 // HEALPix ring-bilinear interpolation weights at (theta, phi): up to 8 pixel
 // indices / weights (linear in theta between bracketing rings, linear in
 // phi on each ring; above the first / below the last ring the ring is
@@ -379,39 +377,83 @@ struct Interp8 {
   double w[8];
 };
 
+// Two pixels of ring r bracketing phi and the weight of the second
+__device__ __forceinline__ void ring_pair_of(const Ring& r, double phi, int64_t* p0, int64_t* p1, double* f) {
+  const double t = (phi - r.phi0) * (double)r.npix / (2.0 * kPi);
+  const double j0 = floor(t);
+  *f = t - j0;
+  int64_t j = (int64_t)j0;
+  j = imod(j, r.npix);
+  *p0 = r.first + j;
+  *p1 = r.first + (j + 1 == r.npix ? 0 : j + 1);
+}
+
 __device__ __forceinline__ Interp8 interp_weights(int nside, double theta, double phi) {
   Interp8 o;
   const double z = cos(theta);
   int i1 = ring_above(nside, z, 0.0);
   const int nr = 4 * nside - 1;
   // ring_above is exact up to rounding; settle the bracket on ring colatitudes
-  while (i1 >= 1 && ring_theta(nside, i1) > theta) --i1;
-  while (i1 + 1 <= nr && ring_theta(nside, i1 + 1) <= theta) ++i1;
+  // (each ring's geometry and colatitude is formed once)
+  Ring ra{}, rb{};
+  double ta = -1.0, tb = 4.0;   // ring i1 (0: above the first), ring i1 + 1
+  if (i1 >= 1) {
+    ra = ring_geom(nside, i1);
+    ta = atan2(ra.s, ra.z);
+  }
+  if (i1 + 1 <= nr) {
+    rb = ring_geom(nside, i1 + 1);
+    tb = atan2(rb.s, rb.z);
+  }
+  while (i1 >= 1 && ta > theta) {
+    --i1;
+    rb = ra;
+    tb = ta;
+    ta = -1.0;
+    if (i1 >= 1) {
+      ra = ring_geom(nside, i1);
+      ta = atan2(ra.s, ra.z);
+    }
+  }
+  while (i1 + 1 <= nr && tb <= theta) {
+    ++i1;
+    ra = rb;
+    ta = tb;
+    tb = 4.0;
+    if (i1 + 1 <= nr) {
+      rb = ring_geom(nside, i1 + 1);
+      tb = atan2(rb.s, rb.z);
+    }
+  }
+#pragma unroll
   for (int k = 0; k < 8; ++k) { o.p[k] = 0; o.w[k] = 0.0; }
   if (i1 == 0 || i1 == nr) {
-    const int ir = (i1 == 0) ? 1 : nr;
-    const double tr = ring_theta(nside, ir);
+    const Ring r = i1 == 0 ? rb : ra;
+    const double tr = i1 == 0 ? tb : ta;
     const double w = (i1 == 0) ? theta / tr : (kPi - theta) / (kPi - tr);
     int64_t a0, a1;
     double fa;
-    ring_pair(nside, ir, phi, &a0, &a1, &fa);
+    ring_pair_of(r, phi, &a0, &a1, &fa);
     o.p[0] = a0; o.w[0] = w * (1.0 - fa);
     o.p[1] = a1; o.w[1] = w * fa;
-    const Ring r = ring_geom(nside, ir);
+#pragma unroll
     for (int k = 0; k < 4; ++k) { o.p[4 + k] = r.first + k; o.w[4 + k] = (1.0 - w) * 0.25; }
     return o;
   }
-  const double ta = ring_theta(nside, i1), tb = ring_theta(nside, i1 + 1);
   const double w = (theta - ta) / (tb - ta);
   int64_t a0, a1, b0, b1;
   double fa, fb;
-  ring_pair(nside, i1, phi, &a0, &a1, &fa);
-  ring_pair(nside, i1 + 1, phi, &b0, &b1, &fb);
+  ring_pair_of(ra, phi, &a0, &a1, &fa);
+  ring_pair_of(rb, phi, &b0, &b1, &fb);
   o.p[0] = a0; o.w[0] = (1.0 - w) * (1.0 - fa);
   o.p[1] = a1; o.w[1] = (1.0 - w) * fa;
   o.p[2] = b0; o.w[2] = w * (1.0 - fb);
   o.p[3] = b1; o.w[3] = w * fb;
   return o;
+}
+
+__device__ __forceinline__ void ring_pair(int nside, int i, double phi, int64_t* p0, int64_t* p1, double* f) {
+  ring_pair_of(ring_geom(nside, i), phi, p0, p1, f);
 }
 
 // Same interpolation with the ring colatitudes taken from a table
@@ -450,6 +492,60 @@ __device__ __forceinline__ Interp8 interp_weights_tab(int nside, const double* _
   o.p[2] = b0; o.w[2] = w * (1.0 - fb);
   o.p[3] = b1; o.w[3] = w * fb;
   return o;
+}
+
+// The same interpolation from the context's ring table (get_ring_table): the
+// bracket from an FP32 estimate settled on the table's colatitudes, up to six
+// pixels with their ring and position on it.
+struct RingInterp {
+  int64_t p[6];
+  double w[6];
+  int ring[6], pos[6];
+  int n;
+};
+
+__device__ __forceinline__ void ring_interp_pair(const Ring& r, int i, double phi, double w, RingInterp& o, int k) {
+  const double t = (phi - r.phi0) * (double)r.npix / (2.0 * kPi);
+  const double j0 = floor(t), f = t - j0;
+  const int j = (int)imod((int64_t)j0, r.npix), j1 = j + 1 == r.npix ? 0 : j + 1;
+  o.p[k] = r.first + j;
+  o.w[k] = w * (1.0 - f);
+  o.ring[k] = o.ring[k + 1] = i;
+  o.pos[k] = j;
+  o.p[k + 1] = r.first + j1;
+  o.w[k + 1] = w * f;
+  o.pos[k + 1] = j1;
+}
+
+__device__ __forceinline__ void ring_interp(int nside, const RingS* __restrict__ rings, double theta, double phi,
+                                            RingInterp& o) {
+  const int nr = 4 * nside - 1;
+  const float th = (float)theta, z = cosf(th), nf = (float)nside;
+  const float x = z > 2.f / 3.f ? nf * 2.44948974f * sinf(0.5f * th)
+                                : z < -2.f / 3.f ? 4.f * nf - nf * 2.44948974f * cosf(0.5f * th) : nf * (2.f - 1.5f * z);
+  int i1 = min(max((int)floorf(x), 0), nr);
+  while (i1 >= 1 && rings[i1 - 1].th > theta) --i1;
+  while (i1 + 1 <= nr && rings[i1].th <= theta) ++i1;
+  if (i1 == 0 || i1 == nr) {
+    const int ir = (i1 == 0) ? 1 : nr;
+    const RingS r = rings[ir - 1];
+    const double w = (i1 == 0) ? theta / r.th : (kPi - theta) / (kPi - r.th);
+    ring_interp_pair(r.r, ir, phi, w, o, 0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      o.p[2 + k] = r.r.first + k;
+      o.w[2 + k] = (1.0 - w) * 0.25;
+      o.ring[2 + k] = ir;
+      o.pos[2 + k] = k;
+    }
+    o.n = 6;
+    return;
+  }
+  const RingS ra = rings[i1 - 1], rb = rings[i1];
+  const double w = (theta - ra.th) / (rb.th - ra.th);
+  ring_interp_pair(ra.r, i1, phi, 1.0 - w, o, 0);
+  ring_interp_pair(rb.r, i1 + 1, phi, w, o, 2);
+  o.n = 4;
 }
 
 __device__ __forceinline__ double interp_map_tab(const double* __restrict__ map, int nside,

@@ -115,6 +115,7 @@ extern "C" int clc_destroy(clc_ctx* ctx) {
   ctx->tc_batches.clear();
   ctx->tc_tables.clear();
   ctx->fft_plans.clear();
+  ctx->ring_tables.clear();
   ctx->leg_tables.clear();
   if (ctx->d_err) cudaFree(ctx->d_err);
   delete ctx;
@@ -125,6 +126,7 @@ extern "C" int clc_release_caches(clc_ctx* ctx) {
   if (!ctx) return CLC_EINVAL;
   cudaStreamSynchronize(ctx->stream);
   ctx->fft_plans.clear();
+  ctx->ring_tables.clear();
   ctx->tc_batches.clear();
   ctx->leg_tables.clear();
   ctx->tc_tables.clear();

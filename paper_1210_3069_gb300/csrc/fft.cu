@@ -91,7 +91,7 @@ PlanDevT<double> plan_dev<double>(const FftPlan& p) {
   d.cls = (const int4*)p.cls.p;
   d.chirp = (const C2<double>*)p.chirp.p;
   d.filter = (const C2<double>*)p.filter.p;
-  d.rings = (const RingS*)p.rings.p;
+  d.rings = (const RingS*)p.rings->p;
   d.phase = (const C2<double>*)p.phase.p;
   d.logmmax = 0;
   while ((1 << d.logmmax) < p.mmax_fft) ++d.logmmax;
@@ -105,7 +105,7 @@ PlanDevT<float> plan_dev<float>(const FftPlan& p) {
   d.cls = (const int4*)p.cls.p;
   d.chirp = (const C2<float>*)p.chirp32.p;
   d.filter = (const C2<float>*)p.filter32.p;
-  d.rings = (const RingS*)p.rings.p;
+  d.rings = (const RingS*)p.rings->p;
   d.phase = (const C2<double>*)p.phase.p;
   d.logmmax = 0;
   while ((1 << d.logmmax) < p.mmax_fft) ++d.logmmax;
@@ -118,6 +118,24 @@ static int next_pow2(int v) {
   return p;
 }
 
+const RingS* get_ring_table(clc_ctx* ctx, int nside, int* rc) {
+  *rc = CLC_OK;
+  auto it = ctx->ring_tables.find(nside);
+  if (it != ctx->ring_tables.end()) return (const RingS*)it->second->p;
+  auto b = std::make_shared<Buffer>();
+  b->bytes = sizeof(RingS) * (4 * (size_t)nside - 1);
+  if (cudaMalloc(&b->p, b->bytes) != cudaSuccess) {
+    cudaGetLastError();
+    b->p = nullptr;
+    *rc = set_err(ctx, CLC_ENOMEM, "ring table allocation failed");
+    return nullptr;
+  }
+  CLC_LAUNCH(ctx, "k_ring_table", k_ring_table, (4 * nside + 126) / 128, 128, 0, nside, (RingS*)b->p);
+  if ((*rc = launch_check(ctx, "k_ring_table"))) return nullptr;
+  ctx->ring_tables[nside] = b;
+  return (const RingS*)b->p;
+}
+
 std::shared_ptr<FftPlan> get_fft_plan(clc_ctx* ctx, int nside, int* rc) {
   auto it = ctx->fft_plans.find(nside);
   if (it != ctx->fft_plans.end()) {
@@ -126,6 +144,8 @@ std::shared_ptr<FftPlan> get_fft_plan(clc_ctx* ctx, int nside, int* rc) {
   }
   auto p = std::make_shared<FftPlan>();
   p->nside = nside;
+  if (!get_ring_table(ctx, nside, rc)) return nullptr;
+  p->rings = ctx->ring_tables[nside];
   std::vector<int4> cls(std::max(nside, 1), make_int4(0, 0, 0, 0));
   int mmax = std::max(2 * nside, 1);
   size_t chirp_n = 0, filt_n = 0;
@@ -155,7 +175,7 @@ std::shared_ptr<FftPlan> get_fft_plan(clc_ctx* ctx, int nside, int* rc) {
   if (!alloc(p->twiddle, sizeof(double2) * std::max(mmax / 2, 1)) || !alloc(p->cls, sizeof(int4) * cls.size()) ||
       !alloc(p->chirp, sizeof(double2) * chirp_n) || !alloc(p->filter, sizeof(double2) * filt_n) ||
       !alloc(p->twiddle32, sizeof(float2) * std::max(mmax / 2, 1)) || !alloc(p->chirp32, sizeof(float2) * chirp_n) ||
-      !alloc(p->filter32, sizeof(float2) * filt_n) || !alloc(p->rings, sizeof(RingS) * (4 * (size_t)nside - 1)) ||
+      !alloc(p->filter32, sizeof(float2) * filt_n) ||
       !alloc(p->phase, sizeof(double2) * phase_offset(nside + 1))) {
     *rc = set_err(ctx, CLC_ENOMEM, "FFT plan allocation failed");
     return nullptr;
@@ -164,7 +184,6 @@ std::shared_ptr<FftPlan> get_fft_plan(clc_ctx* ctx, int nside, int* rc) {
                                         ctx->stream), "plan upload");
   if (*rc) return nullptr;
   CLC_LAUNCH(ctx, "k_twiddle", k_twiddle, 64, 256, 0, (double2*)p->twiddle.p, mmax);
-  CLC_LAUNCH(ctx, "k_ring_table", k_ring_table, (4 * nside + 126) / 128, 128, 0, nside, (RingS*)p->rings.p);
   CLC_LAUNCH(ctx, "k_phase_table", k_phase_table, nside, 256, 0, (C2<double>*)p->phase.p);
   PlanDevT<double> d = plan_dev<double>(*p);
   if (nside > 1 && chirp_n > 0) {

@@ -11,12 +11,6 @@ struct alignas(2 * sizeof(T)) C2 {
   T x, y;
 };
 
-// Geometry of a ring with 1 / sin(theta) and its colatitude
-struct RingS {
-  Ring r;
-  double is, th;
-};
-
 // The phase table of ring class k (1 .. nside - 1: the polar rings of 4 k
 // pixels; nside: the equatorial rings) holds e^{i pi b / n}, b <= n / 4 = k, at
 // phase_offset(k) + b.
@@ -30,7 +24,7 @@ struct FftPlan {
   Buffer chirp;            // double2: e^{i pi j^2 / N} per Bluestein class
   Buffer filter;           // double2: FFT_M of the Bluestein filter per class
   Buffer twiddle32, chirp32, filter32;   // the same tables rounded to FP32
-  Buffer rings;            // RingS[4 nside - 1]
+  std::shared_ptr<Buffer> rings;   // the ring table (get_ring_table)
   Buffer phase;            // double2: phase_offset(nside + 1) phases
   size_t chirp_n = 0, filt_n = 0;
 };
