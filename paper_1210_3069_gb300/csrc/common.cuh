@@ -333,11 +333,20 @@ __device__ __forceinline__ int pix2ring(int nside, int64_t p, int64_t* j) {
   return (int)(4 * n - i);
 }
 
-// Geometry of a ring with 1 / sin(theta) and its colatitude
+// Geometry of a ring with 1 / sin(theta), its colatitude and pi / npix
 struct RingS {
   Ring r;
-  double is, th;
+  double is, th, half;
 };
+
+// Continuous ring coordinate of colatitude th in FP32 (ring i at its own
+// colatitude; rounding below 0.01 up to nside 8192)
+__device__ __forceinline__ float ring_coord32(int nside, float th) {
+  const float z = cosf(th), n = (float)nside;
+  if (z > 2.f / 3.f) return n * 2.44948974f * sinf(0.5f * th);            // sqrt(3 (1 - z))
+  if (z < -2.f / 3.f) return 4.f * n - n * 2.44948974f * cosf(0.5f * th);
+  return n * (2.f - 1.5f * z);
+}
 
 // continuous ring coordinate of z (ring i at z_i gives i)
 __device__ __forceinline__ double ring_coord(int nside, double z) {
@@ -520,10 +529,7 @@ __device__ __forceinline__ void ring_interp_pair(const Ring& r, int i, double ph
 __device__ __forceinline__ void ring_interp(int nside, const RingS* __restrict__ rings, double theta, double phi,
                                             RingInterp& o) {
   const int nr = 4 * nside - 1;
-  const float th = (float)theta, z = cosf(th), nf = (float)nside;
-  const float x = z > 2.f / 3.f ? nf * 2.44948974f * sinf(0.5f * th)
-                                : z < -2.f / 3.f ? 4.f * nf - nf * 2.44948974f * cosf(0.5f * th) : nf * (2.f - 1.5f * z);
-  int i1 = min(max((int)floorf(x), 0), nr);
+  int i1 = min(max((int)floorf(ring_coord32(nside, (float)theta)), 0), nr);
   while (i1 >= 1 && rings[i1 - 1].th > theta) --i1;
   while (i1 + 1 <= nr && rings[i1].th <= theta) ++i1;
   if (i1 == 0 || i1 == nr) {

@@ -52,6 +52,7 @@ __global__ void k_ring_table(int nside, RingS* __restrict__ rings) {
   o.r = ring_geom(nside, r + 1);
   o.is = 1.0 / o.r.s;
   o.th = atan2(o.r.s, o.r.z);
+  o.half = kPi / (double)o.r.npix;
   rings[r] = o;
 }
 

@@ -227,14 +227,6 @@ __device__ __forceinline__ void ring_zs32(int nside, int r, float* z, float* s) 
   }
 }
 
-// continuous ring coordinate of colatitude th (ring i at its own colatitude)
-__device__ __forceinline__ float ring_coord32(int nside, float th) {
-  const float z = cosf(th), n = (float)nside;
-  if (z > 2.f / 3.f) return n * 2.44948974f * sinf(0.5f * th);            // sqrt(3 (1 - z))
-  if (z < -2.f / 3.f) return 4.f * n - n * 2.44948974f * cosf(0.5f * th);
-  return n * (2.f - 1.5f * z);
-}
-
 // unit vector of the centre of pixel p
 __device__ __forceinline__ void centre_vec(int nside, const RingS* __restrict__ rings, int64_t p, double c[3]) {
   int64_t k;
