@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kRingThreads) k_tc_ring_analysis(TcBatchDev b)
   }
 }
 
-__global__ void __launch_bounds__(kRingThreads) k_tc_ring_synthesis(TcBatchDev b, int buf_len) {
+__global__ void __launch_bounds__(kRingThreads, 2) k_tc_ring_synthesis(TcBatchDev b, int buf_len) {
   extern __shared__ __align__(16) unsigned char smem_rs[];
   C2<float>* s = reinterpret_cast<C2<float>*>(smem_rs);
   const int nf = b.mode ? 6 : 1;
@@ -264,73 +264,120 @@ __global__ void __launch_bounds__(kRingThreads) k_tc_ring_synthesis(TcBatchDev b
 // 1/sin^2(theta)-sized parts, so the synthesis takes them from these sums
 // instead of the tensor-core ones (the FP32 rounding of the latter would be
 // amplified by up to Nside^2).  Only the ncap rings next to each pole
-// (sin theta < 0.29) need them.  One thread per (plane, northern cap ring,
-// which also gives its southern mirror); the unscaled recurrence is safe for
-// m <= 1.
+// (sin theta < 0.29) need them.
+//
+// lambda of the two orders on those rings is kept with the batch (it depends on
+// neither plane nor map), so the sums have no recurrence and split over l: a
+// block takes one (plane, order) on 32 northern rings (and their mirrors by the
+// parity of l + m), its eight warps every eighth l, the l-dependent factors
+// staged once.  One thread per (plane, ring) running the recurrence through
+// every l took 1.33 ms of the 2.25 ms of a batch of 12 small planes (now 0.04)
+// and 2.67 of the 12.4 ms of 21 planes at nside 512 (now 0.12).
 
-__global__ void k_tc_low_orders(TcBatchDev b) {
-  for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < b.n_low;
-       it += (long long)gridDim.x * blockDim.x) {
+// the unscaled recurrence is safe for m <= 1
+__global__ void k_tc_lam01(int nside, int L, int ncap, const double* __restrict__ co01, double* __restrict__ lam01) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, ld = tc_cap_pad(ncap), m = blockIdx.y;
+  if (t >= ld) return;
+  const Ring g = ring_geom(nside, min(t + 1, ncap));
+  const double* co = co01 + (size_t)m * (L + 3) * 4;
+  double* out = lam01 + (size_t)m * (L + 2) * ld + t;
+  double p2 = m == 0 ? 0.28209479177387814347 : -0.34549414947133547927 * g.s, p1 = 0.0;   // lambda_mm
+  for (int l = 0; l <= L + 1; ++l) {
+    double lam = 0.0;
+    if (l == m) {
+      lam = p2;
+    } else if (l == m + 1) {
+      lam = p1 = sqrt(2.0 * m + 3.0) * g.z * p2;
+    } else if (l > m) {
+      lam = co[4 * l] * (g.z * p1 - co[4 * l + 1] * p2);
+      p2 = p1;
+      p1 = lam;
+    }
+    out[(size_t)l * ld] = lam;
+  }
+}
+
+int tc_build_lam01(clc_ctx* ctx, const TcClass& C, double* lam01) {
+  CLC_LAUNCH(ctx, "k_tc_lam01", k_tc_lam01, dim3((tc_cap_pad(C.ncap) + 63) / 64, 2), 64, 0, C.nside, C.lmax, C.ncap,
+             C.co01, lam01);
+  return launch_check(ctx, "k_tc_lam01");
+}
+
+constexpr int kLowChunk = 512;   // degrees staged at a time
+constexpr int kLowWarps = 8;
+
+__global__ void __launch_bounds__(32 * kLowWarps) k_tc_low_orders(TcBatchDev b) {
+  __shared__ double cf[kLowChunk][6];   // psi, b, kappa_bl (re, im) of a degree
+  __shared__ double red[kLowWarps][12][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (long long it = blockIdx.x; it < b.n_low; it += gridDim.x) {
     const TcClass& C = b.cls[find_class(b, it, &TcClass::low0)];
-    const long long loc = it - C.low0;
-    const int ns = C.nside, L = C.lmax;
-    const int pl = (int)(loc / C.ncap), i = (int)(loc % C.ncap) + 1;
-    const Ring g = ring_geom(ns, i);
-    const double z = g.z;
-    const bool has_s = i != 2 * ns;
+    const int ld = tc_cap_pad(C.ncap), nc = ld / 32, L = C.lmax, ns = C.nside;
+    const int loc = (int)(it - C.low0), ch = loc % nc, m = (loc / nc) & 1, pl = loc / (2 * nc);
     const float2* a = C.alm + pl * C.astride;
-    double2* out = C.G01 + (size_t)pl * C.nq * 2 * C.ldf;
-    for (int m = 0; m <= 1; ++m) {
-      const double* co = C.co01 + (size_t)m * (L + 3) * 4;
-      auto kap = [&](int l) -> double2 {
-        if (l < m || l > L || l < 1) return make_double2(0.0, 0.0);
-        const float2 v = a[alm_idx(L, l, m)];
-        return make_double2((double)v.x, m ? (double)v.y : 0.0);
-      };
-      auto psi = [&](int l) -> double2 {
-        const double2 k = kap(l);
-        const double d = (l >= 1 && l <= L) ? co[4 * l + 3] : 0.0;
-        return make_double2(k.x * d, k.y * d);
-      };
-      double2 n0 = make_double2(0, 0), n1 = n0, n2 = n0, s0 = n0, s1 = n0, s2 = n0;
-      double p2 = m == 0 ? 0.28209479177387814347 : -0.34549414947133547927 * g.s;   // lambda_mm
-      double p1 = 0.0;
-      double2 pm1 = psi(m - 1), p0 = psi(m), pp1 = psi(m + 1);
-      for (int l = m; l <= L + 1; ++l) {
-        double lam;
-        if (l == m) {
-          lam = p2;
-        } else if (l == m + 1) {
-          p1 = sqrt(2.0 * m + 3.0) * z * p2;
-          lam = p1;
-        } else {
-          lam = co[4 * l] * (z * p1 - co[4 * l + 1] * p2);
-          p2 = p1;
-          p1 = lam;
-        }
+    const double* co = C.co01 + (size_t)m * (L + 3) * 4;
+    const double* lam = C.lam01 + (size_t)m * (L + 2) * ld + ch * 32 + lane;
+    auto kap = [&](int l) -> double2 {
+      if (l < m || l > L || l < 1) return make_double2(0.0, 0.0);
+      const float2 v = a[alm_idx(L, l, m)];
+      return make_double2((double)v.x, m ? (double)v.y : 0.0);
+    };
+    auto psi = [&](int l) -> double2 {
+      const double2 k = kap(l);
+      const double d = (l >= 1 && l <= L) ? co[4 * l + 3] : 0.0;
+      return make_double2(k.x * d, k.y * d);
+    };
+    double acc[2][6];   // parity of l + m
+#pragma unroll
+    for (int i = 0; i < 6; ++i) acc[0][i] = acc[1][i] = 0.0;
+    for (int l0 = m; l0 <= L + 1; l0 += kLowChunk) {
+      const int n = min(kLowChunk, L + 2 - l0);
+      __syncthreads();
+      for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        const int l = l0 + t;
+        const double2 p0 = psi(l), pm = psi(l - 1), pp = psi(l + 1), kb = kap(l);
         const double c1 = (l - 1.0) * co[4 * l + 2], c2 = (l + 2.0) * co[4 * (l + 1) + 2];
-        const double2 bl = make_double2(c1 * pm1.x - c2 * pp1.x, c1 * pm1.y - c2 * pp1.y);
-        const double2 kb = (l >= 1 && l <= L) ? kap(l) : make_double2(0.0, 0.0);
-        const double sg = ((l + m) & 1) ? -1.0 : 1.0;
-        n0.x += p0.x * lam; n0.y += p0.y * lam;
-        n1.x += bl.x * lam; n1.y += bl.y * lam;
-        n2.x += kb.x * lam; n2.y += kb.y * lam;
-        s0.x += sg * p0.x * lam; s0.y += sg * p0.y * lam;
-        s1.x += sg * bl.x * lam; s1.y += sg * bl.y * lam;
-        s2.x += sg * kb.x * lam; s2.y += sg * kb.y * lam;
-        pm1 = p0;
-        p0 = pp1;
-        pp1 = psi(l + 2);
+        cf[t][0] = p0.x;
+        cf[t][1] = p0.y;
+        cf[t][2] = c1 * pm.x - c2 * pp.x;
+        cf[t][3] = c1 * pm.y - c2 * pp.y;
+        cf[t][4] = kb.x;
+        cf[t][5] = kb.y;
       }
-      const size_t q = 2 * (size_t)C.ldf, mo = (size_t)m * C.ldf;
-      out[mo + i - 1] = n0;
-      out[q + mo + i - 1] = n1;
-      out[2 * q + mo + i - 1] = n2;
-      if (has_s) {
-        const size_t j = 4 * ns - i - 1;
-        out[mo + j] = s0;
-        out[q + mo + j] = s1;
-        out[2 * q + mo + j] = s2;
+      __syncthreads();
+      // l + m = 2 m + (l - m): even and odd terms alternate from l0 = m + multiples of kLowChunk on
+      for (int t = 2 * warp; t < n; t += 2 * kLowWarps) {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          if (t + p >= n) break;
+          const double x = lam[(size_t)(l0 + t + p) * ld];
+#pragma unroll
+          for (int i = 0; i < 6; ++i) acc[p][i] = fma(cf[t + p][i], x, acc[p][i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      red[warp][i][lane] = acc[0][i];
+      red[warp][6 + i][lane] = acc[1][i];
+    }
+    __syncthreads();
+    double2* out = C.G01 + (size_t)pl * C.nq * 2 * C.ldf;
+    const size_t qs = 2 * (size_t)C.ldf, mo = (size_t)m * C.ldf;
+    if (warp < 3) {   // quantity q = warp
+      double e[2], o[2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        e[c] = o[c] = 0.0;
+        for (int w = 0; w < kLowWarps; ++w) {
+          e[c] += red[w][2 * warp + c][lane];
+          o[c] += red[w][6 + 2 * warp + c][lane];
+        }
+      }
+      const int i = ch * 32 + lane + 1;
+      if (i <= C.ncap) {
+        out[warp * qs + mo + i - 1] = make_double2(e[0] + o[0], e[1] + o[1]);
+        if (i != 2 * ns) out[warp * qs + mo + 4 * ns - i - 1] = make_double2(e[0] - o[0], e[1] - o[1]);
       }
     }
   }
@@ -811,11 +858,18 @@ static int grid_of(clc_ctx* ctx, K kern, int threads, int smem, long long items,
   return (int)std::max<long long>(g, 1);
 }
 
+// The ring kernels get fft_ctas blocks per SM, more than stay resident: rings
+// differ in length, and the blocks that start later even that out (synthesis of
+// 21 planes at nside 512: 5.60 ms with 8 per SM, 5.74 with 32, 5.19 with 128).
+static int ring_grid(clc_ctx* ctx, long long items, int per_sm) {
+  return (int)std::max<long long>(1, std::min<long long>(items, (long long)num_sms(ctx) * per_sm));
+}
+
 int tc_run_stage(clc_ctx* ctx, const TcBatchDev& b, const TcItems& it, const TcLaunch& L, int stage) {
   switch (stage) {
     case 0: {
       cudaFuncSetAttribute(k_tc_ring_analysis, cudaFuncAttributeMaxDynamicSharedMemorySize, it.fft_smem);
-      const int g = grid_of(ctx, k_tc_ring_analysis, it.fft_threads, it.fft_smem, b.n_ring, L.fft_ctas);
+      const int g = ring_grid(ctx, b.n_ring, L.fft_ctas);
       CLC_LAUNCH(ctx, "k_tc_ring_analysis", k_tc_ring_analysis, g, it.fft_threads, it.fft_smem, b);
       return launch_check(ctx, "k_tc_ring_analysis");
     }
@@ -836,8 +890,8 @@ int tc_run_stage(clc_ctx* ctx, const TcBatchDev& b, const TcItems& it, const TcL
     }
     case 3: {
       if (b.mode && b.n_low > 0) {
-        const int g = (int)std::min<long long>((b.n_low + 127) / 128, (long long)num_sms(ctx) * 16);
-        CLC_LAUNCH(ctx, "k_tc_low_orders", k_tc_low_orders, g, 128, 0, b);
+        const int g = (int)std::min<long long>(b.n_low, (long long)num_sms(ctx) * 4);
+        CLC_LAUNCH(ctx, "k_tc_low_orders", k_tc_low_orders, g, 32 * kLowWarps, 0, b);
         const int rc = launch_check(ctx, "k_tc_low_orders");
         if (rc) return rc;
       }
@@ -858,7 +912,7 @@ int tc_run_stage(clc_ctx* ctx, const TcBatchDev& b, const TcItems& it, const TcL
     }
     default: {
       cudaFuncSetAttribute(k_tc_ring_synthesis, cudaFuncAttributeMaxDynamicSharedMemorySize, it.fft_smem);
-      const int g = grid_of(ctx, k_tc_ring_synthesis, it.fft_threads, it.fft_smem, b.n_ring * (b.mode ? 6 : 1), L.fft_ctas);
+      const int g = ring_grid(ctx, b.n_ring * (b.mode ? 6 : 1), L.fft_ctas);
       CLC_LAUNCH(ctx, "k_tc_ring_synthesis", k_tc_ring_synthesis, g, it.fft_threads, it.fft_smem, b,
                  it.fft_smem / (int)sizeof(float2));
       return launch_check(ctx, "k_tc_ring_synthesis");

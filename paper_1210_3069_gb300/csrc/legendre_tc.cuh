@@ -60,6 +60,7 @@ struct TcClass {
   double2* G01;                   // [P][nq][m = 0, 1][ring] FP64 Legendre sums of the two lowest orders
   const double* co01;             // [m = 0, 1][l = 0 .. lmax + 2][4] recurrence a_lm, b_lm, eps_lm, -1/(l(l+1))
   int ncap;                       // rings from each pole that use the FP64 sums
+  const double* lam01;            // [m = 0, 1][l = 0 .. lmax + 1][round32(ncap)] lambda_lm of those rings
   long long ring0, pa0, ps0, low0;  // first flat item of the class: ring FFTs, packs, low-order sums
 };
 
@@ -76,7 +77,7 @@ struct TcBatchDev {
 struct TcLaunch {
   int an_stages = 2, an_ctas = 2;     // analysis pipeline depth, resident CTAs per SM
   int sy_stages = 2, sy_ctas = 2;     // synthesis
-  int fft_ctas = 8;                   // ring FFT kernels, resident CTAs per SM
+  int fft_ctas = 128;                 // ring FFT kernels, CTAs per SM
 };
 
 // Device-side work lists of a batch (built once per batch layout).
@@ -87,6 +88,9 @@ struct TcItems {
   int fft_smem = 0, fft_threads = 64, pack_s_smem = 0;
 };
 
+__host__ __device__ constexpr int tc_cap_pad(int ncap) { return (ncap + 31) / 32 * 32; }
+// Fill the class's lam01 (on the context's stream).
+int tc_build_lam01(clc_ctx* ctx, const TcClass& C, double* lam01);
 int tc_build_items(clc_ctx* ctx, const TcBatchDev& b, const std::vector<std::shared_ptr<TcTable>>& tabs,
                    TcItems* it);
 // The six launches of one mixed-precision Poisson pass over every plane of the batch.

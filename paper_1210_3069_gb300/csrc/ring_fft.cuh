@@ -409,7 +409,7 @@ __device__ __forceinline__ C2<S> spec_combine(int mode, int f, int m, C2<S> g0, 
 template <typename T>
 struct RingFac {
   T is, is2, c;
-  double isd, is2d, cd;
+  double isd, cd;
 };
 
 template <typename T>
@@ -419,7 +419,7 @@ __device__ __forceinline__ C2<T> spec_of(const SynthArgsT<T>& a, int mode, int f
     const C2<double>* P = a.P01 + (size_t)m * a.p01m + ring0;
     const C2<double> z = cx<double>(0.0, 0.0);
     const C2<double> h = spec_combine<double>(mode, f, m, P[0], mode ? P[a.p01q] : z, mode ? P[2 * a.p01q] : z, g.isd,
-                                              g.is2d, g.cd);
+                                              g.isd * g.isd, g.cd);
     return cx<T>((T)h.x, (T)h.y);
   }
   const size_t idx = a.quad ? (size_t)(m >> 2) * a.sm + (size_t)ring0 * 4 + (m & 3)
@@ -449,11 +449,15 @@ __device__ void ring_synthesis_ring(const SynthArgsT<T>& a, int nside, int lmax,
   const bool shifted = r.phi0 != 0.0;
   RingFac<T> gf;
   gf.isd = rs.is;
-  gf.is2d = gf.isd * gf.isd;
   gf.cd = r.z;
-  gf.is = (T)gf.isd;
+  if constexpr (sizeof(T) == 4) {   // rounded on the integer pipe
+    gf.is = d2f_rn(rs.is);
+    gf.c = d2f_rn(r.z);
+  } else {
+    gf.is = rs.is;
+    gf.c = r.z;
+  }
   gf.is2 = gf.is * gf.is;
-  gf.c = (T)r.z;
   Phase<T> ph;
   phase_init(ph, P, nside, i, n);
   // X_k = c_k [sum_{q>=0} (-1)^q g_{k+qn} + sum_{q>=1} (-1)^q conj(g_{qn-k})]

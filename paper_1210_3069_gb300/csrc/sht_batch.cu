@@ -87,7 +87,7 @@ static int tc_batch_build(clc_ctx* ctx, int nplanes, const int* nside, const int
   B->slot.assign(nplanes, 0);
   // sizes of every class buffer
   struct Sz {
-    size_t F, V, Ve, A, S, Se, So, G, G01, Co;
+    size_t F, V, Ve, A, S, Se, So, G, G01, Co, La;
   };
   std::vector<std::vector<double>> co01(key.size());
   std::vector<Sz> sz(d.ncls);
@@ -164,13 +164,14 @@ static int tc_batch_build(clc_ctx* ctx, int nplanes, const int* nside, const int
     z.G = r256(sizeof(float2) * C.gstride * P);
     z.G01 = r256(sizeof(double2) * (size_t)P * nq * 2 * C.ldf);
     z.Co = r256(sizeof(double) * co01[c].size());
-    total += z.F + 2 * z.V + z.Ve + z.A + 2 * z.S + z.Se + z.So + z.G + z.G01 + z.Co;
+    z.La = mode ? r256(sizeof(double) * 2 * (size_t)(L + 2) * tc_cap_pad(C.ncap)) : 0;
+    total += z.F + 2 * z.V + z.Ve + z.A + 2 * z.S + z.Se + z.So + z.G + z.G01 + z.Co + z.La;
     for (int j = 0; j < P; ++j) B->slot[members[c][j]] = plane0 + j;
     plane0 += P;
     ring0 += (long long)P * (4 * ns - 1);
     pa0 += L + 1;
     ps0 += G;
-    low0 += (long long)P * C.ncap;
+    low0 += (long long)P * 2 * (tc_cap_pad(C.ncap) / 32);
   }
   d.n_ring = ring0;
   d.n_pa = pa0;
@@ -222,6 +223,9 @@ static int tc_batch_build(clc_ctx* ctx, int nplanes, const int* nside, const int
                          "batch coefficient upload")))
       return rc;
     w += z.Co;
+    C.lam01 = (const double*)w;
+    if (mode && (rc = tc_build_lam01(ctx, C, (double*)w))) return rc;
+    w += z.La;
   }
   // pointer tables: kappa[n], out[n][6]
   B->ptr_bytes = sizeof(void*) * (size_t)nplanes * 7;
@@ -301,7 +305,7 @@ static int tc_autotune(TcBatch* B) {
     TcLaunch pick = L;
     std::vector<TcLaunch> cand;
     if (stage == 0 || stage == 5) {
-      for (int c : {4, 8, 16}) {
+      for (int c : {8, 32, 128}) {
         TcLaunch x = L;
         x.fft_ctas = c;
         cand.push_back(x);
