@@ -1019,8 +1019,7 @@ static int sht_poisson_adjoint(clc_gal_tape* T, const clc_derivs& Fb, double* kb
   double2* kt = rb + 3 * Q;
   const double* maps[5] = {Fb.a_th, Fb.a_ph, Fb.u_tt, Fb.u_pp, Fb.u_tp};
   // transposed ring synthesis: ring analysis without quadrature weight
-  for (int f = 0; f < 5; ++f)
-    if ((rc = ring_analysis(ctx, *plan, maps[f], L, 1.0, Fh + f * fq, ldf))) return rc;
+  if ((rc = ring_analysis_maps(ctx, *plan, 5, maps, L, 1.0, Fh, fq, ldf))) return rc;
   dim3 g1((4 * ns - 1 + 127) / 128, L + 1);
   CLC_LAUNCH(ctx, "k_spec_adjoint", k_spec_adjoint, g1, 128, 0, ns, L, Fh, fq, ldf, Gb, fq);
   if ((rc = launch_check(ctx, "k_spec_adjoint"))) return rc;

@@ -68,12 +68,17 @@ __global__ void k_round_to_float(const double2* __restrict__ in, size_t n, float
     out[j] = make_float2((float)in[j].x, (float)in[j].y);
 }
 
-// one CTA per ring
+struct RingMaps {
+  const double* map[8];
+};
+
+// one CTA per (ring, map)
 template <typename T>
-__global__ void __launch_bounds__(512) k_ring_analysis(const double* __restrict__ map, int nside, int lmax,
-                                                       double weight, C2<T>* __restrict__ F, int ldf, PlanDevT<T> P) {
+__global__ void __launch_bounds__(512) k_ring_analysis(RingMaps maps, int nside, int lmax, double weight,
+                                                       C2<T>* __restrict__ F, size_t fstride, int ldf, PlanDevT<T> P) {
   extern __shared__ __align__(16) unsigned char smem_fft[];
-  ring_analysis_ring<T>(map, nside, lmax, weight, F, ldf, P, blockIdx.x + 1, reinterpret_cast<C2<T>*>(smem_fft));
+  ring_analysis_ring<T>(maps.map[blockIdx.y], nside, lmax, weight, F + blockIdx.y * fstride, ldf, P, blockIdx.x + 1,
+                        reinterpret_cast<C2<T>*>(smem_fft));
 }
 
 // one CTA per (field, ring)
@@ -208,12 +213,15 @@ std::shared_ptr<FftPlan> get_fft_plan(clc_ctx* ctx, int nside, int* rc) {
 }
 
 template <typename T>
-int ring_analysis_t(clc_ctx* ctx, const FftPlan& plan, const double* map, int lmax, double weight, C2<T>* F,
-                    int ldf) {
+int ring_analysis_t(clc_ctx* ctx, const FftPlan& plan, int n, const double* const* maps, int lmax, double weight,
+                    C2<T>* F, size_t fstride, int ldf) {
   const int nside = plan.nside;
   const int smem = ring_fft_smem<T>(plan);
+  RingMaps a{};
+  for (int k = 0; k < n; ++k) a.map[k] = maps[k];
   cudaFuncSetAttribute(k_ring_analysis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  CLC_LAUNCH(ctx, "k_ring_analysis", (k_ring_analysis<T>), 4 * nside - 1, std::max(128, ring_fft_threads(plan.mmax_fft)), smem, map, nside, lmax, weight, F, ldf,
+  CLC_LAUNCH(ctx, "k_ring_analysis", (k_ring_analysis<T>), dim3(4 * nside - 1, n),
+             std::max(128, ring_fft_threads(plan.mmax_fft)), smem, a, nside, lmax, weight, F, fstride, ldf,
              plan_dev<T>(plan));
   return launch_check(ctx, "k_ring_analysis");
 }
@@ -242,8 +250,8 @@ int ring_synthesis_t(clc_ctx* ctx, const FftPlan& plan, const C2<T>* G, int ld, 
   return launch_check(ctx, "k_ring_synthesis");
 }
 
-template int ring_analysis_t<double>(clc_ctx*, const FftPlan&, const double*, int, double, C2<double>*, int);
-template int ring_analysis_t<float>(clc_ctx*, const FftPlan&, const double*, int, double, C2<float>*, int);
+template int ring_analysis_t<double>(clc_ctx*, const FftPlan&, int, const double* const*, int, double, C2<double>*, size_t, int);
+template int ring_analysis_t<float>(clc_ctx*, const FftPlan&, int, const double* const*, int, double, C2<float>*, size_t, int);
 template int ring_synthesis_t<double>(clc_ctx*, const FftPlan&, const C2<double>*, int, int, int, double* const[6]);
 template int ring_synthesis_t<float>(clc_ctx*, const FftPlan&, const C2<float>*, int, int, int, double* const[6]);
 

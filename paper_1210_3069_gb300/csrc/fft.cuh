@@ -57,11 +57,12 @@ int ring_fft_smem(const FftPlan& p) { return fft_buf_len<T>(p.mmax_fft) * (int)s
 // threads of a ring block: one per 16 points of the longest FFT
 inline int ring_fft_threads(int mmax) { return mmax / 16 < 64 ? 64 : mmax / 16 > 512 ? 512 : mmax / 16; }
 
-// F[m * ldf + (i - 1)] = sum_j map_j e^{-i m phi_j} over ring i, m = 0 .. lmax,
-// times `weight` (all 4 nside - 1 rings; ldf >= 4 nside - 1).
+// F_k[m * ldf + (i - 1)] = weight * sum_j map_k,j e^{-i m phi_j} over ring i, m =
+// 0 .. lmax, for k < n <= 8 maps (all 4 nside - 1 rings; ldf >= 4 nside - 1);
+// F_k at F + k * fstride.
 template <typename T>
-int ring_analysis_t(clc_ctx* ctx, const FftPlan& plan, const double* map, int lmax, double weight, C2<T>* F,
-                    int ldf);
+int ring_analysis_t(clc_ctx* ctx, const FftPlan& plan, int n, const double* const* maps, int lmax, double weight,
+                    C2<T>* F, size_t fstride, int ldf);
 
 // Synthesis of real ring values from per-ring Fourier coefficients G_q[m][ring]
 // (q = 0 .. nq-1; ld = row length; G_q at G + q * ld * (lmax + 2)).
@@ -75,7 +76,11 @@ int ring_synthesis_t(clc_ctx* ctx, const FftPlan& plan, const C2<T>* G, int ld, 
 // FP64 forms
 inline int ring_analysis(clc_ctx* ctx, const FftPlan& plan, const double* map, int lmax, double weight,
                          double2* F, int ldf) {
-  return ring_analysis_t<double>(ctx, plan, map, lmax, weight, reinterpret_cast<C2<double>*>(F), ldf);
+  return ring_analysis_t<double>(ctx, plan, 1, &map, lmax, weight, reinterpret_cast<C2<double>*>(F), 0, ldf);
+}
+inline int ring_analysis_maps(clc_ctx* ctx, const FftPlan& plan, int n, const double* const* maps, int lmax,
+                              double weight, double2* F, size_t fstride, int ldf) {
+  return ring_analysis_t<double>(ctx, plan, n, maps, lmax, weight, reinterpret_cast<C2<double>*>(F), fstride, ldf);
 }
 inline int ring_synthesis(clc_ctx* ctx, const FftPlan& plan, const double2* G, int ld, int lmax, int mode,
                           double* const out[6]) {

@@ -62,18 +62,39 @@ __global__ void k_eb_combine(const double2* __restrict__ S, size_t q, int lmax, 
   B[o] = make_double2((a[1].x - b[0].y) * inv, (a[1].y + b[0].x) * inv);
 }
 
-// C_l = (a_l0 b_l0* + 2 sum_{m>0} Re a_lm b_lm*) / (2l+1), one thread per l;
-// coefficients packed with band limit lpack
-__global__ void k_cl(const double2* __restrict__ a, const double2* __restrict__ b, int lmax, int lpack,
-                     double* __restrict__ cl) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l > lmax) return;
+// C_l = (a_l0 b_l0* + 2 sum_{m>0} Re a_lm b_lm*) / (2l+1) of up to four pairs of
+// coefficient sets (blockIdx.y), each packed with its own band limit.  A block
+// takes 32 neighbouring l, which are neighbours in memory for every m, and its
+// warps every kClWarps-th m (one thread per l and all its m in turn: 0.34 ms per
+// spectrum at lmax 1024, against 0.02 ms for all four now).
+constexpr int kClWarps = 32;
+
+struct ClArgs {
+  const double2* a[4];
+  const double2* b[4];
+  int lpack[4];
+  double* cl[4];
+};
+
+__global__ void __launch_bounds__(32 * kClWarps) k_cl(ClArgs s, int lmax) {
+  __shared__ double red[kClWarps][33];
+  const int q = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int l = blockIdx.x * 32 + lane;
+  const double2 *a = s.a[q], *b = s.b[q];
+  const int lp = s.lpack[q];
   double acc = 0.0;
-  for (int m = 0; m <= l; ++m) {
-    const double2 x = a[alm_idx(lpack, l, m)], y = b[alm_idx(lpack, l, m)];
-    acc += (m ? 2.0 : 1.0) * (x.x * y.x + x.y * y.y);
+  for (int m = warp; m <= min(lmax, blockIdx.x * 32 + 31); m += kClWarps)
+    if (l <= lmax && m <= l) {
+      const double2 x = a[alm_idx(lp, l, m)], y = b[alm_idx(lp, l, m)];
+      acc += (m ? 2.0 : 1.0) * (x.x * y.x + x.y * y.y);
+    }
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (warp == 0 && l <= lmax) {
+    double t = 0.0;
+    for (int w = 0; w < kClWarps; ++w) t += red[w][lane];
+    s.cl[q][l] = t / (2.0 * l + 1.0);
   }
-  cl[l] = acc / (2.0 * l + 1.0);
 }
 
 // kappa, gamma_1, gamma_2, omega maps of A (SoA A[4][n], Eq. invmagmat)
@@ -99,28 +120,39 @@ __global__ void k_decompose_A_image(const double* __restrict__ x, const double* 
   const Ring r = ring_geom(nside, i);
   const double inv = 1.0 / (double)r.npix;
   const int shift = r.phi0 != 0.0 ? 1 : 0;
-  for (int j = threadIdx.x; j < r.npix; j += blockDim.x) {
-    const int64_t k = r.first + j;
-    double sp, cp;
-    sincospi((double)(2 * j + shift) * inv, &sp, &cp);
-    const double n0[3] = {r.s * cp, r.s * sp, r.z};
-    const double xv[3] = {x[k], x[n + k], x[2 * n + k]};
-    const double ix = rsqrt(dot3(xv, xv));
-    const double nx[3] = {xv[0] * ix, xv[1] * ix, xv[2] * ix};
-    double t[3], q[3], Q[4], Ai[4];
-    tangent_basis(nx, t, q);
-    transport_q(nx, t, n0, Q);
-    const double Ak[4] = {A[k], A[n + k], A[2 * n + k], A[3 * n + k]};
-    qaqt(Q, Ak, Ai);
-    out[k] = 1.0 - 0.5 * (Ai[0] + Ai[3]);
-    out[n + k] = -0.5 * (Ai[0] - Ai[3]);
-    out[2 * n + k] = -0.5 * (Ai[1] + Ai[2]);
-    out[3 * n + k] = 0.5 * (Ai[1] - Ai[2]);
+  const int quarter = r.npix / 4;
+  for (int j = threadIdx.x; j < quarter; j += blockDim.x) {
+    double s0, c0;
+    sincospi((double)(2 * j + shift) * inv, &s0, &c0);
+    for (int qd = 0; qd < 4; ++qd) {   // the pixels a quarter turn apart: swapped and negated, exactly
+      const double cp = qd == 0 ? c0 : qd == 1 ? -s0 : qd == 2 ? -c0 : s0;
+      const double sp = qd == 0 ? s0 : qd == 1 ? c0 : qd == 2 ? -s0 : -c0;
+      const int64_t k = r.first + j + qd * quarter;
+      const double n0[3] = {r.s * cp, r.s * sp, r.z};
+      const double xv[3] = {x[k], x[n + k], x[2 * n + k]};
+      const double ix = rsqrt(dot3(xv, xv));
+      const double nx[3] = {xv[0] * ix, xv[1] * ix, xv[2] * ix};
+      // transport along the geodesic as a plane rotation (q0, q1) (Appendix B);
+      // the basis at the pixel centre is (z cos, z sin, -s), (-sin, cos, 0)
+      double t[3], q[3];
+      tangent_basis(nx, t, q);
+      const double w = dot3(n0, t) / (1.0 + dot3(nx, n0));
+      const double t1x = r.z * cp, t1y = r.z * sp;
+      const double q0 = (t1x * t[0] + t1y * t[1] - r.s * t[2]) - w * (t1x * nx[0] + t1y * nx[1] - r.s * nx[2]);
+      const double q1 = (cp * t[1] - sp * t[0]) - w * (cp * nx[1] - sp * nx[0]);
+      // trace and antisymmetric part are kept, the shear turns by twice the angle
+      const double a = A[k], b = A[n + k], c = A[2 * n + k], d = A[3 * n + k];
+      const double c2 = fma(q0, q0, -q1 * q1), s2 = 2.0 * q0 * q1, df = a - d, sy = b + c;
+      out[k] = fma(-0.5, a + d, 1.0);
+      out[n + k] = -0.5 * fma(c2, df, -s2 * sy);
+      out[2 * n + k] = -0.5 * fma(s2, df, c2 * sy);
+      out[3 * n + k] = 0.5 * (b - c);
+    }
   }
 }
 
-static int power_spectrum(clc_ctx* ctx, const double2* a, const double2* b, int lmax, int lpack, double* cl) {
-  CLC_LAUNCH(ctx, "k_cl", k_cl, (lmax + 128) / 128, 128, 0, a, b, lmax, lpack, cl);
+static int power_spectra(clc_ctx* ctx, const ClArgs& s, int n, int lmax) {
+  CLC_LAUNCH(ctx, "k_cl", k_cl, dim3(lmax / 32 + 1, n), 32 * kClWarps, 0, s, lmax);
   return launch_check(ctx, "k_cl");
 }
 
@@ -138,8 +170,8 @@ static int eb_analysis(clc_ctx* ctx, const double* const* g, int ns, const doubl
   double2* S = (double2*)scratch(ctx, 2, 6 * sizeof(double2) * Q);
   if (!F || !S) return CLC_ENOMEM;
   const double w = 4.0 * kPi / (12.0 * (double)nside * nside);
-  for (int f = 0; f < 2 + ns; ++f)
-    if ((rc = ring_analysis(ctx, *plan, f < 2 ? g[f] : s[f - 2], lmax, w, F + f * fq, ldf))) return rc;
+  const double* in[4] = {g[0], g[1], ns > 0 ? s[0] : nullptr, ns > 1 ? s[1] : nullptr};
+  if ((rc = ring_analysis_maps(ctx, *plan, 2 + ns, in, lmax, w, F, fq, ldf))) return rc;
   const double2* cols[8];
   double2* out[8];
   int kind[8];
@@ -175,7 +207,12 @@ extern "C" int clc_power_spectrum(clc_ctx* ctx, const double* alm, const double*
   if (!ctx) return CLC_EINVAL;
   if (lmax < 0 || !alm || !cl) return set_err(ctx, CLC_EINVAL, "clc_power_spectrum: bad arguments");
   cudaSetDevice(ctx->device);
-  return power_spectrum(ctx, (const double2*)alm, (const double2*)(alm2 ? alm2 : alm), lmax, lmax, cl);
+  ClArgs s{};
+  s.a[0] = (const double2*)alm;
+  s.b[0] = (const double2*)(alm2 ? alm2 : alm);
+  s.lpack[0] = lmax;
+  s.cl[0] = cl;
+  return power_spectra(ctx, s, 1, lmax);
 }
 
 extern "C" int clc_lensing_spectra(clc_ctx* ctx, const double* x, const double* A, int nside, int lmax,
@@ -199,8 +236,11 @@ extern "C" int clc_lensing_spectra(clc_ctx* ctx, const double* x, const double* 
   const double *g[2] = {maps + np, maps + 2 * np}, *sc[2] = {maps, maps + 3 * np};
   if ((rc = eb_analysis(ctx, g, 2, sc, nside, lmax, E, B, salm))) return rc;
   const double2* alm[4] = {salm[0], E, B, salm[1]};   // kappa, E, B, omega
-  for (int q = 0; q < 4; ++q)
-    if ((rc = power_spectrum(ctx, alm[q], alm[q], lmax, q == 0 || q == 3 ? lmax + 1 : lmax, cl_out + (size_t)q * (lmax + 1))))
-      return rc;
-  return CLC_OK;
+  ClArgs cs{};
+  for (int q = 0; q < 4; ++q) {
+    cs.a[q] = cs.b[q] = alm[q];
+    cs.lpack[q] = q == 0 || q == 3 ? lmax + 1 : lmax;
+    cs.cl[q] = cl_out + (size_t)q * (lmax + 1);
+  }
+  return power_spectra(ctx, cs, 4, lmax);
 }
