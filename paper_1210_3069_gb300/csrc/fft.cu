@@ -251,8 +251,6 @@ int ring_synthesis_t(clc_ctx* ctx, const FftPlan& plan, const C2<T>* G, int ld, 
 }
 
 template int ring_analysis_t<double>(clc_ctx*, const FftPlan&, int, const double* const*, int, double, C2<double>*, size_t, int);
-template int ring_analysis_t<float>(clc_ctx*, const FftPlan&, int, const double* const*, int, double, C2<float>*, size_t, int);
 template int ring_synthesis_t<double>(clc_ctx*, const FftPlan&, const C2<double>*, int, int, int, double* const[6]);
-template int ring_synthesis_t<float>(clc_ctx*, const FftPlan&, const C2<float>*, int, int, int, double* const[6]);
 
 }  // namespace clc

@@ -72,10 +72,17 @@ __device__ __forceinline__ double times_pow2(double p, int e) {
 
 __device__ __forceinline__ int abs_hi(double v) { return __double2hiint(v) & 0x7fffffff; }
 
-// x (|x| <= 2^62) as eight signed base-256 digits: byte i of x + 0x80..80 is
-// digit i plus 128
-__device__ __forceinline__ unsigned long long dig_bias(double x) {
-  return (unsigned long long)__double2ll_rn(x) + 0x8080808080808080ull;
+// The integer nearest to v 2^e (at most 2^62 in magnitude) as eight signed
+// base-256 digits: byte i of it + 0x80..80 is digit i plus 128.  All on the
+// integer pipe: scaling and conversion were most of the packing's FP64
+// instructions (0.56 ms for eight columns at nside 512, lmax 1024).
+__device__ __forceinline__ unsigned long long dig_of(double v, int e) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  const int ex = (int)(u >> 52) & 0x7ff, sh = ex - 1075 + e;
+  const unsigned long long m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
+  unsigned long long r = 0;
+  if (ex && sh > -64) r = sh >= 0 ? m << sh : (m + (1ull << (-sh - 1))) >> -sh;
+  return ((long long)u < 0 ? 0 - r : r) + 0x8080808080808080ull;
 }
 // digit plane s (0 = most significant) of two values as FP16 integers
 __device__ __forceinline__ unsigned dig_pair(unsigned long long y0, unsigned long long y1, int s) {
@@ -200,7 +207,7 @@ __global__ void __launch_bounds__(256) k_dig_fill(int lmax, int R, int ms, const
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int r = rb * 64 + ch * 8 + q;
-      y[q] = dig_bias(ok && r < R ? times_pow2(src[r], (int)cexp[(size_t)ml * ldc + r] + 62 - er) : 0.0);
+      y[q] = ok && r < R ? dig_of(src[r], (int)cexp[(size_t)ml * ldc + r] + 62 - er) : dig_of(0.0, 0);
     }
 #pragma unroll
     for (int s = 0; s < kDigits; ++s)
@@ -424,6 +431,14 @@ __device__ __forceinline__ int col_exp(int hi) {
   return hi ? max(hi >> 20, 1) - 1022 : 0;
 }
 
+// high word of |v| scaled by a power of two given as an exponent field (0 for a
+// zero or a result below the normal range; infinities and NaN stay)
+__device__ __forceinline__ int scaled_hi(double v, int field) {
+  const int h = abs_hi(v);
+  if (h >= 0x7ff00000) return 0x7ff00000;
+  return h < 0x00100000 || h + field < 0x00100000 ? 0 : min(h + field, 0x7fefffff);
+}
+
 struct AnaCols {
   const double2* F[8];
   int kind[8];
@@ -441,7 +456,7 @@ __global__ void __launch_bounds__(256) k_dig_pack_analysis(AnaCols a, int nside,
   for (int v = blockIdx.y; v < a.nv; v += gridDim.y) {
     const double2* F = a.F[v] + (size_t)m * ldf;
     const int kind = a.kind[v];
-    // (even re, even im, odd re, odd im) of ring r, scaled
+    // (even re, even im, odd re, odd im) of ring r
     auto vals = [&](int r, double x[4]) {
       if (r >= R) {
         x[0] = x[1] = x[2] = x[3] = 0.0;
@@ -450,20 +465,24 @@ __global__ void __launch_bounds__(256) k_dig_pack_analysis(AnaCols a, int nside,
       const double2 n = F[r];
       double2 s = make_double2(0.0, 0.0);
       if (r + 1 != 2 * nside) s = F[4 * nside - r - 2];
-      double w = __longlong_as_double((long long)(1023 - (int)cx[r]) << 52);
-      if (kind) w *= fac[(size_t)(kind - 1) * R + r];
-      const double sg = kind == 1 ? -1.0 : 1.0;
-      x[0] = fma(sg, s.x, n.x) * w;
-      x[1] = fma(sg, s.y, n.y) * w;
-      x[2] = fma(-sg, s.x, n.x) * w;
-      x[3] = fma(-sg, s.y, n.y) * w;
+      if (kind == 1) s = make_double2(-s.x, -s.y);
+      x[0] = n.x + s.x;
+      x[1] = n.y + s.y;
+      x[2] = n.x - s.x;
+      x[3] = n.y - s.y;
+      if (kind) {
+        const double w = fac[(size_t)(kind - 1) * R + r];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) x[i] *= w;
+      }
     };
     int top[4] = {0, 0, 0, 0};
     for (int r = threadIdx.x; r < R; r += 256) {
       double x[4];
       vals(r, x);
+      const int c = (int)cx[r] << 20;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) top[i] = max(top[i], abs_hi(x[i]));
+      for (int i = 0; i < 4; ++i) top[i] = max(top[i], scaled_hi(x[i], -c));
     }
     block_max4(top, sh);
     int ec[4];
@@ -475,11 +494,12 @@ __global__ void __launch_bounds__(256) k_dig_pack_analysis(AnaCols a, int nside,
       double x0[4], x1[4];
       vals(r, x0);
       vals(r + 1, x1);
+      const int c0 = cx[r], c1 = cx[r + 1];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const bool ok = ec[i] != kNonFinite;
-        const unsigned long long y0 = dig_bias(ok ? times_pow2(x0[i], 62 - ec[i]) : 0.0);
-        const unsigned long long y1 = dig_bias(ok ? times_pow2(x1[i], 62 - ec[i]) : 0.0);
+        const unsigned long long y0 = ok ? dig_of(x0[i], 62 - ec[i] - c0) : 0;
+        const unsigned long long y1 = ok ? dig_of(x1[i], 62 - ec[i] - c1) : 0;
         __half* dst = op + ((size_t)(2 * ml + (i >> 1)) * nkb + (r >> 6)) * kOpBlock;
 #pragma unroll
         for (int s = 0; s < kDigits; ++s)
@@ -505,21 +525,22 @@ __global__ void __launch_bounds__(256) k_dig_pack_synthesis(SynthRhs s, int lmax
   const int np = max(gb[1] - gb[0], gb[2] - gb[1]) * 32;   // pairs of rows
   for (int q = blockIdx.y; q < s.nq; q += gridDim.y) {
     const double2* rhs = s.rhs + (size_t)q * (alm_idx(lt, lt, lt) + 1);
-    // (re, im) of row k of parity p, scaled
-    auto val = [&](int p, int k) -> double2 {
+    // (re, im) of row k of parity p and the row's exponent
+    auto val = [&](int p, int k, int& e) -> double2 {
       const int l = m + p + 2 * k;
+      e = 0;
       if (l > s.lq[q] || l > lt) return make_double2(0.0, 0.0);
-      const double2 v = rhs[alm_idx(lt, l, m)];
-      const int e = rexp[(size_t)gb[p] * 64 + k];
-      return make_double2(times_pow2(v.x, e), times_pow2(v.y, e));
+      e = rexp[(size_t)gb[p] * 64 + k];
+      return rhs[alm_idx(lt, l, m)];
     };
     int top[4] = {0, 0, 0, 0};
     for (int k = threadIdx.x; k < 2 * np; k += 256) {
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
-        const double2 v = val(p, k);
-        top[2 * p] = max(top[2 * p], abs_hi(v.x));
-        top[2 * p + 1] = max(top[2 * p + 1], abs_hi(v.y));
+        int e;
+        const double2 v = val(p, k, e);
+        top[2 * p] = max(top[2 * p], scaled_hi(v.x, e * 0x100000));
+        top[2 * p + 1] = max(top[2 * p + 1], scaled_hi(v.y, e * 0x100000));
       }
     }
     block_max4(top, sh);
@@ -533,14 +554,15 @@ __global__ void __launch_bounds__(256) k_dig_pack_synthesis(SynthRhs s, int lmax
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
         if (k >= (gb[p + 1] - gb[p]) * 64) continue;
-        const double2 a = val(p, k), b = val(p, k + 1);
+        int ea, eb;
+        const double2 a = val(p, k, ea), b = val(p, k + 1, eb);
         __half* dst = op + (size_t)(gb[p] + (k >> 6)) * kOpBlock;
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           const int e = ec[2 * p + i];
           const bool ok = e != kNonFinite;
-          const unsigned long long y0 = dig_bias(ok ? times_pow2(i ? a.y : a.x, 62 - e) : 0.0);
-          const unsigned long long y1 = dig_bias(ok ? times_pow2(i ? b.y : b.x, 62 - e) : 0.0);
+          const unsigned long long y0 = ok ? dig_of(i ? a.y : a.x, 62 - e + ea) : 0;
+          const unsigned long long y1 = ok ? dig_of(i ? b.y : b.x, 62 - e + eb) : 0;
 #pragma unroll
           for (int j = 0; j < kDigits; ++j)
             *reinterpret_cast<unsigned*>(dst + dig_off(j * kCols + 2 * q + i, k & 63)) = dig_pair(y0, y1, j);
