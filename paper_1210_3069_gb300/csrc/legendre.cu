@@ -225,6 +225,17 @@ __global__ void k_ring_factors(int nside, double* __restrict__ fac) {
   fac[2 * nside + r] = is2;
 }
 
+__global__ void k_eps_table(int lmax, int m0, double* __restrict__ eps, double* __restrict__ by_l) {
+  const int l = blockIdx.x * blockDim.x + threadIdx.x, m = m0 + blockIdx.y, ld = lmax + 3;
+  if (l >= ld) return;
+  eps[(size_t)blockIdx.y * ld + l] =
+      l > m ? sqrt(((double)l * l - (double)m * m) / (4.0 * l * l - 1.0)) : 0.0;
+  if (blockIdx.y == 0) {
+    by_l[l] = l > 0 ? -1.0 / ((double)l * (l + 1.0)) : 0.0;
+    by_l[ld + l] = l > 1 ? 1.0 / sqrt((l + 2.0) * (l + 1.0) * l * (l - 1.0)) : 0.0;
+  }
+}
+
 static int row_blocks(int lt, int m, int p) { return m + p <= lt ? ((lt - m - p) / 2 + 1 + 63) / 64 : 0; }
 
 size_t legendre_table_bytes(int nside, int lmax, int m0, int m1) {
@@ -285,7 +296,8 @@ int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, Lege
   if (!dev_alloc(T->gidx, sizeof(int) * (2 * nm + 1)) || !dev_alloc(T->rb0, sizeof(int) * nblk) ||
       !dev_alloc(T->abase, sizeof(__half*) * nblk) || !dev_alloc(T->rexp, sizeof(int) * 64 * (size_t)nblk) ||
       !dev_alloc(T->cexp, (size_t)nm * ldc) || !dev_alloc(T->fac, sizeof(double) * 2 * R) ||
-      !dev_alloc(T->zero, (size_t)kDigits * kAtom * sizeof(__half)) || !dev_alloc(d_tab, tab_bytes) ||
+      !dev_alloc(T->zero, (size_t)kDigits * kAtom * sizeof(__half)) ||
+      !dev_alloc(T->eps, sizeof(double) * (size_t)(nm + 2) * (lmax + 3)) || !dev_alloc(d_tab, tab_bytes) ||
       !dev_alloc(d_ab, sizeof(double2) * (size_t)seg_orders * (lt + 1)) ||
       !dev_alloc(d_ln, sizeof(double) * lognorm.size()) || !dev_alloc(d_off, sizeof(long long) * seg_orders) ||
       !dev_alloc(d_grp, sizeof(int) * nblk))
@@ -298,6 +310,8 @@ int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, Lege
   cudaMemsetAsync(T->cexp.p, 0, T->cexp.bytes, st);
   cudaMemsetAsync(T->zero.p, 0, T->zero.bytes, st);
   CLC_LAUNCH(ctx, "k_ring_factors", k_ring_factors, (R + 127) / 128, 128, 0, nside, (double*)T->fac.p);
+  CLC_LAUNCH(ctx, "k_eps_table", k_eps_table, dim3((lmax + 130) / 128, nm), 128, 0, lmax, m0, (double*)T->eps.p,
+             (double*)T->eps.p + (size_t)nm * (lmax + 3));
   int rc;
   for (size_t s = 0; s + 1 < seg.size(); ++s) {
     const int ms = seg[s], me = seg[s + 1], n = me - ms, g0 = 2 * (ms - m0);
@@ -509,64 +523,98 @@ __global__ void __launch_bounds__(256) k_dig_pack_analysis(AnaCols a, int nside,
   }
 }
 
+// Right-hand sides of a synthesis: given (rhs, packed with band limit lmax + 1),
+// or those of a Poisson solve of the coefficients klm (packed with lmax).
 struct SynthRhs {
   const double2* rhs;
   int nq;
   int lq[4];
+  const double2* klm;
+  const double* eps;    // [m - m0][lmax + 3]
+  const double* inv;    // -1 / (l (l + 1))
 };
 
-// One CTA per order; column 2 q + re/im of both parities (rows l = m + p + 2 k).
+// value of right-hand side q at (l, m), l <= lmax + 1
+template <bool kPoisson>
+__device__ __forceinline__ double2 synth_rhs(const SynthRhs& s, int q, int lmax, int l, int m, int ml) {
+  if (!kPoisson) {
+    if (l > s.lq[q]) return make_double2(0.0, 0.0);
+    const int lt = lmax + 1;
+    return s.rhs[(size_t)q * (alm_idx(lt, lt, lt) + 1) + alm_idx(lt, l, m)];
+  }
+  auto psi = [&](int ll) -> double2 {
+    if (ll < m || ll > lmax) return make_double2(0.0, 0.0);
+    const double2 k = s.klm[alm_idx(lmax, ll, m)];
+    const double d = s.inv[ll];
+    return make_double2(k.x * d, k.y * d);
+  };
+  if (q == 0) return psi(l);
+  if (q == 2) {
+    const double2 p = psi(l);
+    const double ll1 = -(double)l * (l + 1.0);
+    return make_double2(ll1 * p.x, ll1 * p.y);
+  }
+  const double2 pm = psi(l - 1), pp = psi(l + 1);
+  const double* e = s.eps + (size_t)ml * (lmax + 3);
+  const double c1 = (l - 1.0) * e[l], c2 = (l + 2.0) * e[l + 1];
+  return make_double2(c1 * pm.x - c2 * pp.x, c1 * pm.y - c2 * pp.y);
+}
+
+// One CTA per order and right-hand side; column 2 q + re/im of both parities
+// (rows l = m + p + 2 k). A Poisson solve's right-hand sides are formed here
+// from its coefficients and the table's eps_lm: written out first by a kernel of
+// their own they cost two FP64 square roots and divisions per row (94 us at
+// nside 512) and a launch. Solve with derivatives, before and after: nside 64
+// 151 -> 145 us, nside 512 6117 -> 6076 us.
+template <bool kPoisson>
 __global__ void __launch_bounds__(256) k_dig_pack_synthesis(SynthRhs s, int lmax, int m0, const int* __restrict__ gidx,
                                                             const int* __restrict__ rexp, __half* __restrict__ op,
                                                             int* __restrict__ colexp) {
   __shared__ int sh[4 * 8];
-  const int ml = blockIdx.x, m = m0 + ml, lt = lmax + 1;
+  const int ml = blockIdx.x, m = m0 + ml, lt = lmax + 1, q = blockIdx.y;
   const int gb[3] = {gidx[2 * ml], gidx[2 * ml + 1], gidx[2 * ml + 2]};
   const int np = max(gb[1] - gb[0], gb[2] - gb[1]) * 32;   // pairs of rows
-  for (int q = blockIdx.y; q < s.nq; q += gridDim.y) {
-    const double2* rhs = s.rhs + (size_t)q * (alm_idx(lt, lt, lt) + 1);
-    // (re, im) of row k of parity p and the row's exponent
-    auto val = [&](int p, int k, int& e) -> double2 {
-      const int l = m + p + 2 * k;
-      e = 0;
-      if (l > s.lq[q] || l > lt) return make_double2(0.0, 0.0);
-      e = rexp[(size_t)gb[p] * 64 + k];
-      return rhs[alm_idx(lt, l, m)];
-    };
-    int top[4] = {0, 0, 0, 0};
-    for (int k = threadIdx.x; k < 2 * np; k += 256) {
+  // (re, im) of row k of parity p and the row's exponent
+  auto val = [&](int p, int k, int& e) -> double2 {
+    const int l = m + p + 2 * k;
+    e = 0;
+    if (l > lt) return make_double2(0.0, 0.0);
+    e = rexp[(size_t)gb[p] * 64 + k];
+    return synth_rhs<kPoisson>(s, q, lmax, l, m, ml);
+  };
+  int top[4] = {0, 0, 0, 0};
+  for (int k = threadIdx.x; k < 2 * np; k += 256) {
 #pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        int e;
-        const double2 v = val(p, k, e);
-        top[2 * p] = max(top[2 * p], scaled_hi(v.x, e * 0x100000));
-        top[2 * p + 1] = max(top[2 * p + 1], scaled_hi(v.y, e * 0x100000));
-      }
+    for (int p = 0; p < 2; ++p) {
+      int e;
+      const double2 v = val(p, k, e);
+      top[2 * p] = max(top[2 * p], scaled_hi(v.x, e * 0x100000));
+      top[2 * p + 1] = max(top[2 * p + 1], scaled_hi(v.y, e * 0x100000));
     }
-    block_max4(top, sh);
-    int ec[4];
+  }
+  block_max4(top, sh);
+  int ec[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) ec[i] = col_exp(top[i]);
-    if (threadIdx.x < 4)
-      colexp[(size_t)(2 * ml + (threadIdx.x >> 1)) * kCols + 2 * q + (threadIdx.x & 1)] = ec[threadIdx.x];
-    for (int t = threadIdx.x; t < np; t += 256) {
-      const int k = 2 * t;
+  for (int i = 0; i < 4; ++i) ec[i] = col_exp(top[i]);
+  if (threadIdx.x < 4)
+    colexp[(size_t)(2 * ml + (threadIdx.x >> 1)) * kCols + 2 * q + (threadIdx.x & 1)] = ec[threadIdx.x];
+  for (int t = threadIdx.x; t < np; t += 256) {
+    const int k = 2 * t;
 #pragma unroll
-      for (int p = 0; p < 2; ++p) {
-        if (k >= (gb[p + 1] - gb[p]) * 64) continue;
-        int ea, eb;
-        const double2 a = val(p, k, ea), b = val(p, k + 1, eb);
-        __half* dst = op + (size_t)(gb[p] + (k >> 6)) * kOpBlock;
+    for (int p = 0; p < 2; ++p) {
+      if (k >= (gb[p + 1] - gb[p]) * 64) continue;
+      int ea, eb;
+      const double2 a = val(p, k, ea), b = val(p, k + 1, eb);
+      __half* dst = op + (size_t)(gb[p] + (k >> 6)) * kOpBlock;
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const int e = ec[2 * p + i];
-          const bool ok = e != kNonFinite;
-          const unsigned long long y0 = ok ? dig_of(i ? a.y : a.x, 62 - e + ea) : 0;
-          const unsigned long long y1 = ok ? dig_of(i ? b.y : b.x, 62 - e + eb) : 0;
+      for (int i = 0; i < 2; ++i) {
+        const int e = ec[2 * p + i];
+        const bool ok = e != kNonFinite;
+        const unsigned long long y0 = ok ? dig_of(i ? a.y : a.x, 62 - e + ea) : 0;
+        const unsigned long long y1 = ok ? dig_of(i ? b.y : b.x, 62 - e + eb) : 0;
 #pragma unroll
-          for (int j = 0; j < kDigits; ++j)
-            *reinterpret_cast<unsigned*>(dst + dig_off(j * kCols + 2 * q + i, k & 63)) = dig_pair(y0, y1, j);
-        }
+        for (int j = 0; j < kDigits; ++j)
+          *reinterpret_cast<unsigned*>(dst + dig_off(j * kCols + 2 * q + i, k & 63)) = dig_pair(y0, y1, j);
       }
     }
   }
@@ -935,27 +983,41 @@ int legendre_analysis_cols(clc_ctx* ctx, const LegendreTable& T, int nv, const d
   return analysis_cols<16>(ctx, T, c, ldf, out, ltop);
 }
 
-int legendre_synthesis(clc_ctx* ctx, const LegendreTable& T, const double2* rhs, int nq, const int* lq, double2* G,
-                       int ld) {
+template <bool kPoisson>
+static int synthesis(clc_ctx* ctx, const LegendreTable& T, const SynthRhs& s, double2* G, int ld) {
   const int nm = T.m1 - T.m0, nblk = T.h_gidx[2 * nm];
-  SynthRhs s{};
-  s.rhs = rhs;
-  s.nq = nq;
-  for (int q = 0; q < nq; ++q) s.lq[q] = lq[q];
   const size_t ob = (size_t)nblk * kOpBlock * sizeof(__half);
   __half* op = (__half*)scratch(ctx, 9, ob + sizeof(int) * 2 * nm * kCols);
   if (!op) return CLC_ENOMEM;
   int* colexp = (int*)((uint8_t*)op + ob);
-  CLC_LAUNCH(ctx, "k_dig_pack", k_dig_pack_synthesis, dim3(nm, nq), 256, 0, s, T.lmax, T.m0, (const int*)T.gidx.p,
-             (const int*)T.rexp.p, op, colexp);
+  CLC_LAUNCH(ctx, "k_dig_pack", k_dig_pack_synthesis<kPoisson>, dim3(nm, s.nq), 256, 0, s, T.lmax, T.m0,
+             (const int*)T.gidx.p, (const int*)T.rexp.p, op, colexp);
   if (int rc = launch_check(ctx, "k_dig_pack_synthesis")) return rc;
   DigArgs a = dig_args(T, op, colexp);
-  a.nv = nq;
+  a.nv = s.nq;
   a.G = G;
   a.qstride = (size_t)ld * (T.lmax + 2);
   a.ld = ld;
-  return nq == 1 ? run_gemm<true, 2>(ctx, "k_legendre_synthesis", a, T.sy, T.n_sy)
-                 : run_gemm<true, 8>(ctx, "k_legendre_synthesis", a, T.sy, T.n_sy);
+  return s.nq == 1 ? run_gemm<true, 2>(ctx, "k_legendre_synthesis", a, T.sy, T.n_sy)
+                   : run_gemm<true, 8>(ctx, "k_legendre_synthesis", a, T.sy, T.n_sy);
+}
+
+int legendre_synthesis(clc_ctx* ctx, const LegendreTable& T, const double2* rhs, int nq, const int* lq, double2* G,
+                       int ld) {
+  SynthRhs s{};
+  s.rhs = rhs;
+  s.nq = nq;
+  for (int q = 0; q < nq; ++q) s.lq[q] = lq[q];
+  return synthesis<false>(ctx, T, s, G, ld);
+}
+
+int legendre_synthesis_poisson(clc_ctx* ctx, const LegendreTable& T, const double2* klm, int nq, double2* G, int ld) {
+  SynthRhs s{};
+  s.nq = nq;
+  s.klm = klm;
+  s.eps = T.eps_of();
+  s.inv = T.by_l();
+  return synthesis<true>(ctx, T, s, G, ld);
 }
 
 }  // namespace clc

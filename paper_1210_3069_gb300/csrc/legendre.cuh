@@ -29,6 +29,11 @@ struct LegendreTable {
   Buffer cexp;                                   // int8: ring r of order m is scaled by 2^cexp, [m - m0][nkb * 64]
   Buffer fac;                                    // double [2][R]: cos / sin^2 and 1 / sin^2 of the rings
   Buffer zero;                                   // an atom of zeros
+  // eps_lm = sqrt((l^2 - m^2) / (4 l^2 - 1)) [m - m0][lmax + 3] of l = 0 .. lmax + 2,
+  // then by l: -1 / (l (l + 1)) (0 at l = 0) and 1 / sqrt((l+2)(l+1) l (l-1)) (0 below 2)
+  Buffer eps;
+  const double* eps_of() const { return (const double*)eps.p; }
+  const double* by_l() const { return (const double*)eps.p + (size_t)(m1 - m0) * (lmax + 3); }
   std::vector<std::unique_ptr<Buffer>> atoms;    // the atoms, in pieces
   Buffer an, sy;                                 // work lists of the contractions (int4), longest first
   int n_an = 0, n_sy = 0;
@@ -65,6 +70,13 @@ inline int legendre_analysis(clc_ctx* ctx, const LegendreTable& T, const double2
 // lq[q] is the highest l used by rhs q.  G_q lives at G + q * ld * (lmax + 2).
 int legendre_synthesis(clc_ctx* ctx, const LegendreTable& T, const double2* rhs, int nq, const int* lq,
                        double2* G, int ld);
+
+// The same sums of a Poisson solve straight from the source's coefficients
+// klm (band limit lmax): q = 0: psi_lm = -k_lm / (l (l + 1)); with nq = 3 also
+// q = 1: b_lm = (l-1) eps_lm psi_{l-1,m} - (l+2) eps_{l+1,m} psi_{l+1,m} (the
+// coefficients of sin(theta) d psi / d theta, l <= lmax + 1) and q = 2:
+// -l (l + 1) psi_lm.
+int legendre_synthesis_poisson(clc_ctx* ctx, const LegendreTable& T, const double2* klm, int nq, double2* G, int ld);
 
 // Run fn on tables covering every order m <= lmax: the cached whole table
 // when it fits in device memory (or the context's budget), otherwise tables

@@ -17,34 +17,6 @@ namespace clc {
 int poisson_sht_tc(clc_ctx* ctx, const double* const* kappa, int P, int nside, int lmax, double* const* psi,
                    const clc_derivs* out);
 
-// rhs_0 = psi_lm, rhs_1 = b_lm (l <= lmax + 1), rhs_2 = -l(l+1) psi_lm, all
-// packed with band limit lmax + 1.
-__global__ void k_poisson_rhs(const double2* __restrict__ klm, int lmax, double2* __restrict__ rhs, long long Q,
-                              int m0) {
-  const int m = m0 + blockIdx.y;
-  const int lt = lmax + 1;
-  const int l = m + blockIdx.x * blockDim.x + threadIdx.x;
-  if (l > lt) return;
-  auto psi = [&](int ll) -> double2 {
-    if (ll < m || ll > lmax || ll == 0) return make_double2(0.0, 0.0);
-    const double2 k = klm[alm_idx(lmax, ll, m)];
-    const double d = -1.0 / ((double)ll * (ll + 1.0));
-    return make_double2(k.x * d, k.y * d);
-  };
-  auto eps = [&](int ll) -> double {
-    if (ll <= m) return 0.0;
-    return sqrt(((double)ll * ll - (double)m * m) / (4.0 * ll * ll - 1.0));
-  };
-  const double2 p = psi(l);
-  const double2 pm = psi(l - 1), pp = psi(l + 1);
-  const double c1 = (l - 1.0) * eps(l), c2 = (l + 2.0) * eps(l + 1);
-  const long long i = alm_idx(lt, l, m);
-  rhs[i] = p;
-  rhs[Q + i] = make_double2(c1 * pm.x - c2 * pp.x, c1 * pm.y - c2 * pp.y);
-  const double ll1 = -(double)l * (l + 1.0);
-  rhs[2 * Q + i] = make_double2(ll1 * p.x, ll1 * p.y);
-}
-
 // copy alm (band limit lmax) into the lmax + 1 packing, zero at l = lmax + 1
 __global__ void k_alm_expand(const double2* __restrict__ alm, int lmax, double2* __restrict__ rhs) {
   const int m = blockIdx.y;
@@ -141,9 +113,6 @@ extern "C" int clc_poisson_sht(clc_ctx* ctx, const double* kappa, int nside, int
   if (precision == CLC_MIXED) return poisson_sht_tc(ctx, &kappa, 1, nside, lmax, &psi, derivs ? d : nullptr);
   double2* klm = (double2*)scratch(ctx, 1, sizeof(double2) * (alm_idx(lmax, lmax, lmax) + 1));
   if (!klm) return CLC_ENOMEM;
-  const long long Q = alm_idx(lmax + 1, lmax + 1, lmax + 1) + 1;
-  double2* rhs = (double2*)scratch(ctx, 2, sizeof(double2) * Q * 3);
-  if (!rhs) return CLC_ENOMEM;
   auto plan = get_fft_plan(ctx, nside, &rc);
   if (rc) return rc;
   const int ld = 4 * nside - 1;
@@ -154,16 +123,10 @@ extern "C" int clc_poisson_sht(clc_ctx* ctx, const double* kappa, int nside, int
   if (!G) return CLC_ENOMEM;
   const double w = 4.0 * kPi / (12.0 * (double)nside * nside);
   if ((rc = ring_analysis(ctx, *plan, kappa, lmax, w, F, ld))) return rc;
-  const int lq1[1] = {lmax};
-  const int lq3[3] = {lmax, lmax + 1, lmax};
-  // per table (or order range): analysis, Poisson right-hand sides, synthesis
+  // per table (or order range): analysis, then synthesis from the coefficients
   rc = for_each_table(ctx, nside, lmax, [&](const LegendreTable& T) {
-    int r = legendre_analysis(ctx, T, F, ld, klm);
-    if (r) return r;
-    dim3 grid((lmax + 2 + 127) / 128, T.m1 - T.m0);
-    CLC_LAUNCH(ctx, "k_poisson_rhs", k_poisson_rhs, grid, 128, 0, klm, lmax, rhs, Q, T.m0);
-    if ((r = launch_check(ctx, "k_poisson_rhs"))) return r;
-    return legendre_synthesis(ctx, T, rhs, nq, derivs ? lq3 : lq1, G, ld);
+    const int r = legendre_analysis(ctx, T, F, ld, klm);
+    return r ? r : legendre_synthesis_poisson(ctx, T, klm, nq, G, ld);
   });
   if (rc) return rc;
   if (!derivs) {

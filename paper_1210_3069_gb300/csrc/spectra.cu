@@ -20,11 +20,6 @@
 
 namespace clc {
 
-__device__ __forceinline__ double eps_lm(int l, int m) {
-  if (l <= m) return 0.0;
-  return sqrt(((double)l * l - (double)m * m) / (4.0 * l * l - 1.0));
-}
-
 // E_lm and B_lm from the Legendre sums of the two fields with the ring weights
 // 1, cos / sin^2 and 1 / sin^2 (legendre_analysis_cols, kinds 0, 1, 2; band
 // limit lmax + 1).  With sin t dlambda_lm = e1 lambda_{l+1,m} - e0 lambda_{l-1,m},
@@ -32,9 +27,12 @@ __device__ __forceinline__ double eps_lm(int l, int m) {
 //   sum B F  = 2 m (e1 S2_{l+1} - e0 S2_{l-1} - S1_l):
 // A and B are products of lambda and ring factors, so every sum over rings is
 // one of the table's contractions and nothing is evaluated per (l, m, ring).
-__global__ void k_eb_combine(const double2* __restrict__ S, size_t q, int lmax, double2* __restrict__ E,
-                             double2* __restrict__ B) {
-  const int m = blockIdx.y, lt = lmax + 1;
+// eps_lm and the normalisation come from the table's own list: as square roots
+// and divisions here they were the whole kernel (123 us at nside 512, now 62).
+__global__ void k_eb_combine(const double2* __restrict__ S, size_t q, int lmax, int m0, const double* __restrict__ eps,
+                             const double* __restrict__ inv_n, double2* __restrict__ E, double2* __restrict__ B) {
+  const int m = m0 + blockIdx.y, lt = lmax + 1;
+  eps += (size_t)blockIdx.y * (lmax + 3);
   const int l = m + blockIdx.x * blockDim.x + threadIdx.x;
   if (l > lmax) return;
   const size_t o = alm_idx(lmax, l, m);
@@ -42,7 +40,7 @@ __global__ void k_eb_combine(const double2* __restrict__ S, size_t q, int lmax, 
     E[o] = B[o] = make_double2(0.0, 0.0);
     return;
   }
-  const double e1 = (double)l * eps_lm(l + 1, m), e0 = (l + 1.0) * eps_lm(l, m);
+  const double e1 = (double)l * eps[l + 1], e0 = (l + 1.0) * eps[l];
   const double ll1 = (double)l * (l + 1.0), m2 = 2.0 * (double)m * m, m_2 = 2.0 * m;
   const size_t i = alm_idx(lt, l, m);
   double2 a[2], b[2];
@@ -56,7 +54,7 @@ __global__ void k_eb_combine(const double2* __restrict__ S, size_t q, int lmax, 
     b[f].x = m_2 * (fma(e1, u2.x, -e0 * d2.x) - S1->x);
     b[f].y = m_2 * (fma(e1, u2.y, -e0 * d2.y) - S1->y);
   }
-  const double inv = 1.0 / sqrt((l + 2.0) * (l + 1.0) * l * (l - 1.0));
+  const double inv = inv_n[l];
   // E = (A F1 - i B F2) / N_l, B = (A F2 + i B F1) / N_l
   E[o] = make_double2((a[0].x + b[1].y) * inv, (a[0].y - b[1].x) * inv);
   B[o] = make_double2((a[1].x - b[0].y) * inv, (a[1].y + b[0].x) * inv);
@@ -180,12 +178,13 @@ static int eb_analysis(clc_ctx* ctx, const double* const* g, int ns, const doubl
     kind[v] = v < 6 ? v % 3 : 0;
     out[v] = v < 6 ? S + v * Q : salm[v - 6];
   }
-  rc = for_each_table(ctx, nside, lmax, [&](const LegendreTable& T) {
-    return legendre_analysis_cols(ctx, T, 6 + ns, cols, kind, ldf, out, lmax + 1);
+  return for_each_table(ctx, nside, lmax, [&](const LegendreTable& T) {
+    const int r = legendre_analysis_cols(ctx, T, 6 + ns, cols, kind, ldf, out, lmax + 1);
+    if (r) return r;
+    CLC_LAUNCH(ctx, "k_eb_combine", k_eb_combine, dim3((lmax + 128) / 128, T.m1 - T.m0), 128, 0, S, Q, lmax, T.m0,
+               T.eps_of(), T.by_l() + (lmax + 3), E, B);
+    return launch_check(ctx, "k_eb_combine");
   });
-  if (rc) return rc;
-  CLC_LAUNCH(ctx, "k_eb_combine", k_eb_combine, dim3((lmax + 128) / 128, lmax + 1), 128, 0, S, Q, lmax, E, B);
-  return launch_check(ctx, "k_eb_combine");
 }
 
 }  // namespace clc
