@@ -128,16 +128,27 @@ const RingS* get_ring_table(clc_ctx* ctx, int nside, int* rc) {
   *rc = CLC_OK;
   auto it = ctx->ring_tables.find(nside);
   if (it != ctx->ring_tables.end()) return (const RingS*)it->second->p;
+  // built and finished on a stream of its own: the caller's may be in capture
+  // (its work runs later, if ever, and allocations are refused there), and later
+  // calls may come on another stream
   auto b = std::make_shared<Buffer>();
   b->bytes = sizeof(RingS) * (4 * (size_t)nside - 1);
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  cudaStream_t cs = nullptr;
   if (cudaMalloc(&b->p, b->bytes) != cudaSuccess) {
     cudaGetLastError();
     b->p = nullptr;
     *rc = set_err(ctx, CLC_ENOMEM, "ring table allocation failed");
-    return nullptr;
+  } else if (!(*rc = cuda_check(ctx, cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking), "ring table stream"))) {
+    k_ring_table<<<(4 * nside + 126) / 128, 128, 0, cs>>>(nside, (RingS*)b->p);
+    *rc = launch_check(ctx, "k_ring_table");
+    const cudaError_t e = cudaStreamSynchronize(cs);
+    if (!*rc) *rc = cuda_check(ctx, e, "ring table");
+    cudaStreamDestroy(cs);
   }
-  CLC_LAUNCH(ctx, "k_ring_table", k_ring_table, (4 * nside + 126) / 128, 128, 0, nside, (RingS*)b->p);
-  if ((*rc = launch_check(ctx, "k_ring_table"))) return nullptr;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (*rc) return nullptr;
   ctx->ring_tables[nside] = b;
   return (const RingS*)b->p;
 }

@@ -75,48 +75,39 @@ __global__ void k_rays_init_pixels(int nside, double chi0, int nb, RayPtrs R) {
   }
 }
 
-// Lens fields at the ray from RING maps: alpha as a tangent 3-vector and U as
-// a tangent 3x3 tensor, ring-bilinear interpolation, projection on the basis
-// at the ray.
-__device__ void map_lens_fields(const clc_derivs& M, int nside, const double nv[3], double out[5]) {
+// Lens fields at the ray from RING maps, in the ray's basis (t, q): ring-bilinear
+// interpolation of alpha as a tangent vector and U as a tangent tensor, each
+// neighbour's components projected by the four products of the two bases.  FP64
+// bound: the neighbours' bases come from the ring table and one sincospi each
+// (a pixel stands at pi (2 pos + 0 or 1) / npix), and nothing is held in 3x3 form.
+__device__ void map_lens_fields(const clc_derivs& M, int nside, const RingS* __restrict__ rings, const double nv[3],
+                                const double t[3], const double q[3], double out[5]) {
   const double th = atan2(sqrt(nv[0] * nv[0] + nv[1] * nv[1]), nv[2]);
   double ph = atan2(nv[1], nv[0]);
   if (ph < 0) ph += 2.0 * kPi;
-  const Interp8 w = interp_weights(nside, th, ph);
-  double a3[3] = {0, 0, 0}, U3[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-  for (int k = 0; k < 8; ++k) {
-    if (w.w[k] == 0.0) continue;
-    const int64_t p = w.p[k];
-    int64_t j;
-    const int i = pix2ring(nside, p, &j);
-    const Ring r = ring_geom(nside, i);
-    const double phi = r.phi0 + (2.0 * kPi) * (double)j / (double)r.npix;
-    const double cp = cos(phi), sp = sin(phi);
-    const double t[3] = {r.z * cp, r.z * sp, -r.s};
-    const double q[3] = {-sp, cp, 0.0};
-    const double at = M.a_th[p], ap = M.a_ph[p], utt = M.u_tt[p], upp = M.u_pp[p], utp = M.u_tp[p];
+  RingInterp w;
+  ring_interp(nside, rings, th, ph, w);
+#pragma unroll
+  for (int a = 0; a < 5; ++a) out[a] = 0.0;
+  for (int k = 0; k < w.n; ++k) {
     const double ww = w.w[k];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      a3[a] += ww * (at * t[a] + ap * q[a]);
-#pragma unroll
-      for (int b = 0; b < 3; ++b)
-        U3[a][b] += ww * (utt * t[a] * t[b] + upp * q[a] * q[b] + utp * (t[a] * q[b] + q[a] * t[b]));
-    }
+    if (ww == 0.0) continue;
+    const int64_t p = w.p[k];
+    const RingS& r = rings[w.ring[k] - 1];
+    double sp, cp;
+    sincospi((double)(2 * w.pos[k] + (r.r.phi0 != 0.0 ? 1 : 0)) / (double)r.r.npix, &sp, &cp);
+    // bases at the pixel: tk = (z c, z s, -sin), qk = (-s, c, 0)
+    const double h = t[0] * cp + t[1] * sp, g = q[0] * cp + q[1] * sp;
+    const double tt = r.r.z * h - r.r.s * t[2], tq = t[1] * cp - t[0] * sp;   // t.tk, t.qk
+    const double qt = r.r.z * g - r.r.s * q[2], qq = q[1] * cp - q[0] * sp;   // q.tk, q.qk
+    const double at = M.a_th[p], ap = M.a_ph[p], utt = M.u_tt[p], upp = M.u_pp[p], utp = M.u_tp[p];
+    out[0] += ww * (at * tt + ap * tq);
+    out[1] += ww * (at * qt + ap * qq);
+    const double b = utt * tt + utp * tq, c = utp * tt + upp * tq;   // U t in the pixel's basis
+    out[2] += ww * (b * tt + c * tq);
+    out[4] += ww * (b * qt + c * qq);
+    out[3] += ww * (qt * (utt * qt + utp * qq) + qq * (utp * qt + upp * qq));
   }
-  double t[3], q[3];
-  tangent_basis(nv, t, q);
-  out[0] = dot3(a3, t);
-  out[1] = dot3(a3, q);
-  double Ut[3], Uq[3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    Ut[a] = U3[a][0] * t[0] + U3[a][1] * t[1] + U3[a][2] * t[2];
-    Uq[a] = U3[a][0] * q[0] + U3[a][1] * q[1] + U3[a][2] * q[2];
-  }
-  out[2] = dot3(t, Ut);
-  out[3] = dot3(q, Uq);
-  out[4] = dot3(t, Uq);
 }
 
 struct StepCoef {
@@ -183,7 +174,8 @@ __device__ __forceinline__ void rotate_2x2(double q0, double q1, const double A[
 }
 
 template <bool kMG>
-__global__ void k_ray_step(RayPtrs R, MGView V, clc_derivs M, int nside_maps, StepCoef sc) {
+__global__ void k_ray_step(RayPtrs R, MGView V, clc_derivs M, int nside_maps, const RingS* __restrict__ rings,
+                           StepCoef sc) {
   const int64_t n = R.n;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
     double x[3], be[3], A[4], Ap[4];
@@ -198,7 +190,7 @@ __global__ void k_ray_step(RayPtrs R, MGView V, clc_derivs M, int nside_maps, St
     tangent_basis(nv, t, q);
     double L[5];
     if (kMG) patch_lens_fields(V, R.bundle[k], nv, t, q, L);
-    else map_lens_fields(M, nside_maps, nv, L);
+    else map_lens_fields(M, nside_maps, rings, nv, t, q, L);
     // Eq. Atraj in the basis at n
     const double U[4] = {L[2], L[4], L[4], L[3]};
     double An[4];
@@ -301,10 +293,14 @@ extern "C" int clc_ray_step(clc_ctx* ctx, const clc_plane_solution* sol, const c
   clc_derivs M{};
   if (maps) M = *maps;
   if (sol) {
-    CLC_LAUNCH(ctx, "k_ray_step", k_ray_step<true>, blocks(ctx, r->n, 128), 128, 0, ray_ptrs(r), mg_view(sol), M, 0, sc);
+    CLC_LAUNCH(ctx, "k_ray_step", k_ray_step<true>, blocks(ctx, r->n, 128), 128, 0, ray_ptrs(r), mg_view(sol), M, 0,
+               nullptr, sc);
   } else {
     MGView V{};
-    CLC_LAUNCH(ctx, "k_ray_step", k_ray_step<false>, blocks(ctx, r->n, 128), 128, 0, ray_ptrs(r), V, M, nside_maps, sc);
+    const RingS* rings = get_ring_table(ctx, nside_maps, &rc);
+    if (rc) return rc;
+    CLC_LAUNCH(ctx, "k_ray_step", k_ray_step<false>, blocks(ctx, r->n, 128), 128, 0, ray_ptrs(r), V, M,
+               nside_maps, rings, sc);
   }
   return launch_check(ctx, "k_ray_step");
 }
