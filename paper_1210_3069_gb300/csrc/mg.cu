@@ -185,18 +185,24 @@ __global__ void k_mg_setup_defect(int n, const double* __restrict__ rot, const d
   if (threadIdx.x == 0 && ff != 0.0) atomicAdd(fnorm + b, ff);
 }
 
-// Float-float form of the four weights of a plan entry (same 32 bytes as
-// the FP64 form), for the mixed-precision set-up.
-struct alignas(32) FF4 {
-  float2 w[4];
+// Plan entry of the mixed-precision set-up: the first pixel on each of the two
+// rings (the second one follows it, or with kWrap set begins the ring; indices
+// stay below 2^30 up to nside 8192), the positions fa, fb between them and w
+// between the rings as float-float pairs.  Entries that need the 8-pixel polar
+// stencil have pa = -1 and (theta, phi) in FP64 in fa, fb.  32 bytes in one load;
+// four indices and four weights took 48.
+struct alignas(32) PlanFF {
+  float2 fa, fb, w;
+  int pa, pb;
 };
+constexpr int kWrap = 1 << 30;
 
 // Interpolation plan of one map for the positions of a patch level: either
-// all (n+2)^2 positions (ring = 1) or the n^2 interior cells (ring = 0).
-// ffw: weights stored as float-float pairs.  Entries that need the 8-pixel
-// polar stencil keep (theta, phi) in FP64 with index -1.
+// all (n+2)^2 positions (ring = 1) or the n^2 interior cells (ring = 0).  Four
+// indices and FP64 weights, or (idx null) PlanFF entries in w.  Entries that
+// need the 8-pixel polar stencil keep (theta, phi) in FP64 with index -1.
 __global__ void k_mg_plan(int n, int ring, const double* __restrict__ rot, const double* __restrict__ pvec, int nside,
-                          const double* __restrict__ ring_th, int ffw, int4* __restrict__ idx,
+                          const double* __restrict__ ring_th, int4* __restrict__ idx,
                           double4_32a* __restrict__ w) {
   const int b = blockIdx.z;
   const int side = n + 2;
@@ -208,20 +214,32 @@ __global__ void k_mg_plan(int n, int ring, const double* __restrict__ rot, const
   cell_angles(rot + 9 * (size_t)b, pvec + 3 * (size_t)cell, &th, &ph);
   const Interp8 o = interp_weights_tab(nside, ring_th, th, ph);
   const size_t pos = (size_t)b * m * m + (size_t)k1 * m + k2;
-  if (o.w[4] != 0.0 || o.w[5] != 0.0) {
+  const bool polar = o.w[4] != 0.0 || o.w[5] != 0.0;
+  if (!idx) {
+    PlanFF q{};
+    q.pa = -1;
+    if (polar) {
+      *reinterpret_cast<double*>(&q.fa) = th;
+      *reinterpret_cast<double*>(&q.fb) = ph;
+    } else {
+      // fractions back from the weights (1 - w)(1 - fa), (1 - w) fa, w (1 - fb), w fb
+      const double wa = o.w[0] + o.w[1], wb = o.w[2] + o.w[3];
+      q.pa = (int)o.p[0] | (o.p[1] != o.p[0] + 1 ? kWrap : 0);
+      q.pb = (int)o.p[2] | (o.p[3] != o.p[2] + 1 ? kWrap : 0);
+      q.fa = from_double<float2>(wa > 0.0 ? o.w[1] / wa : 0.0);
+      q.fb = from_double<float2>(wb > 0.0 ? o.w[3] / wb : 0.0);
+      q.w = from_double<float2>(wb);
+    }
+    reinterpret_cast<PlanFF*>(w)[pos] = q;
+    return;
+  }
+  if (polar) {
     idx[pos] = make_int4(-1, 0, 0, 0);
     w[pos] = double4_32a{th, ph, 0.0, 0.0};
     return;
   }
   idx[pos] = make_int4((int)o.p[0], (int)o.p[1], (int)o.p[2], (int)o.p[3]);
-  if (ffw) {
-    FF4 q;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) q.w[k] = from_double<float2>(o.w[k]);
-    reinterpret_cast<FF4*>(w)[pos] = q;
-  } else {
-    w[pos] = double4_32a{o.w[0], o.w[1], o.w[2], o.w[3]};
-  }
+  w[pos] = double4_32a{o.w[0], o.w[1], o.w[2], o.w[3]};
 }
 
 // FP64 map -> float-float pairs
@@ -230,64 +248,123 @@ __global__ void k_split_ff(const double* __restrict__ src, float2* __restrict__ 
     dst[k] = from_double<float2>(src[k]);
 }
 
-// plan interpolation in float-float arithmetic (FP32 pipe); polar entries in FP64
-__device__ __forceinline__ float2 apply_plan_ff(const float2* __restrict__ map_ff, const double* __restrict__ map,
-                                                int nside, const double* __restrict__ ring_th, int4 ix,
-                                                const double4_32a* __restrict__ wp, size_t pos) {
-  if (ix.x < 0) {
-    const double4_32a w = wp[pos];
-    return from_double<float2>(interp_map_tab(map, nside, ring_th, w.x, w.y));
+// Plan interpolation of kRows positions in float-float arithmetic (FP32 pipe):
+// all entries, then all pixels are in flight before the first use (one position
+// after the other, each behind the branch to the FP64 form, waits twice for
+// memory per position); entries with pa < 0 in FP64 at the end.  Bound by
+// instructions in flight (IPC 1.9, a quarter of the warps): two positions at a
+// time leave more warps than four and wait less than one (defect 3033, 3616,
+// 3451 us at Nside 1024, 201M cells), and sums with one two-sum, accurate
+// relative to their terms, take a third of the instructions out.  Base and
+// defect: 2500 + 3039 us with 48-byte entries of four weights, full sums and
+// one position at a time, 2097 + 2790 us now.
+template <int kRows>
+__device__ __forceinline__ void apply_plan_ff(const float2* __restrict__ map_ff, const double* __restrict__ map,
+                                              int nside, const double* __restrict__ ring_th,
+                                              const PlanFF* __restrict__ plan, const size_t pos[kRows],
+                                              const bool ok[kRows], float2 v[kRows]) {
+  double4_32a r[kRows];
+  float2 m[kRows][4];
+#pragma unroll
+  for (int k = 0; k < kRows; ++k)
+    r[k] = ok[k] ? reinterpret_cast<const double4_32a*>(plan)[pos[k]] : double4_32a{0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int k = 0; k < kRows; ++k) {
+    int pa = max(__double2loint(r[k].w), 0), pb = __double2hiint(r[k].w), pa1 = pa + 1, pb1 = pb + 1;
+    if ((pa | pb) & kWrap) {
+      int64_t ja, jb;
+      if (pa & kWrap) { pa ^= kWrap; pix2ring(nside, pa, &ja); pa1 = pa - (int)ja; }
+      if (pb & kWrap) { pb ^= kWrap; pix2ring(nside, pb, &jb); pb1 = pb - (int)jb; }
+    }
+    m[k][0] = map_ff[pa];
+    m[k][1] = map_ff[pa1];
+    m[k][2] = map_ff[pb];
+    m[k][3] = map_ff[pb1];
   }
-  const FF4 q = reinterpret_cast<const FF4*>(wp)[pos];
-  float2 v = ff_mul(q.w[0], map_ff[ix.x]);
-  v = ff_add(v, ff_mul(q.w[1], map_ff[ix.y]));
-  v = ff_add(v, ff_mul(q.w[2], map_ff[ix.z]));
-  return ff_add(v, ff_mul(q.w[3], map_ff[ix.w]));
+  auto ff = [](double x) { return make_float2(__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x))); };
+  bool general = false;
+#pragma unroll
+  for (int k = 0; k < kRows; ++k) {
+    const float2 a = ff_add_lite(m[k][0], ff_mul(ff(r[k].x), ff_add_lite(m[k][1], ff_neg(m[k][0]))));
+    const float2 b = ff_add_lite(m[k][2], ff_mul(ff(r[k].y), ff_add_lite(m[k][3], ff_neg(m[k][2]))));
+    v[k] = ff_add_lite(a, ff_mul(ff(r[k].z), ff_add_lite(b, ff_neg(a))));
+    general |= __double2loint(r[k].w) < 0;
+  }
+  if (general) {
+#pragma unroll
+    for (int k = 0; k < kRows; ++k)
+      if (__double2loint(r[k].w) < 0) v[k] = from_double<float2>(interp_map_tab(map, nside, ring_th, r[k].x, r[k].y));
+  }
 }
+
+// Rows per thread of the set-up kernels: kPlanRows at a time, kSetupRows in all.
+constexpr int kPlanRows = 2, kSetupRows = 8;
 
 // Mixed set-up, float-float: base = psi_SHT interpolated (2 psi_SHT on the
 // ghost ring), kept both as float-float pairs and as their FP64 sum.
-// Rows per thread of the defect set-up (independent kappa gathers in flight).
-constexpr int kSetupRows = 8;
-
-__global__ void k_mg_setup_base_ff(int n, const int4* __restrict__ idx, const double4_32a* __restrict__ w,
-                                   const float2* __restrict__ psi_ff, const double* __restrict__ psi, int ns,
-                                   const double* __restrict__ ring_th, float2* __restrict__ base_ff,
-                                   double* __restrict__ base) {
-  const int b = blockIdx.z;
-  const int k1 = blockIdx.y * kBY + threadIdx.y, k2 = blockIdx.x * kBX + threadIdx.x;
-  const int side = n + 2;
-  if (k1 >= side || k2 >= side) return;
-  const size_t pos = (size_t)b * side * side + (size_t)k1 * side + k2;
-  float2 v = apply_plan_ff(psi_ff, psi, ns, ring_th, idx[pos], w, pos);
-  if (k1 == 0 || k2 == 0 || k1 == n + 1 || k2 == n + 1) v = make_float2(2.f * v.x, 2.f * v.y);
-  base_ff[pos] = v;
-  base[pos] = f2d_exact(v.x) + f2d_exact(v.y);
+__global__ void k_mg_setup_base_ff(int n, const PlanFF* __restrict__ plan, const float2* __restrict__ psi_ff,
+                                   const double* __restrict__ psi, int ns, const double* __restrict__ ring_th,
+                                   float2* __restrict__ base_ff, double* __restrict__ base) {
+  const int b = blockIdx.z, side = n + 2;
+  const int k2 = blockIdx.x * kBX + threadIdx.x, k0 = (blockIdx.y * kBY + threadIdx.y) * kPlanRows;
+  size_t pos[kPlanRows];
+  bool ok[kPlanRows];
+  float2 v[kPlanRows];
+#pragma unroll
+  for (int k = 0; k < kPlanRows; ++k) {
+    ok[k] = k0 + k < side && k2 < side;
+    pos[k] = (size_t)b * side * side + (size_t)(k0 + k) * side + k2;
+  }
+  apply_plan_ff<kPlanRows>(psi_ff, psi, ns, ring_th, plan, pos, ok, v);
+#pragma unroll
+  for (int k = 0; k < kPlanRows; ++k) {
+    if (!ok[k]) continue;
+    const int k1 = k0 + k;
+    if (k1 == 0 || k2 == 0 || k1 == n + 1 || k2 == n + 1) v[k] = make_float2(2.f * v[k].x, 2.f * v[k].y);
+    base_ff[pos[k]] = v[k];
+    base[pos[k]] = f2d_exact(v[k].x) + f2d_exact(v[k].y);
+  }
 }
 
 // Mixed set-up, float-float: defect source f' = kappa - L base at the cells,
-// ||kappa||^2 per patch.
-__global__ void k_mg_setup_defect_ff(int n, const int4* __restrict__ idx, const double4_32a* __restrict__ w,
-                                     const float2* __restrict__ kap_ff, const double* __restrict__ kappa, int nf,
-                                     const double* __restrict__ ring_th, const float2* __restrict__ base_ff,
-                                     const float2* __restrict__ coef, const float2* __restrict__ diag,
-                                     float2* __restrict__ f, double* __restrict__ fnorm) {
-  const int b = blockIdx.z;
-  const int j = blockIdx.x * kBX + threadIdx.x;
-  const int side = n + 2;
+// ||kappa||^2 per patch.  A thread walks consecutive rows: the rows of base
+// above and below a cell stay in registers.
+__global__ void k_mg_setup_defect_ff(int n, const PlanFF* __restrict__ plan, const float2* __restrict__ kap_ff,
+                                     const double* __restrict__ kappa, int nf, const double* __restrict__ ring_th,
+                                     const float2* __restrict__ base_ff, const float2* __restrict__ coef,
+                                     const float2* __restrict__ diag, float2* __restrict__ f,
+                                     double* __restrict__ fnorm) {
+  const int b = blockIdx.z, side = n + 2;
+  const int j = blockIdx.x * kBX + threadIdx.x, i0 = (blockIdx.y * kBY + threadIdx.y) * kSetupRows;
   float ff = 0.f;
+  if (i0 < n && j < n) {
+    const float2* U = base_ff + (size_t)b * side * side + (size_t)(i0 + 1) * side + (j + 1);
+    float2 un = U[-side], uc = U[0];
+    for (int c = 0; c < kSetupRows && i0 + c < n; c += kPlanRows) {
+      size_t pos[kPlanRows];
+      bool ok[kPlanRows];
+      float2 src[kPlanRows];
 #pragma unroll
-  for (int kr = 0; kr < kSetupRows; ++kr) {
-    const int i = (blockIdx.y * kSetupRows + kr) * kBY + threadIdx.y;
-    if (i >= n || j >= n) continue;
-    const size_t pos = (size_t)b * n * n + (size_t)i * n + j;
-    const float2 src = apply_plan_ff(kap_ff, kappa, nf, ring_th, idx[pos], w, pos);
-    const float2* U = base_ff + (size_t)b * side * side + (size_t)(i + 1) * side + (j + 1);
-    // L base = aS uS + aN uN + b (uE + uW) - diag uC
-    const float2 nb = ff_add(ff_add(ff_mul(coef[i], U[side]), ff_mul(coef[n + i], U[-side])),
-                             ff_add(ff_mul(coef[2 * n + i], ff_add(U[1], U[-1])), ff_neg(ff_mul(diag[i * n + j], U[0]))));
-    f[(size_t)b * n * n + fidx(n, i, j)] = ff_add(src, ff_neg(nb));
-    ff = fmaf(src.x, src.x, ff);
+      for (int k = 0; k < kPlanRows; ++k) {
+        ok[k] = i0 + c + k < n;
+        pos[k] = (size_t)b * n * n + (size_t)(i0 + c + k) * n + j;
+      }
+      apply_plan_ff<kPlanRows>(kap_ff, kappa, nf, ring_th, plan, pos, ok, src);
+#pragma unroll
+      for (int k = 0; k < kPlanRows; ++k) {
+        if (!ok[k]) continue;
+        const int i = i0 + c + k;
+        const float2* u = U + (size_t)(c + k) * side;
+        const float2 us = u[side];
+        // L base = aS uS + aN uN + b (uE + uW) - diag uC
+        const float2 nb = ff_add(ff_add(ff_mul(coef[i], us), ff_mul(coef[n + i], un)),
+                                 ff_add(ff_mul(coef[2 * n + i], ff_add(u[1], u[-1])), ff_neg(ff_mul(diag[i * n + j], uc))));
+        f[(size_t)b * n * n + fidx(n, i, j)] = ff_add(src[k], ff_neg(nb));
+        ff = fmaf(src[k].x, src[k].x, ff);
+        un = uc;
+        uc = us;
+      }
+    }
   }
   for (int o = 16; o > 0; o >>= 1) ff += __shfl_xor_sync(0xffffffffu, ff, o);
   if (threadIdx.x == 0 && ff != 0.f) atomicAdd(fnorm + b, (double)ff);
@@ -2555,15 +2632,14 @@ struct MG {
                (float2*)s->psi_ff.p, ns2);
     CLC_LAUNCH(ctx, "k_split_ff", k_split_ff, blocks_for(ctx, nf2, 256), 256, 0, kappa_fine, (float2*)s->kap_ff.p,
                nf2);
-    const dim3 gb = grid3(n + 2, n + 2, s->npatch);
+    const dim3 gb((n + 2 + kBX - 1) / kBX, (n + 2 + kBY * kPlanRows - 1) / (kBY * kPlanRows), s->npatch);
     const dim3 gd((n + kBX - 1) / kBX, (n + kBY * kSetupRows - 1) / (kBY * kSetupRows), s->npatch);
     CLC_LAUNCH(ctx, "k_mg_setup_base", k_mg_setup_base_ff, gb, blk, 0, n,
-               (const int4*)s->plan_psi_idx.p, (const double4_32a*)s->plan_psi_w.p, (const float2*)s->psi_ff.p,
-               (const double*)s->psi_sht.p, s->p.nside_sht, (const double*)s->ring_th_sht.p, (float2*)s->base_ff.p,
+               (const PlanFF*)s->plan_psi_w.p, (const float2*)s->psi_ff.p, (const double*)s->psi_sht.p,
+               s->p.nside_sht, (const double*)s->ring_th_sht.p, (float2*)s->base_ff.p,
                (double*)s->base.p);
     CLC_LAUNCH(ctx, "k_mg_setup_defect", k_mg_setup_defect_ff, gd, blk, 0, n,
-               (const int4*)s->plan_kap_idx.p, (const double4_32a*)s->plan_kap_w.p, (const float2*)s->kap_ff.p,
-               kappa_fine, s->nside_fine, (const double*)s->ring_th_fine.p, (const float2*)s->base_ff.p,
+               (const PlanFF*)s->plan_kap_w.p, (const float2*)s->kap_ff.p, kappa_fine, s->nside_fine, (const double*)s->ring_th_fine.p, (const float2*)s->base_ff.p,
                (const float2*)s->coef_ff.p, (const float2*)s->diag_ff.p, (float2*)s->fd64.p, (double*)s->fnorm.p);
     cudaMemsetAsync(s->e64.p, 0, s->e64.bytes, ctx->stream);
     return launch_check(ctx, "MG set-up (float-float)");
@@ -3035,23 +3111,24 @@ static int solution_create(clc_ctx* ctx, int nf, const clc_mg_params* p, const i
   // interpolation plans, if they fit with 4 GiB to spare
   {
     const size_t pr = (size_t)s->npatch * (n0 + 2) * (n0 + 2), pk = (size_t)s->npatch * n0 * n0;
-    const size_t bytes = (pr + pk) * (sizeof(int4) + 4 * sizeof(double));
+    const bool mx = p->precision == CLC_MIXED;
+    const size_t idx_bytes = mx ? 0 : sizeof(int4);   // PlanFF entries hold their indices
+    const size_t bytes = (pr + pk) * (idx_bytes + 4 * sizeof(double));
     size_t fb = 0, tb = 0;
     cudaMemGetInfo(&fb, &tb);
-    const bool mx = p->precision == CLC_MIXED;
     const int64_t ns2 = 12ll * p->nside_sht * p->nside_sht, nf2 = 12ll * nf * nf;
     const size_t ffb = mx ? (pr + ns2 + nf2) * sizeof(float2) : 0;   // base, psi and kappa as float-float
-    if (bytes + ffb + (4ull << 30) < fb && alloc(s->plan_psi_idx, pr * sizeof(int4)) &&
-        alloc(s->plan_psi_w, pr * 4 * sizeof(double)) && alloc(s->plan_kap_idx, pk * sizeof(int4)) &&
-        alloc(s->plan_kap_w, pk * 4 * sizeof(double)) &&
+    if (bytes + ffb + (4ull << 30) < fb &&
+        (mx || (alloc(s->plan_psi_idx, pr * sizeof(int4)) && alloc(s->plan_kap_idx, pk * sizeof(int4)))) &&
+        alloc(s->plan_psi_w, pr * 4 * sizeof(double)) && alloc(s->plan_kap_w, pk * 4 * sizeof(double)) &&
         (!mx || (alloc(s->base_ff, pr * sizeof(float2)) && alloc(s->psi_ff, ns2 * sizeof(float2)) &&
                  alloc(s->kap_ff, nf2 * sizeof(float2))))) {
       const dim3 blk(kBX, kBY);
       CLC_LAUNCH(ctx, "k_mg_plan", k_mg_plan, grid3(n0 + 2, n0 + 2, s->npatch), blk, 0, (int)n0, 1,
                  (const double*)s->rot.p, (const double*)s->pvec.p, p->nside_sht, (const double*)s->ring_th_sht.p,
-                 (int)mx, (int4*)s->plan_psi_idx.p, (double4_32a*)s->plan_psi_w.p);
+                 (int4*)s->plan_psi_idx.p, (double4_32a*)s->plan_psi_w.p);
       CLC_LAUNCH(ctx, "k_mg_plan", k_mg_plan, grid3(n0, n0, s->npatch), blk, 0, (int)n0, 0, (const double*)s->rot.p,
-                 (const double*)s->pvec.p, nf, (const double*)s->ring_th_fine.p, (int)mx, (int4*)s->plan_kap_idx.p,
+                 (const double*)s->pvec.p, nf, (const double*)s->ring_th_fine.p, (int4*)s->plan_kap_idx.p,
                  (double4_32a*)s->plan_kap_w.p);
       s->plan = true;
     }
