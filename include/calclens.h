@@ -221,7 +221,7 @@ int clc_poisson_sht_batch(clc_ctx* ctx, const double* const* kappa, int nplanes,
  * FFTs) whose work lists span all sizes.  flags: CLC_PLAN_GRAPH captures the
  * six launches in a CUDA graph on the first execution and replays it;
  * CLC_PLAN_TUNE times candidate launch shapes (pipeline depth, resident CTAs
- * per SM) on the first execution and keeps the fastest.  The plan owns its
+ * per SM, blocks per SM of the FFT grids) on the first execution and keeps the fastest.  The plan owns its
  * intermediate buffers (device memory, freed by clc_sht_plan_destroy) and the
  * shared FP16 tables stay cached in the context.  Errors: CLC_EINVAL for
  * sizes outside the limits, CLC_ENOMEM if the tables or buffers do not fit. */
@@ -237,7 +237,7 @@ int clc_sht_plan_create(clc_ctx* ctx, int nplanes, const int* nside_host, const 
 int clc_sht_plan_execute(clc_sht_plan* plan, const double* const* kappa, double* const* psi,
                          const clc_derivs* out);
 /* Launch shapes in use (5 ints: analysis stages, analysis CTAs/SM, synthesis
- * stages, synthesis CTAs/SM, FFT CTAs/SM), the tuned time of each of the six
+ * stages, synthesis CTAs/SM, FFT blocks/SM of the grid), the tuned time of each of the six
  * launches in ms (0 before tuning), and the device bytes the plan uses
  * (buffers plus its share of cached tables).  Any output may be NULL. */
 int clc_sht_plan_info(const clc_sht_plan* plan, int* shape5, double* stage_ms6, size_t* device_bytes);

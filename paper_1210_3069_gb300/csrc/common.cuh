@@ -348,20 +348,6 @@ __device__ __forceinline__ float ring_coord32(int nside, float th) {
   return n * (2.f - 1.5f * z);
 }
 
-// continuous ring coordinate of z (ring i at z_i gives i)
-__device__ __forceinline__ double ring_coord(int nside, double z) {
-  const double n = nside;
-  if (z > 2.0 / 3.0) return n * sqrt(3.0 * (1.0 - z));
-  if (z < -2.0 / 3.0) return 4.0 * n - n * sqrt(3.0 * (1.0 + z));
-  return n * (2.0 - 1.5 * z);
-}
-
-// theta of ring i
-__device__ __forceinline__ double ring_theta(int nside, int i) {
-  const Ring r = ring_geom(nside, i);
-  return atan2(r.s, r.z);
-}
-
 // Continuous ring coordinate of colatitude theta (cos z, sin s): ring centres
 // sit at integers 1 .. 4 nside - 1; used to find the bracketing rings.
 __device__ __forceinline__ int ring_above(int nside, double z, double s) {
@@ -397,75 +383,11 @@ __device__ __forceinline__ void ring_pair_of(const Ring& r, double phi, int64_t*
   *p1 = r.first + (j + 1 == r.npix ? 0 : j + 1);
 }
 
-__device__ __forceinline__ Interp8 interp_weights(int nside, double theta, double phi) {
-  Interp8 o;
-  const double z = cos(theta);
-  int i1 = ring_above(nside, z, 0.0);
-  const int nr = 4 * nside - 1;
-  // ring_above is exact up to rounding; settle the bracket on ring colatitudes
-  // (each ring's geometry and colatitude is formed once)
-  Ring ra{}, rb{};
-  double ta = -1.0, tb = 4.0;   // ring i1 (0: above the first), ring i1 + 1
-  if (i1 >= 1) {
-    ra = ring_geom(nside, i1);
-    ta = atan2(ra.s, ra.z);
-  }
-  if (i1 + 1 <= nr) {
-    rb = ring_geom(nside, i1 + 1);
-    tb = atan2(rb.s, rb.z);
-  }
-  while (i1 >= 1 && ta > theta) {
-    --i1;
-    rb = ra;
-    tb = ta;
-    ta = -1.0;
-    if (i1 >= 1) {
-      ra = ring_geom(nside, i1);
-      ta = atan2(ra.s, ra.z);
-    }
-  }
-  while (i1 + 1 <= nr && tb <= theta) {
-    ++i1;
-    ra = rb;
-    ta = tb;
-    tb = 4.0;
-    if (i1 + 1 <= nr) {
-      rb = ring_geom(nside, i1 + 1);
-      tb = atan2(rb.s, rb.z);
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < 8; ++k) { o.p[k] = 0; o.w[k] = 0.0; }
-  if (i1 == 0 || i1 == nr) {
-    const Ring r = i1 == 0 ? rb : ra;
-    const double tr = i1 == 0 ? tb : ta;
-    const double w = (i1 == 0) ? theta / tr : (kPi - theta) / (kPi - tr);
-    int64_t a0, a1;
-    double fa;
-    ring_pair_of(r, phi, &a0, &a1, &fa);
-    o.p[0] = a0; o.w[0] = w * (1.0 - fa);
-    o.p[1] = a1; o.w[1] = w * fa;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) { o.p[4 + k] = r.first + k; o.w[4 + k] = (1.0 - w) * 0.25; }
-    return o;
-  }
-  const double w = (theta - ta) / (tb - ta);
-  int64_t a0, a1, b0, b1;
-  double fa, fb;
-  ring_pair_of(ra, phi, &a0, &a1, &fa);
-  ring_pair_of(rb, phi, &b0, &b1, &fb);
-  o.p[0] = a0; o.w[0] = (1.0 - w) * (1.0 - fa);
-  o.p[1] = a1; o.w[1] = (1.0 - w) * fa;
-  o.p[2] = b0; o.w[2] = w * (1.0 - fb);
-  o.p[3] = b1; o.w[3] = w * fb;
-  return o;
-}
-
 __device__ __forceinline__ void ring_pair(int nside, int i, double phi, int64_t* p0, int64_t* p1, double* f) {
   ring_pair_of(ring_geom(nside, i), phi, p0, p1, f);
 }
 
-// Same interpolation with the ring colatitudes taken from a table
+// Its weights, with the ring colatitudes taken from a table
 // (ring_th[i - 1] = theta of ring i).
 __device__ __forceinline__ Interp8 interp_weights_tab(int nside, const double* __restrict__ ring_th, double theta,
                                                      double phi) {

@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(128) k_find_images(const double* __restrict__ 
       load3(x, npx, pk, xr);
       normalize3(xr, xn);
       tangent_basis(xn, t0, p0);
-      // the transport's plane rotation (transport_q without its axis)
+      // the transport's plane rotation (without its axis)
       const double wq = dot3(ni, t0) / (1.0 + dot3(xn, ni));
       const double q0 = dot3(t1, t0) - wq * dot3(t1, xn), q1 = dot3(p1, t0) - wq * dot3(p1, xn);
       const double Q[4] = {q0, -q1, q1, q0};

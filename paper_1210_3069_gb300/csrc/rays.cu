@@ -147,8 +147,7 @@ __device__ __forceinline__ void rotate_by_deflection(const double be[3], const d
 // orthogonal to n0 to v - ((n1 . v) / (1 + n0 . n1)) (n0 + n1); with
 // t1 . n1 = p1 . n1 = 0 the change of basis is the plane rotation
 // [[q0, -q1], [q1, q0]], q0 = t1 . t0 - (n1 . t0)(t1 . n0) / (1 + c),
-// q1 = p1 . t0 - (n1 . t0)(p1 . n0) / (1 + c).  (The same Q as transport_q,
-// without the normalised axis.)
+// q1 = p1 . t0 - (n1 . t0)(p1 . n0) / (1 + c), with no normalised axis.
 __device__ __forceinline__ void transport_q_closed(const double n0[3], const double t0[3], const double n1[3],
                                                    const double t1[3], const double p1[3], double Q[4]) {
   const double w = dot3(n1, t0) / (1.0 + dot3(n0, n1));

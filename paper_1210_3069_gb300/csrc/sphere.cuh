@@ -31,42 +31,6 @@ __device__ __forceinline__ double dot3(const double a[3], const double b[3]) {
   return a[0] * b[0] + a[1] * b[1] + a[2] * b[2];
 }
 
-// rotate v about unit axis k by the angle with cosine c, sine s
-__device__ __forceinline__ void rodrigues(const double v[3], const double k[3], double c, double s, double o[3]) {
-  double kv[3];
-  cross3(k, v, kv);
-  const double kd = dot3(k, v) * (1.0 - c);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) o[i] = v[i] * c + kv[i] * s + k[i] * kd;
-}
-
-// Transport matrix Q (2x2) from the basis (t0, p0) at n0 to the basis at n1
-// along the great circle: the rotation R taking n0 to n1 maps (t0, p0, n0)
-// to the right-handed frame (R t0, n1 x R t0, n1) of the tangent plane at n1,
-// so Q is the plane rotation [[c, -s], [s, c]] with c = t1 . R t0,
-// s = p1 . R t0.
-__device__ __forceinline__ void transport_q(const double n0[3], const double t0[3], const double n1[3],
-                                            double Q[4]) {
-  double cr[3];
-  cross3(n0, n1, cr);
-  const double s2 = dot3(cr, cr);
-  const double c = dot3(n0, n1);
-  double t1[3], p1[3];
-  tangent_basis(n1, t1, p1);
-  double tr[3];
-  if (s2 > 0.0) {
-    const double is = rsqrt(s2), s = s2 * is;
-    const double k[3] = {cr[0] * is, cr[1] * is, cr[2] * is};
-    rodrigues(t0, k, c, s, tr);
-  } else {
-    for (int i = 0; i < 3; ++i) tr[i] = t0[i];
-  }
-  Q[0] = dot3(t1, tr);
-  Q[2] = dot3(p1, tr);
-  Q[1] = -Q[2];
-  Q[3] = Q[0];
-}
-
 // o = Q A Q^T (row-major 2x2)
 __device__ __forceinline__ void qaqt(const double Q[4], const double A[4], double o[4]) {
   const double m0 = Q[0] * A[0] + Q[1] * A[2], m1 = Q[0] * A[1] + Q[1] * A[3];
