@@ -55,8 +55,11 @@ struct clc_ctx {
   std::map<std::pair<int, int>, std::shared_ptr<clc::TcTable>> tc_tables;
   size_t table_budget = 0;  // FP64 Legendre table limit in bytes (0: device memory decides)
   std::map<std::tuple<int, int, int, int>, std::shared_ptr<clc::TcBatch>> tc_batches;
-  // growable scratch buffers, reused across calls on this context's stream
-  clc::Buffer scratch[10];
+  // Growable scratch buffers, reused across calls on this context's stream.  A
+  // buffer that grows is freed first, and a captured graph that uses it is then
+  // stale, so a call shares a slot only with calls of its own kind: 0 - 3, 8, 9
+  // SHT, 4 ray tracing, 5, 12, 13 spectra, 6, 10, 11 image search, 7 sources.
+  clc::Buffer scratch[14];
 };
 
 namespace clc {

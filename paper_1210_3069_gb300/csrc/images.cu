@@ -587,7 +587,7 @@ extern "C" int clc_find_images(clc_ctx* ctx, int nside, const double* x, const d
   auto* bounds = (unsigned*)scratch(ctx, 6, 2 * sizeof(unsigned));
   if (!bounds) return CLC_ENOMEM;
   if (cuda_check(ctx, cudaMemsetAsync(bounds, 0, 2 * sizeof(unsigned), ctx->stream), "memset")) return CLC_ECUDA;
-  float4* u = (float4*)scratch(ctx, 5, (size_t)npx * sizeof(float4));
+  float4* u = (float4*)scratch(ctx, 11, (size_t)npx * sizeof(float4));
   if (!u) return CLC_ENOMEM;
   CLC_LAUNCH(ctx, "k_image_units", k_image_units, (int)std::min<int64_t>((npx + 255) / 256, (int64_t)num_sms(ctx) * 16),
              256, 0, x, npx, u);
@@ -621,7 +621,7 @@ extern "C" int clc_find_images(clc_ctx* ctx, int nside, const double* x, const d
   if (rc) return rc;
   // candidate lists (28 bytes per galaxy) for up to 2^24 galaxies at a time
   const int64_t part = std::min<int64_t>(ngal, (int64_t)1 << 24);
-  auto* cand = (unsigned*)scratch(ctx, 7, (size_t)part * (kCand + 1) * sizeof(unsigned));
+  auto* cand = (unsigned*)scratch(ctx, 10, (size_t)part * (kCand + 1) * sizeof(unsigned));
   if (!cand) return CLC_ENOMEM;
   int* ncand = (int*)(cand + part * kCand);
   for (int64_t m0 = 0; m0 < ngal; m0 += part) {

@@ -164,8 +164,8 @@ static int eb_analysis(clc_ctx* ctx, const double* const* g, int ns, const doubl
   if (rc) return rc;
   const int ldf = 4 * nside - 1;
   const size_t fq = (size_t)ldf * (lmax + 1), Q = (size_t)(lmax + 2) * (lmax + 3) / 2;
-  double2* F = (double2*)scratch(ctx, 0, (2 + ns) * sizeof(double2) * fq);
-  double2* S = (double2*)scratch(ctx, 2, 6 * sizeof(double2) * Q);
+  double2* F = (double2*)scratch(ctx, ns ? 13 : 0, (2 + ns) * sizeof(double2) * fq);
+  double2* S = (double2*)scratch(ctx, 12, 6 * sizeof(double2) * Q);
   if (!F || !S) return CLC_ENOMEM;
   const double w = 4.0 * kPi / (12.0 * (double)nside * nside);
   const double* in[4] = {g[0], g[1], ns > 0 ? s[0] : nullptr, ns > 1 ? s[1] : nullptr};
