@@ -123,6 +123,20 @@ const char* clc_last_error(const clc_ctx* ctx);
 /* Release cached plans and Legendre tables (they are rebuilt on demand). */
 int clc_release_caches(clc_ctx* ctx);
 
+/* Calls under CUDA graph capture: a call whose scratch, plans and tables exist
+ * (the same call ran before at this size) can be captured; binning, smoothing
+ * and ray steps need no such first call.  A captured graph holds pointers to the
+ * caller's arrays and to the context's (and the plane solution's) memory, and
+ * must not be replayed any more
+ *  - after clc_destroy, or clc_solution_destroy of a solution it uses;
+ *  - after clc_release_caches, if it has transforms, spectra or plane solves;
+ *  - after a later call on the same context that needed more scratch than the
+ *    captured one: transforms and solves share theirs; the spectra also have
+ *    their own, and so have the image search and the sources.
+ * Binning, sources (clc_counts_to_kappa, also masked), smoothing and ray steps
+ * are touched by the first rule only.  A program that replays transforms next
+ * to others of larger sizes keeps a context for each. */
+
 /* ------------------------------------------------------------------------ */
 /* Step 1: binning (paper Sec. 3.2 source construction; Sec. 3.1 indexing)   */
 

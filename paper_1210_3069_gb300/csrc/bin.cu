@@ -258,7 +258,8 @@ extern "C" int clc_counts_to_kappa_masked(clc_ctx* ctx, const uint32_t* counts, 
   if (!counts || !covered || !kappa) return set_err(ctx, CLC_EINVAL, "clc_counts_to_kappa_masked: null pointer");
   cudaSetDevice(ctx->device);
   const int64_t npix = 12ll * nside * nside;
-  unsigned long long* sums = (unsigned long long*)scratch(ctx, 7, 2 * sizeof(unsigned long long));
+  // as large as the kappa table in the same slot, so that neither call frees the other's
+  unsigned long long* sums = (unsigned long long*)scratch(ctx, 7, sizeof(double) * kKappaTable);
   if (!sums) return CLC_ENOMEM;
   cudaMemsetAsync(sums, 0, 2 * sizeof(unsigned long long), ctx->stream);
   CLC_LAUNCH(ctx, "k_masked_sums", k_masked_sums, grid_for(ctx, npix, 256), 256, 0, counts, covered, npix, sums);

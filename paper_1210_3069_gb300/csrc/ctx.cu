@@ -126,7 +126,7 @@ extern "C" int clc_release_caches(clc_ctx* ctx) {
   if (!ctx) return CLC_EINVAL;
   cudaStreamSynchronize(ctx->stream);
   ctx->fft_plans.clear();
-  ctx->ring_tables.clear();
+  // ring tables stay (2 MB at nside 8192): captured ray steps and smoothings read them
   ctx->tc_batches.clear();
   ctx->leg_tables.clear();
   ctx->tc_tables.clear();

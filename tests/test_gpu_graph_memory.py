@@ -73,6 +73,7 @@ def test_source_table_outlives_image_search(own):
 
     def call():
         c.counts_to_kappa(counts, 128, 1.0, 1.0, kappa=kappa)
+    c.counts_to_kappa_masked(counts, torch.ones(hp.npix(128), dtype=torch.uint8, device="cuda"), 128, 1.0, kappa=kappa)
     call()
     tab = _captured(stream, call, 0, 2)   # k_kappa_table(nbar, scale, tab)
     x = hp.pix2vec_ring(16, torch.arange(hp.npix(16))).T.contiguous().cuda()
@@ -102,3 +103,22 @@ def test_transform_buffers_outlive_spectra(own):
     stream.synchronize()
     for call, arg, ptr in held:
         assert _live(ptr) and _captured(stream, call, 0, arg) == ptr
+
+
+def test_ring_table_outlives_release_caches(own):
+    c, stream = own
+    z = torch.linspace(-1.0, 1.0, 100, dtype=F64, device="cuda")
+    rho = torch.zeros(hp.npix(32), dtype=F64, device="cuda")
+
+    def smooth():
+        c.smooth_particles(z, z.abs(), 32, 0.1, rho=rho)
+    rs = c.rays(hp.npix(32))
+    c.rays_init_pixels(rs, 32, 2.0)
+    maps = {k: torch.zeros(hp.npix(32), dtype=F64, device="cuda") for k in ("a_th", "a_ph", "u_tt", "u_pp", "u_tp")}
+
+    def step():
+        c.ray_step(rs, 1.0, 2.0, 3.0, maps=maps, nside_maps=32)
+    # k_smooth_particles(z, phi, sig_each, n, nside, sigma, rings, map), k_ray_step(R, V, M, nside_maps, rings, sc)
+    held = [_captured(stream, smooth, 0, 6), _captured(stream, step, 0, 4)]
+    c.release_caches()
+    assert all(_live(p) for p in held)
