@@ -25,8 +25,6 @@
 namespace clc {
 
 constexpr int kSmoothThreads = 128;
-constexpr int kSmoothCache = 32;   // weights kept per particle
-constexpr int kSmoothRings = 9;    // rings kept per particle
 
 // theta^2 from the chord c^2 of two unit vectors, 4 asin^2(c / 2): the Taylor
 // series of asin^2 (through c^6 for c^2 <= 1e-5, through c^14 for c^2 <= 1/400:
@@ -80,9 +78,16 @@ struct RingReach {
   float span;
 };
 
-__device__ __forceinline__ bool ring_reach(const Particle& q, const RingS& R, RingReach& o) {
+__device__ __forceinline__ double ring_a(const Particle& q, const RingS& R) {
   const double ds = R.r.s - q.sp, dz = R.r.z - q.zp;
-  o.a = fma(ds, ds, dz * dz);
+  return fma(ds, ds, dz * dz);
+}
+__device__ __forceinline__ double ring_x0(const Particle& q, const RingS& R, int jl) {
+  return fma((double)jl, R.half, 0.5 * (R.r.phi0 - q.pp));
+}
+
+__device__ __forceinline__ bool ring_reach(const Particle& q, const RingS& R, RingReach& o) {
+  o.a = ring_a(q, R);
   const double rem = q.c2max - o.a;
   if (!positive(rem) || !(__double2hiint(rem) < 0x7ff00000)) return false;   // every centre is at least that far (or NaN)
   const int np = R.r.npix;
@@ -103,7 +108,7 @@ __device__ __forceinline__ bool ring_reach(const Particle& q, const RingS& R, Ri
       o.span = span + 0.07f / (float)np;
     }
   }
-  o.x0 = fma((double)o.jl, R.half, 0.5 * (R.r.phi0 - q.pp));
+  o.x0 = ring_x0(q, R, o.jl);
   return o.n > 0;
 }
 
@@ -131,13 +136,122 @@ __device__ void kernel_pixels(const Particle& q, const RingS* __restrict__ rings
 // The rings of a particle are set up first and its centres then taken in one
 // loop over all of them: loops ring by ring run, in every ring, as long as the
 // widest of a warp's 32 particles (22 of 32 lanes active).  Particles with more
-// rings or centres than the shared arrays hold go ring by ring, twice.
-struct SmoothShared {
-  double a[kSmoothRings][kSmoothThreads], b[kSmoothRings][kSmoothThreads], x0[kSmoothRings][kSmoothThreads];
-  int ring[kSmoothRings][kSmoothThreads], jl[kSmoothRings][kSmoothThreads], end[kSmoothRings][kSmoothThreads];
-  double w[kSmoothCache][kSmoothThreads];
-};
+// rings or centres than the shared arrays hold go ring by ring, twice, and a
+// warp with both kinds takes both ways.  Two forms of the arrays, three blocks
+// of either on an SM (rings and centres in reach counted at nside 64 and 1024
+// over the whole sphere and close to the poles):
+//   small: 9 rings, 32 centres, ring terms kept (576 bytes a particle): every
+//     particle up to 2.9 pixels (at most 9 and 31; 1 % do not fit at 3.0);
+//   large: 13 rings, 60 centres, ring terms formed again (584 bytes): up to
+//     4.2 pixels (13 and 60; 10 % do not fit at 4.3).
+// With lengths of their own a warp takes the form of its longest.
+// 4e6 uniform particles at nside 1024, sigma 1, 2.5, 3, 3.25, 4 and 6 pixels:
+// 1.12, 3.94, 7.1, 10.3, 15.1 and 184 ms; with the small form alone 1.12, 3.94,
+// 12.2, 102, 52 and 185; with the large one alone 5.4 at 2.5.  Lengths of their
+// own, uniform in 1 .. 4 pixels: 28 ms (the small form alone: 71).
+constexpr int kMaxRings = 13;
 
+template <int kR, int kC, bool kK>
+struct SmoothShared {
+  static_assert(kR <= kMaxRings && kC < 256, "rows and packing");
+  static constexpr int kRings = kR, kCentres = kC;
+  static constexpr bool kKeep = kK;
+  // The two forms' columns of a thread are the same addresses (the integers have
+  // equally many rows in both), so warps of a block may use different forms.
+  int jl[kMaxRings][kSmoothThreads], ring_end[kMaxRings][kSmoothThreads];   // 256 ring + centres up to its end
+  double w[kC][kSmoothThreads];
+  double a[kK ? kR : 0][kSmoothThreads], b[kK ? kR : 0][kSmoothThreads], x0[kK ? kR : 0][kSmoothThreads];
+};
+using SmoothSmall = SmoothShared<9, 32, true>;
+using SmoothLarge = SmoothShared<kMaxRings, 60, false>;
+constexpr double kSmallPixels = 2.9;   // largest sigma of the small form in pixels (square root of their area)
+
+template <typename Sh>
+__device__ __forceinline__ void deposit(const Particle& q, double phi_i, int nside, const RingS* __restrict__ rings,
+                                        double* __restrict__ map, Sh& S) {
+  const int me = threadIdx.x;
+  int nr = 0, nc = 0;
+  float span = 0.f;
+  for (int r = q.i0; r <= q.i1 && nr <= Sh::kRings; ++r) {
+    RingReach o;
+    if (!ring_reach(q, rings[r - 1], o)) continue;
+    if (nr < Sh::kRings && nc + o.n <= Sh::kCentres) {
+      nc += o.n;
+      if constexpr (Sh::kKeep) {
+        S.a[nr][me] = o.a;
+        S.b[nr][me] = o.b;
+        S.x0[nr][me] = o.x0;
+      }
+      S.jl[nr][me] = o.jl;
+      S.ring_end[nr][me] = r << 8 | nc;
+      span = fmaxf(span, o.span);
+    } else {
+      nr = Sh::kRings;   // does not fit
+    }
+    ++nr;
+  }
+  double tot = 0.0;
+  if (nr <= Sh::kRings) {
+    double a = 0.0, b = 0.0, x = 0.0, h = 0.0;
+    int k = 0, end = 0;
+    for (int c = 0; c < nc; ++c) {
+      if (c == end) {
+        const int re = S.ring_end[k][me];
+        const RingS& R = rings[(re >> 8) - 1];
+        if constexpr (Sh::kKeep) {
+          a = S.a[k][me];
+          b = S.b[k][me];
+          x = S.x0[k][me];
+        } else {
+          a = ring_a(q, R);
+          b = R.r.s * q.sp4;
+          x = ring_x0(q, R, S.jl[k][me]);
+        }
+        h = R.half;
+        end = re & 255;
+        ++k;
+      }
+      const double w = weight_at(q, a, b, x, span);
+      x += h;
+      if (positive(w)) tot += w;
+      S.w[c][me] = w;
+    }
+    if (positive(tot)) {
+      const double inv = 1.0 / tot;
+      int j = 0;
+      Ring r{};
+      k = end = 0;
+      for (int c = 0; c < nc; ++c, ++j) {
+        if (c == end) {
+          const int re = S.ring_end[k][me];
+          r = rings[(re >> 8) - 1].r;
+          j = S.jl[k][me];
+          end = re & 255;
+          ++k;
+        }
+        const double w = S.w[c][me];
+        if (positive(w)) atomicAdd(map + wrapped(r, j), w * inv);
+      }
+      return;
+    }
+  } else {
+    kernel_pixels(q, rings, [&](const Ring&, int, double w) {
+      if (positive(w)) tot += w;
+    });
+    if (positive(tot)) {
+      const double inv = 1.0 / tot;
+      kernel_pixels(q, rings, [&](const Ring& r, int j, double w) {
+        if (positive(w)) atomicAdd(map + wrapped(r, j), w * inv);
+      });
+      return;
+    }
+  }
+  atomicAdd(map + ang2pix_ring(nside, q.zp, phi_i), 1.0);
+}
+
+enum { kFormSmall = 0, kFormLarge = 1, kFormWarp = 2 };
+
+template <int kForm>
 __global__ void __launch_bounds__(kSmoothThreads) k_smooth_particles(const double* __restrict__ z,
                                                                      const double* __restrict__ phi,
                                                                      const double* __restrict__ sig_each, int64_t n,
@@ -145,8 +259,6 @@ __global__ void __launch_bounds__(kSmoothThreads) k_smooth_particles(const doubl
                                                                      const RingS* __restrict__ rings,
                                                                      double* __restrict__ map) {
   extern __shared__ __align__(16) unsigned char smem_sm[];
-  SmoothShared& S = *reinterpret_cast<SmoothShared*>(smem_sm);
-  const int me = threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   double sg = sigma, hs = sin(0.5 * sigma), inv_s2 = 1.0 / (sigma * sigma);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -154,7 +266,7 @@ __global__ void __launch_bounds__(kSmoothThreads) k_smooth_particles(const doubl
     q.zp = z[i];
     const double phi_i = phi[i];
     q.pp = phi_i >= 0.0 && phi_i <= 2.0 * kPi ? phi_i : phi_i - 2.0 * kPi * floor(phi_i / (2.0 * kPi));
-    if (sig_each) {
+    if (kForm == kFormWarp) {
       sg = sig_each[i];
       hs = sin(0.5 * sg);
       inv_s2 = 1.0 / (sg * sg);
@@ -168,73 +280,13 @@ __global__ void __launch_bounds__(kSmoothThreads) k_smooth_particles(const doubl
     const float th = atan2f((float)q.sp, (float)q.zp), sf = (float)sg * 1.00001f;
     q.i0 = max(1, (int)ceilf(ring_coord32(nside, fmaxf(0.f, th - sf)) - 0.1f));
     q.i1 = min(4 * nside - 1, (int)floorf(ring_coord32(nside, fminf(3.14159265f, th + sf)) + 0.1f));
-    int nr = 0, nc = 0;
-    float span = 0.f;
-    for (int r = q.i0; r <= q.i1 && nr <= kSmoothRings; ++r) {
-      RingReach o;
-      if (!ring_reach(q, rings[r - 1], o)) continue;
-      if (nr < kSmoothRings && o.n <= kSmoothCache) {
-        nc += o.n;
-        S.a[nr][me] = o.a;
-        S.b[nr][me] = o.b;
-        S.x0[nr][me] = o.x0;
-        S.ring[nr][me] = r;
-        S.jl[nr][me] = o.jl;
-        S.end[nr][me] = nc;
-        span = fmaxf(span, o.span);
-      } else {
-        nr = kSmoothRings;   // does not fit
-      }
-      ++nr;
-    }
-    double tot = 0.0;
-    if (nr <= kSmoothRings && nc <= kSmoothCache) {
-      double a = 0.0, b = 0.0, x = 0.0, h = 0.0;
-      int k = 0, end = 0;
-      for (int c = 0; c < nc; ++c) {
-        if (c == end) {
-          a = S.a[k][me];
-          b = S.b[k][me];
-          x = S.x0[k][me];
-          h = rings[S.ring[k][me] - 1].half;
-          end = S.end[k][me];
-          ++k;
-        }
-        const double w = weight_at(q, a, b, x, span);
-        x += h;
-        if (positive(w)) tot += w;
-        S.w[c][me] = w;
-      }
-      if (positive(tot)) {
-        const double inv = 1.0 / tot;
-        int j = 0;
-        Ring r{};
-        k = end = 0;
-        for (int c = 0; c < nc; ++c, ++j) {
-          if (c == end) {
-            r = rings[S.ring[k][me] - 1].r;
-            j = S.jl[k][me];
-            end = S.end[k][me];
-            ++k;
-          }
-          const double w = S.w[c][me];
-          if (positive(w)) atomicAdd(map + wrapped(r, j), w * inv);
-        }
-        continue;
-      }
-    } else {
-      kernel_pixels(q, rings, [&](const Ring&, int, double w) {
-        if (positive(w)) tot += w;
-      });
-      if (positive(tot)) {
-        const double inv = 1.0 / tot;
-        kernel_pixels(q, rings, [&](const Ring& r, int j, double w) {
-          if (positive(w)) atomicAdd(map + wrapped(r, j), w * inv);
-        });
-        continue;
-      }
-    }
-    atomicAdd(map + ang2pix_ring(nside, q.zp, phi_i), 1.0);
+    bool large = kForm == kFormLarge;
+    if (kForm == kFormWarp)   // (a wrong guess costs time only)
+      large = __any_sync(__activemask(), sf * (float)nside > (float)kSmallPixels * 1.02332671f);
+    if (large)
+      deposit(q, phi_i, nside, rings, map, *reinterpret_cast<SmoothLarge*>(smem_sm));
+    else
+      deposit(q, phi_i, nside, rings, map, *reinterpret_cast<SmoothSmall*>(smem_sm));
   }
 }
 
@@ -254,9 +306,16 @@ extern "C" int clc_smooth_particles(clc_ctx* ctx, const double* z, const double*
   const RingS* rings = get_ring_table(ctx, nside, &rc);
   if (rc) return rc;
   const int64_t blocks = std::min<int64_t>((n + kSmoothThreads - 1) / kSmoothThreads, (int64_t)num_sms(ctx) * 32);
-  const int smem = (int)sizeof(SmoothShared);
-  cudaFuncSetAttribute(k_smooth_particles, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  CLC_LAUNCH(ctx, "k_smooth_particles", k_smooth_particles, (int)blocks, kSmoothThreads, smem, z, phi, sigma_each, n,
-             nside, sigma, rings, map);
+  auto launch = [&](auto kern, size_t smem) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    CLC_LAUNCH(ctx, "k_smooth_particles", kern, (int)blocks, kSmoothThreads, (int)smem, z, phi, sigma_each, n, nside,
+               sigma, rings, map);
+  };
+  if (sigma_each)
+    launch(k_smooth_particles<kFormWarp>, std::max(sizeof(SmoothSmall), sizeof(SmoothLarge)));
+  else if (sigma <= kSmallPixels * std::sqrt(kPi / 3.0) / nside)
+    launch(k_smooth_particles<kFormSmall>, sizeof(SmoothSmall));
+  else
+    launch(k_smooth_particles<kFormLarge>, sizeof(SmoothLarge));
   return launch_check(ctx, "k_smooth_particles");
 }

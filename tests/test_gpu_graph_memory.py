@@ -108,10 +108,11 @@ def test_transform_buffers_outlive_spectra(own):
 def test_ring_table_outlives_release_caches(own):
     c, stream = own
     z = torch.linspace(-1.0, 1.0, 100, dtype=F64, device="cuda")
+    phi = z.abs()
     rho = torch.zeros(hp.npix(32), dtype=F64, device="cuda")
 
     def smooth():
-        c.smooth_particles(z, z.abs(), 32, 0.1, rho=rho)
+        c.smooth_particles(z, phi, 32, 0.1, rho=rho)
     rs = c.rays(hp.npix(32))
     c.rays_init_pixels(rs, 32, 2.0)
     maps = {k: torch.zeros(hp.npix(32), dtype=F64, device="cuda") for k in ("a_th", "a_ph", "u_tt", "u_pp", "u_tp")}
