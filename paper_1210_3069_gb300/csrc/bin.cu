@@ -100,7 +100,6 @@ __global__ void k_bin(const double* __restrict__ z, const double* __restrict__ p
   }
 }
 
-// kappa = scale * (counts / nbar - 1), each operation rounded separately
 // kappa of a pixel with c particles: scale (c / nbar - 1), each operation
 // correctly rounded
 __device__ __forceinline__ double kappa_of(uint32_t c, double nbar, double scale) {
@@ -118,10 +117,15 @@ __global__ void k_kappa_table(double nbar, double scale, double* __restrict__ ta
   if (c < kKappaTable) tab[c] = kappa_of((uint32_t)c, nbar, scale);
 }
 
-// Small maps (kKappaDirect pixels and below) divide: the table would cost a
-// launch and as many divisions.  kWide: four pixels per thread (16-byte loads
-// and stores; npix is a multiple of 4).
+// Maps of kKappaDirect pixels and below divide: at nside 64 the 49152 divisions,
+// one per thread, take 6.3 us, the launch of the table's 4096 and the pass 8.3
+// (launches back to back); at nside 128 12.5 against 8.3.
 constexpr int64_t kKappaDirect = 12 * 64 * 64;
+// kWide: four pixels per thread (16-byte loads and stores; npix is a multiple of
+// 4), for maps of more than kKappaWide pixels, whose 12 bytes per pixel do not
+// stay in L2: 37 instead of 49 us at nside 1024, 125 instead of 165 at 2048.  At
+// nside 512 (counts just written) one pixel per thread takes 12.5 us, four 14.5.
+constexpr int64_t kKappaWide = 12 * 512 * 512;
 
 template <bool kWide>
 __global__ void k_counts_to_kappa(const uint32_t* __restrict__ counts, int64_t npix, double nbar,
@@ -242,7 +246,7 @@ extern "C" int clc_counts_to_kappa(clc_ctx* ctx, const uint32_t* counts, int nsi
     if (!tab) return CLC_ENOMEM;
     CLC_LAUNCH(ctx, "k_counts_to_kappa", k_kappa_table, kKappaTable / 256, 256, 0, nbar, scale, tab);
   }
-  if (((reinterpret_cast<uintptr_t>(counts) | reinterpret_cast<uintptr_t>(kappa)) & 15) == 0)
+  if (npix > kKappaWide && ((reinterpret_cast<uintptr_t>(counts) | reinterpret_cast<uintptr_t>(kappa)) & 15) == 0)
     CLC_LAUNCH(ctx, "k_counts_to_kappa", k_counts_to_kappa<true>, grid_for(ctx, npix / 4, 256), 256, 0, counts, npix,
                nbar, scale, (const double*)tab, kappa);
   else
