@@ -189,12 +189,14 @@ int clc_degrade(clc_ctx* ctx, const double* map_fine, int nside_fine, double* ma
 /* ------------------------------------------------------------------------ */
 /* Step 2: spherical-harmonic transforms and the SHT Poisson solve (Sec. 3.2) */
 
-/* Limit the Legendre table of the FP64 transforms (16 bytes per (l, m, ring)
- * in 64 x 64 blocks, about 0.7 of the sum over m of (lmax + 2 - m) * 2 nside
- * of them: 7 GB at nside 512, lmax 1024) to `bytes` (0 = the free device
- * memory decides).  Larger tables are built and used one order range m0..m1
- * at a time inside each FP64 SHT call (same results; the recurrence is then
- * recomputed per call). */
+/* Limit the Legendre table of the FP64 transforms (16 bytes per (l, m, ring) in
+ * blocks of 64 x 64, less the blocks that vanish next to the poles: 7.8 GB at
+ * nside 512, lmax 1024, at most 73 GB at nside 1024, lmax 2048) to `bytes` (0 =
+ * the free device memory decides).  A table that fits is kept.  One that does not
+ * is built and used one order range m0..m1 at a time inside each FP64 SHT call
+ * (same results; the recurrence is then recomputed per call); if more than half
+ * of it fits the budget, the first orders stay in three quarters of the budget
+ * from the second call on.  While a table is built, up to 2 GiB more are used. */
 int clc_set_table_budget(clc_ctx* ctx, size_t bytes);
 
 /* a_lm = (4 pi / Npix) sum_p map[p] Y*_lm(p) (uniform quadrature). */

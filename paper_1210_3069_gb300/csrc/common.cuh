@@ -51,7 +51,8 @@ struct clc_ctx {
   std::vector<cudaEvent_t> ev_pool;
   std::map<int, std::shared_ptr<clc::FftPlan>> fft_plans;
   std::map<int, std::shared_ptr<clc::Buffer>> ring_tables;   // RingS[4 nside - 1] by nside
-  std::map<std::tuple<int, int, int>, std::shared_ptr<clc::LegendreTable>> leg_tables;
+  std::map<std::pair<int, int>, std::shared_ptr<clc::LegendreTable>> leg_tables;   // orders from 0 on, by (nside, lmax)
+  std::map<std::pair<int, int>, size_t> leg_bytes;   // size of the whole table, once known
   std::map<std::pair<int, int>, std::shared_ptr<clc::TcTable>> tc_tables;
   size_t table_budget = 0;  // FP64 Legendre table limit in bytes (0: device memory decides)
   std::map<std::tuple<int, int, int, int>, std::shared_ptr<clc::TcBatch>> tc_batches;

@@ -238,14 +238,9 @@ __global__ void k_eps_table(int lmax, int m0, double* __restrict__ eps, double* 
 
 static int row_blocks(int lt, int m, int p) { return m + p <= lt ? ((lt - m - p) / 2 + 1 + 63) / 64 : 0; }
 
-size_t legendre_table_bytes(int nside, int lmax, int m0, int m1) {
-  const size_t nkb = (2 * (size_t)nside + 63) / 64;
-  size_t b = 0;
-  for (int m = m0; m < m1; ++m) b += row_blocks(lmax + 1, m, 0) + row_blocks(lmax + 1, m, 1);
-  return b * nkb * kDigits * kAtom * sizeof(__half);
-}
-
 static bool dev_alloc(Buffer& b, size_t bytes) {
+  if (b.p && b.bytes >= bytes) return true;
+  if (b.p) cudaFree(b.p);
   b.bytes = std::max(bytes, (size_t)16);
   if (cudaMalloc(&b.p, b.bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -256,14 +251,17 @@ static bool dev_alloc(Buffer& b, size_t bytes) {
   return true;
 }
 
-int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, LegendreTable* T) {
-  const int lt = lmax + 1, R = 2 * nside, nkb = (R + 63) / 64, nm = m1 - m0, ldc = nkb * 64;
+int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, size_t limit, bool stays, LegendreBuild& W,
+                         LegendreTable* T) {
+  const int lt = lmax + 1, R = 2 * nside, nkb = (R + 63) / 64, ldc = nkb * 64;
+  int nm = m1 - m0;
   T->nside = nside;
   T->lmax = lmax;
   T->R = R;
   T->nkb = nkb;
   T->m0 = m0;
   T->m1 = m1;
+  T->bytes = 0;
   T->h_gidx.assign(2 * nm + 1, 0);
   for (int g = 0; g < 2 * nm; ++g) T->h_gidx[g + 1] = T->h_gidx[g] + row_blocks(lt, m0 + (g >> 1), g & 1);
   const int nblk = T->h_gidx[2 * nm];
@@ -276,46 +274,52 @@ int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, Lege
     if (m > 0) ln += 0.5 * std::log2((2.0 * m + 1.0) / (2.0 * m));
     lognorm[m] = ln;
   }
-  // segments of orders whose FP64 values fit the build buffer
-  std::vector<int> seg{m0};
-  size_t tab_bytes = 0, acc = 0;
-  int seg_orders = 0;
-  for (int m = m0; m < m1; ++m) {
-    const size_t b = (size_t)(lt - m + 1) * R * sizeof(double);
-    if (acc > 0 && acc + b > kSegBytes) {
-      seg.push_back(m);
-      acc = 0;
-    }
-    acc += b;
-    tab_bytes = std::max(tab_bytes, acc);
-    seg_orders = std::max(seg_orders, m - seg.back() + 1);
-  }
-  seg.push_back(m1);
-  Buffer d_tab, d_ab, d_ln, d_off, d_grp;
+  // A segment: orders whose FP64 values fit the build buffer and whose digits
+  // (1.6 times those bytes with the usual polar cut) about fill the limit.
+  auto order_bytes = [&](int m) { return (size_t)(lt - m + 1) * R * sizeof(double); };
+  auto segment_end = [&](int ms) {
+    const size_t room = std::min<size_t>(kSegBytes, (limit - std::min(limit, T->bytes)) / 8 * 5);
+    size_t acc = order_bytes(ms);
+    int me = ms + 1;
+    while (me < m1 && acc + order_bytes(me) <= room) acc += order_bytes(me++);
+    return me;
+  };
+  size_t tab_bytes = 0;
+  for (int m = m0; m < m1 && tab_bytes < kSegBytes; ++m) tab_bytes += order_bytes(m);
+  tab_bytes = std::max(order_bytes(m0), std::min(std::min<size_t>(tab_bytes, kSegBytes), limit / 8 * 5));
   const char* what = "Legendre table allocation failed";
   if (!dev_alloc(T->gidx, sizeof(int) * (2 * nm + 1)) || !dev_alloc(T->rb0, sizeof(int) * nblk) ||
       !dev_alloc(T->abase, sizeof(__half*) * nblk) || !dev_alloc(T->rexp, sizeof(int) * 64 * (size_t)nblk) ||
       !dev_alloc(T->cexp, (size_t)nm * ldc) || !dev_alloc(T->fac, sizeof(double) * 2 * R) ||
       !dev_alloc(T->zero, (size_t)kDigits * kAtom * sizeof(__half)) ||
-      !dev_alloc(T->eps, sizeof(double) * (size_t)(nm + 2) * (lmax + 3)) || !dev_alloc(d_tab, tab_bytes) ||
-      !dev_alloc(d_ab, sizeof(double2) * (size_t)seg_orders * (lt + 1)) ||
-      !dev_alloc(d_ln, sizeof(double) * lognorm.size()) || !dev_alloc(d_off, sizeof(long long) * seg_orders) ||
-      !dev_alloc(d_grp, sizeof(int) * nblk))
+      !dev_alloc(T->eps, sizeof(double) * (size_t)(nm + 2) * (lmax + 3)) || !dev_alloc(W.tab, tab_bytes) ||
+      !dev_alloc(W.ab, sizeof(double2) * (size_t)nm * (lt + 1)) ||
+      !dev_alloc(W.ln, sizeof(double) * lognorm.size()) || !dev_alloc(W.off, sizeof(long long) * nm) ||
+      !dev_alloc(W.grp, sizeof(int) * nblk))
     return set_err(ctx, CLC_ENOMEM, what);
+  if (stays ? !T->atoms.empty() : !T->arena) {
+    if (int e = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "table chunk")) return e;
+    T->atoms.clear();
+  }
+  T->arena = !stays;
+  if (!stays && T->atoms.empty()) {
+    T->atoms.push_back(std::make_unique<Buffer>());
+    if (!dev_alloc(*T->atoms[0], std::min(limit, (size_t)nblk * nkb * kDigits * kAtom * sizeof(__half))))
+      return set_err(ctx, CLC_ENOMEM, what);
+  }
   cudaStream_t st = ctx->stream;
   cudaMemcpyAsync(T->gidx.p, T->h_gidx.data(), sizeof(int) * (2 * nm + 1), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync(T->rb0.p, h_rb0.data(), sizeof(int) * nblk, cudaMemcpyHostToDevice, st);
-  cudaMemcpyAsync(d_ln.p, lognorm.data(), sizeof(double) * lognorm.size(), cudaMemcpyHostToDevice, st);
+  cudaMemcpyAsync(W.ln.p, lognorm.data(), sizeof(double) * lognorm.size(), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(T->rexp.p, 0, T->rexp.bytes, st);
   cudaMemsetAsync(T->cexp.p, 0, T->cexp.bytes, st);
   cudaMemsetAsync(T->zero.p, 0, T->zero.bytes, st);
   CLC_LAUNCH(ctx, "k_ring_factors", k_ring_factors, (R + 127) / 128, 128, 0, nside, (double*)T->fac.p);
-  CLC_LAUNCH(ctx, "k_eps_table", k_eps_table, dim3((lmax + 130) / 128, nm), 128, 0, lmax, m0, (double*)T->eps.p,
-             (double*)T->eps.p + (size_t)nm * (lmax + 3));
   int rc;
-  for (size_t s = 0; s + 1 < seg.size(); ++s) {
-    const int ms = seg[s], me = seg[s + 1], n = me - ms, g0 = 2 * (ms - m0);
-    const int b0 = T->h_gidx[g0], b1 = T->h_gidx[2 * (me - m0)];
+  for (int ms = m0; ms < T->m1;) {
+    int me = segment_end(ms);
+    const int n = me - ms, g0 = 2 * (ms - m0), b0 = T->h_gidx[g0];
+    int b1 = T->h_gidx[2 * (me - m0)];
     std::vector<long long> off(n);
     long long a = 0;
     for (int m = ms; m < me; ++m) {
@@ -325,31 +329,43 @@ int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, Lege
     std::vector<int> grp(std::max(b1 - b0, 1));
     for (int g = 0; g < 2 * n; ++g)
       for (int b = T->h_gidx[g0 + g]; b < T->h_gidx[g0 + g + 1]; ++b) grp[b - b0] = g;
-    cudaMemcpyAsync(d_off.p, off.data(), sizeof(long long) * n, cudaMemcpyHostToDevice, st);
-    cudaMemcpyAsync(d_grp.p, grp.data(), sizeof(int) * (b1 - b0), cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(W.off.p, off.data(), sizeof(long long) * n, cudaMemcpyHostToDevice, st);
+    cudaMemcpyAsync(W.grp.p, grp.data(), sizeof(int) * (b1 - b0), cudaMemcpyHostToDevice, st);
     int8_t* cx = (int8_t*)T->cexp.p + (size_t)(ms - m0) * ldc;
     const int* gx = (const int*)T->gidx.p + g0;
-    CLC_LAUNCH(ctx, "k_legendre_coef", k_legendre_coef, dim3((lt + 128) / 128, n), 128, 0, lt, ms, (double2*)d_ab.p);
+    CLC_LAUNCH(ctx, "k_legendre_coef", k_legendre_coef, dim3((lt + 128) / 128, n), 128, 0, lt, ms, (double2*)W.ab.p);
     CLC_LAUNCH(ctx, "k_legendre_build", k_legendre_build, dim3((R + 127) / 128, n), 128, 0, nside, lmax, R,
-               (const long long*)d_off.p, (const double*)d_ln.p, (const double2*)d_ab.p, (double*)d_tab.p, ms, cx, ldc);
-    CLC_LAUNCH(ctx, "k_dig_rows", k_dig_rows, dim3((lt - ms + 8) / 8, n), 256, 0, lmax, R, ms, (const long long*)d_off.p,
-               (const double*)d_tab.p, (const int8_t*)cx, ldc, gx, (int*)T->rexp.p, (int*)T->rb0.p);
+               (const long long*)W.off.p, (const double*)W.ln.p, (const double2*)W.ab.p, (double*)W.tab.p, ms, cx, ldc);
+    CLC_LAUNCH(ctx, "k_dig_rows", k_dig_rows, dim3((lt - ms + 8) / 8, n), 256, 0, lmax, R, ms, (const long long*)W.off.p,
+               (const double*)W.tab.p, (const int8_t*)cx, ldc, gx, (int*)T->rexp.p, (int*)T->rb0.p);
     if ((rc = launch_check(ctx, "Legendre table rows"))) return rc;
     cudaMemcpyAsync(h_rb0.data() + b0, (const int*)T->rb0.p + b0, sizeof(int) * (b1 - b0), cudaMemcpyDeviceToHost, st);
     if ((rc = cuda_check(ctx, cudaStreamSynchronize(st), "Legendre table rows"))) return rc;
-    // a row block keeps at least the ring blocks of the one before it (lower l)
-    size_t natom = 0;
-    for (int g = 0; g < 2 * n; ++g)
-      for (int b = T->h_gidx[g0 + g]; b < T->h_gidx[g0 + g + 1]; ++b) {
-        if (b > T->h_gidx[g0 + g]) h_rb0[b] = std::min(h_rb0[b], h_rb0[b - 1]);
-        natom += nkb - h_rb0[b];
+    // a row block keeps at least the ring blocks of the one before it (lower l);
+    // the segment ends with the last order that fits the limit
+    size_t bytes = 0;
+    for (int m = ms; m < me; ++m) {
+      size_t natom = 0;
+      for (int g = 2 * (m - m0); g < 2 * (m - m0) + 2; ++g)
+        for (int b = T->h_gidx[g]; b < T->h_gidx[g + 1]; ++b) {
+          if (b > T->h_gidx[g]) h_rb0[b] = std::min(h_rb0[b], h_rb0[b - 1]);
+          natom += nkb - h_rb0[b];
+        }
+      natom *= kDigits * kAtom * sizeof(__half);
+      if (m > m0 && T->bytes + bytes + natom > limit) {
+        T->m1 = me = m;
+        break;
       }
-    auto piece = std::make_unique<Buffer>();
-    const size_t bytes = natom * kDigits * kAtom * sizeof(__half);
-    if (!dev_alloc(*piece, bytes))
+      bytes += natom;
+    }
+    if (me == ms) break;
+    b1 = T->h_gidx[2 * (me - m0)];
+    if (stays) T->atoms.push_back(std::make_unique<Buffer>());
+    Buffer& mem = *T->atoms.back();
+    const size_t at0 = stays ? 0 : T->bytes;
+    if (!dev_alloc(mem, at0 + bytes))   // an arena grows for a first order above the limit only
       return set_err(ctx, CLC_ENOMEM, "Legendre table of " + std::to_string(bytes >> 20) + " MiB does not fit");
-    __half* at = (__half*)piece->p;
-    T->atoms.push_back(std::move(piece));
+    __half* at = (__half*)((uint8_t*)mem.p + at0);
     for (int b = b0; b < b1; ++b) {
       h_abase[b] = at;
       at += (size_t)(nkb - h_rb0[b]) * kDigits * kAtom;
@@ -358,13 +374,21 @@ int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, Lege
     cudaMemcpyAsync((__half**)T->abase.p + b0, h_abase.data() + b0, sizeof(__half*) * (b1 - b0), cudaMemcpyHostToDevice,
                     st);
     if (b1 > b0)
-      CLC_LAUNCH(ctx, "k_dig_fill", k_dig_fill, dim3(b1 - b0, nkb), 256, 0, lmax, R, ms, (const long long*)d_off.p,
-                 (const double*)d_tab.p, (const int8_t*)cx, ldc, gx, (const int*)d_grp.p, (const int*)T->rexp.p,
+      CLC_LAUNCH(ctx, "k_dig_fill", k_dig_fill, dim3(b1 - b0, nkb), 256, 0, lmax, R, ms, (const long long*)W.off.p,
+                 (const double*)W.tab.p, (const int8_t*)cx, ldc, gx, (const int*)W.grp.p, (const int*)T->rexp.p,
                  (const int*)T->rb0.p, (__half* const*)T->abase.p, b0);
     // the host arrays of the segment and the build buffers are reused: wait
     if ((rc = launch_check(ctx, "k_dig_fill"))) return rc;
     if ((rc = cuda_check(ctx, cudaStreamSynchronize(st), "Legendre table build"))) return rc;
+    T->bytes += bytes;
+    ms = me;
+    if (!stays && T->bytes > limit / 8 * 7) T->m1 = me;
   }
+  nm = T->m1 - m0;
+  T->h_gidx.resize(2 * nm + 1);
+  CLC_LAUNCH(ctx, "k_eps_table", k_eps_table, dim3((lmax + 130) / 128, nm), 128, 0, lmax, m0, (double*)T->eps.p,
+             (double*)T->eps.p + (size_t)nm * (lmax + 3));
+  if ((rc = launch_check(ctx, "k_eps_table"))) return rc;
   // work lists.  Analysis: (group, 128-row tile, first ring block); synthesis:
   // (order, 128-ring tile, first row blocks of the two parities).
   std::vector<std::pair<int, int4>> an, sy;
@@ -399,20 +423,6 @@ int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, Lege
   return upload(sy, T->sy, &T->n_sy);
 }
 
-std::shared_ptr<LegendreTable> get_legendre_table(clc_ctx* ctx, int nside, int lmax, int* rc) {
-  const auto key = std::make_tuple(nside, lmax, 0);
-  auto it = ctx->leg_tables.find(key);
-  if (it != ctx->leg_tables.end()) {
-    *rc = CLC_OK;
-    return it->second;
-  }
-  auto T = std::make_shared<LegendreTable>();
-  *rc = build_legendre_table(ctx, nside, lmax, 0, lmax + 1, T.get());
-  if (*rc) return nullptr;
-  ctx->leg_tables[key] = T;
-  return T;
-}
-
 // ---------------------------------------------------------------------------
 // data operands: columns of doubles to digit planes.  Block of 64 terms:
 // kDigits x kCols rows (digit plane j, column c at row j kCols + c) of 64
@@ -421,6 +431,81 @@ std::shared_ptr<LegendreTable> get_legendre_table(clc_ctx* ctx, int nside, int l
 
 constexpr int kCols = 16;                          // real columns of a contraction
 constexpr int kOpBlock = kDigits * kCols * 64;     // halves of a block
+
+static size_t analysis_op_bytes(int nm, int nkb) { return (size_t)2 * nm * nkb * kOpBlock * sizeof(__half); }
+static size_t synthesis_op_bytes(int nblk) { return (size_t)nblk * kOpBlock * sizeof(__half); }
+
+// What a table may take is its budget, or the free memory less the operands, the
+// build buffers and 2 GiB; what it does take is known when its rows are (the
+// atoms below the polar cut are not stored: 7.74 of at most 9.69 GB at nside 512,
+// lmax 1024), so it is built until the limit is reached rather than compared with
+// a bound.  When a pass has shown that the whole table exceeds the budget, and
+// more than half of it fits, the first orders stay in three quarters of the budget
+// and the others are rebuilt in the rest.  Solve with fields at nside 512, lmax
+// 1024: 6.1 ms from 7.8 GB on, 12.7 with 7, 15.5 with 4.6, 21.5 with 3 and 23.3
+// with 0.5 (compared with the bound and with memory of its own for every range:
+// 25.9 with 7.5 and 26.9 with 4.6; the FP64 table before, 4.3 GB, took 19.2 from
+// there on and 33.9 with 3); at nside 2048, lmax 4096: 888 ms (1207; 2172).  A
+// call on a kept table does not ask for the free memory (10 us of a small one).
+int legendre_table_from(clc_ctx* ctx, int nside, int lmax, int m0, LegendreBuild& W,
+                        std::shared_ptr<LegendreTable>& own, std::shared_ptr<LegendreTable>* out) {
+  const std::pair<int, int> key(nside, lmax);
+  const size_t budget = ctx->table_budget;
+  const auto known = ctx->leg_bytes.find(key);
+  const size_t total = known == ctx->leg_bytes.end() ? 0 : known->second;   // 0: not known yet
+  auto it = ctx->leg_tables.find(key);
+  size_t held = 0;
+  if (it != ctx->leg_tables.end() && !(budget && it->second->bytes > budget)) {
+    const LegendreTable& C = *it->second;
+    if (m0 >= C.m1) {
+      held = C.bytes;
+    } else if (C.m1 > lmax || (budget && total > budget)) {
+      *out = it->second;
+      return CLC_OK;
+    } else {   // a part kept under an earlier, smaller budget
+      if (int rc = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "Legendre table")) return rc;
+      ctx->leg_tables.erase(it);
+      it = ctx->leg_tables.end();
+    }
+  }
+  if (own && own->arena) {   // the next range of a pass
+    *out = own;
+    return build_legendre_table(ctx, nside, lmax, m0, lmax + 1, own->atoms[0]->bytes, false, W, own.get());
+  }
+  const bool first = m0 == 0 && it == ctx->leg_tables.end();
+  const int nkb = (2 * nside + 63) / 64;
+  size_t nblk = 0, build = 0, freeb = 0, totalb = 0;
+  for (int m = 0; m <= lmax; ++m) {
+    nblk += row_blocks(lmax + 1, m, 0) + row_blocks(lmax + 1, m, 1);
+    build += (size_t)(lmax + 2 - m) * 2 * nside * sizeof(double);
+  }
+  cudaMemGetInfo(&freeb, &totalb);
+  if (own)   // a first range that did not take every order: its memory is given back
+    for (auto& p : own->atoms) freeb += p->bytes;
+  auto grow = [&](int slot, size_t bytes) { return bytes > ctx->scratch[slot].bytes ? bytes : 0; };
+  const size_t reserve = (2ull << 30) + std::min(build, kSegBytes) + grow(8, analysis_op_bytes(lmax + 1, nkb)) +
+                         grow(9, synthesis_op_bytes((int)nblk));
+  const size_t room = freeb > reserve + reserve / 2 ? freeb - reserve : freeb / 4;
+  size_t limit = std::min<size_t>(room, 48ull << 30);
+  bool stays = false;
+  if (first && total <= (budget ? std::min(budget, room) : room)) {
+    stays = true;
+    limit = budget ? std::min(budget, room) : room;
+  } else if (first && budget > total / 2 && budget <= room) {
+    stays = true;
+    limit = budget - budget / 4;
+  } else if (budget) {
+    limit = std::min(limit, budget - held);
+  }
+  if (!own) own = std::make_shared<LegendreTable>();
+  if (int rc = build_legendre_table(ctx, nside, lmax, m0, lmax + 1, limit, stays, W, own.get())) return rc;
+  *out = own;
+  if (first && stays && (own->m1 > lmax || total > limit)) {
+    ctx->leg_tables[key] = own;
+    own.reset();
+  }
+  return CLC_OK;
+}
 
 // block-wide maxima of four non-negative integers (results in all threads)
 __device__ __forceinline__ void block_max4(int v[4], int* sh) {
@@ -954,7 +1039,7 @@ static DigArgs dig_args(const LegendreTable& T, const __half* op, const int* col
 template <int NC>
 static int analysis_cols(clc_ctx* ctx, const LegendreTable& T, const AnaCols& c, int ldf, double2* const* out, int ltop) {
   const int nm = T.m1 - T.m0;
-  const size_t ob = (size_t)2 * nm * T.nkb * kOpBlock * sizeof(__half);
+  const size_t ob = analysis_op_bytes(nm, T.nkb);
   __half* op = (__half*)scratch(ctx, 8, ob + sizeof(int) * 2 * nm * kCols);
   if (!op) return CLC_ENOMEM;
   int* colexp = (int*)((uint8_t*)op + ob);
@@ -986,7 +1071,7 @@ int legendre_analysis_cols(clc_ctx* ctx, const LegendreTable& T, int nv, const d
 template <bool kPoisson>
 static int synthesis(clc_ctx* ctx, const LegendreTable& T, const SynthRhs& s, double2* G, int ld) {
   const int nm = T.m1 - T.m0, nblk = T.h_gidx[2 * nm];
-  const size_t ob = (size_t)nblk * kOpBlock * sizeof(__half);
+  const size_t ob = synthesis_op_bytes(nblk);
   __half* op = (__half*)scratch(ctx, 9, ob + sizeof(int) * 2 * nm * kCols);
   if (!op) return CLC_ENOMEM;
   int* colexp = (int*)((uint8_t*)op + ob);

@@ -21,6 +21,7 @@ constexpr int kAtom = 4096;     // halves of one digit plane of a 64 x 64 atom
 struct LegendreTable {
   int nside = 0, lmax = 0, R = 0, nkb = 0;
   int m0 = 0, m1 = 0;                            // orders held
+  size_t bytes = 0;                              // of the atoms
   std::vector<int> h_gidx;                       // first row block of each group (2 nm + 1)
   Buffer gidx;                                   // the same on the device
   Buffer rb0;                                    // int: first ring block kept, per row block
@@ -34,18 +35,27 @@ struct LegendreTable {
   Buffer eps;
   const double* eps_of() const { return (const double*)eps.p; }
   const double* by_l() const { return (const double*)eps.p + (size_t)(m1 - m0) * (lmax + 3); }
-  std::vector<std::unique_ptr<Buffer>> atoms;    // the atoms, in pieces
+  std::vector<std::unique_ptr<Buffer>> atoms;    // the atoms, a piece per segment of a table that stays, else one arena
+  bool arena = false;
   Buffer an, sy;                                 // work lists of the contractions (int4), longest first
   int n_an = 0, n_sy = 0;
 };
 
-// The whole table of (nside, lmax), cached in the context.
-std::shared_ptr<LegendreTable> get_legendre_table(clc_ctx* ctx, int nside, int lmax, int* rc);
-// A table of the orders m0 <= m < m1 only (caller-owned; for solves whose
-// whole table does not fit in device memory).
-int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, LegendreTable* T);
-// bytes such a table needs at most
-size_t legendre_table_bytes(int nside, int lmax, int m0, int m1);
+// Buffers of a build, kept from one range of orders to the next.
+struct LegendreBuild {
+  Buffer tab, ab, ln, off, grp;
+};
+// A table of the orders from m0 on, up to m1 - 1, that fit `limit` bytes of atoms
+// (at least one order); T->m1 tells where it ends.  stays: the table may stay,
+// fill the limit as far as it goes with memory of its size; otherwise one arena of
+// the limit, and an end where the rest would cost another segment.  T may hold an
+// earlier range: its buffers are used again.
+int build_legendre_table(clc_ctx* ctx, int nside, int lmax, int m0, int m1, size_t limit, bool stays, LegendreBuild& W,
+                         LegendreTable* T);
+// The table to use for the orders from m0 on: the context's, or one built into
+// `own` (made if null).
+int legendre_table_from(clc_ctx* ctx, int nside, int lmax, int m0, LegendreBuild& W,
+                        std::shared_ptr<LegendreTable>& own, std::shared_ptr<LegendreTable>* T);
 
 // packed index of (l, m) for band limit lmax (m-major)
 __host__ __device__ __forceinline__ long long alm_idx(int lmax, int l, int m) {
@@ -78,42 +88,25 @@ int legendre_synthesis(clc_ctx* ctx, const LegendreTable& T, const double2* rhs,
 // -l (l + 1) psi_lm.
 int legendre_synthesis_poisson(clc_ctx* ctx, const LegendreTable& T, const double2* klm, int nq, double2* G, int ld);
 
-// Run fn on tables covering every order m <= lmax: the cached whole table
-// when it fits in device memory (or the context's budget), otherwise tables
-// of consecutive order ranges built one after the other, each freed before
-// the next (the recurrence is then recomputed per call).
+// Run fn on tables covering every order m <= lmax: the context's whole table
+// when it fits in device memory (or the context's budget), otherwise tables of
+// consecutive order ranges built one after the other in the same memory (the
+// recurrence is then recomputed per call).
 template <typename Fn>
 int for_each_table(clc_ctx* ctx, int nside, int lmax, Fn fn) {
-  int rc;
-  const bool cached = ctx->leg_tables.count(std::make_tuple(nside, lmax, 0)) > 0;
-  size_t freeb = 0, totalb = 0;
-  cudaMemGetInfo(&freeb, &totalb);
-  const size_t whole = legendre_table_bytes(nside, lmax, 0, lmax + 1);
-  const bool limited = ctx->table_budget > 0 && whole > ctx->table_budget;
-  if (!limited && (cached || whole + (6ull << 30) <= freeb)) {
-    auto T = get_legendre_table(ctx, nside, lmax, &rc);
-    if (rc) return rc;
-    return fn(*T);
-  }
-  size_t budget = freeb > (16ull << 30) ? freeb - (16ull << 30) : freeb / 4;
-  if (budget > (48ull << 30)) budget = 48ull << 30;
-  if (ctx->table_budget > 0 && ctx->table_budget < budget) budget = ctx->table_budget;
+  LegendreBuild W;
+  std::shared_ptr<LegendreTable> own;
+  size_t bytes = 0;
   for (int m0 = 0; m0 <= lmax;) {
-    int m1 = m0 + 1;
-    size_t b = legendre_table_bytes(nside, lmax, m0, m1);
-    while (m1 <= lmax) {
-      const size_t nb = legendre_table_bytes(nside, lmax, m1, m1 + 1);
-      if (b + nb > budget) break;
-      b += nb;
-      ++m1;
-    }
-    LegendreTable T;
-    if ((rc = build_legendre_table(ctx, nside, lmax, m0, m1, &T))) return rc;
-    if ((rc = fn(T))) return rc;
-    if ((rc = cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "table chunk"))) return rc;
-    m0 = m1;
+    std::shared_ptr<LegendreTable> T;
+    int rc = legendre_table_from(ctx, nside, lmax, m0, W, own, &T);
+    if (rc) return rc;
+    if ((rc = fn(*T))) return rc;
+    m0 = T->m1;
+    bytes += T->bytes;
   }
-  return CLC_OK;
+  ctx->leg_bytes[{nside, lmax}] = bytes;
+  return own ? cuda_check(ctx, cudaStreamSynchronize(ctx->stream), "table chunk") : CLC_OK;
 }
 
 }  // namespace clc
