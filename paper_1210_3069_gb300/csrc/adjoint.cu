@@ -246,7 +246,7 @@ __device__ void step_forward(const double x[3], const double be[3], const double
     f.bn[c] = be[c];
   }
   const double a2 = dot3s(f.av, f.av);
-  f.turned = a2 > 0.0;
+  f.turned = a2 >= 0.0;   // zero too: beta's derivative by alpha does not vanish there; a NaN alone turns nothing
   if (f.turned) {
     cross3s(f.n, f.av, f.kk);
     if (a2 < 0.0009765625) {   // Maclaurin series in a^2, first omitted terms below 1e-19
