@@ -185,17 +185,24 @@ __global__ void k_mg_setup_defect(int n, const double* __restrict__ rot, const d
   if (threadIdx.x == 0 && ff != 0.0) atomicAdd(fnorm + b, ff);
 }
 
-// Plan entry of the mixed-precision set-up: the first pixel on each of the two
-// rings (the second one follows it, or with kWrap set begins the ring; indices
-// stay below 2^30 up to nside 8192), the positions fa, fb between them and w
-// between the rings as float-float pairs.  Entries that need the 8-pixel polar
-// stencil have pa = -1 and (theta, phi) in FP64 in fa, fb.  32 bytes in one load;
-// four indices and four weights took 48.
+// Plan entry of the mixed-precision set-up: on each of the two rings, the nearer
+// one first, the pixel nearer to the position (indices stay below 2^30 up to
+// nside 8192), and as float-float pairs the fractions fa, fb of the way to the
+// other pixel and w of the way to the farther ring.  The other pixel follows the
+// nearer one, or precedes it (kBack); with kWrap it is the ring's first or last.
+// Entries that need the 8-pixel polar stencil have pa = kPolar and (theta, phi) in
+// FP64 in fa, fb.  32 bytes in one load; four indices and four weights took 48.
+// Fractions of at most 1/2 keep the error of near + f (far - near) relative to the
+// terms of the weighted sum: 2^-49.1 .. 2^-48.8 rms, like four weights of 48 bits
+// each (see apply_plan_ff).  From the first pixel on, with fractions close to 1, a
+// small weight of a large pixel lost its low bits (2^-48.1 rms on a random
+// map, 2^-45.8 with peaks).
 struct alignas(32) PlanFF {
   float2 fa, fb, w;
   int pa, pb;
 };
-constexpr int kWrap = 1 << 30;
+constexpr int kBack = 1 << 30, kIndex = kBack - 1, kWrap = (int)0x80000000;
+constexpr int kPolar = kWrap;   // (pixel 0 is the first of its ring: wrapped only with kBack)
 
 // Interpolation plan of one map for the positions of a patch level: either
 // all (n+2)^2 positions (ring = 1) or the n^2 interior cells (ring = 0).  Four
@@ -217,18 +224,23 @@ __global__ void k_mg_plan(int n, int ring, const double* __restrict__ rot, const
   const bool polar = o.w[4] != 0.0 || o.w[5] != 0.0;
   if (!idx) {
     PlanFF q{};
-    q.pa = -1;
+    q.pa = kPolar;
     if (polar) {
       *reinterpret_cast<double*>(&q.fa) = th;
       *reinterpret_cast<double*>(&q.fb) = ph;
     } else {
       // fractions back from the weights (1 - w)(1 - fa), (1 - w) fa, w (1 - fb), w fb
-      const double wa = o.w[0] + o.w[1], wb = o.w[2] + o.w[3];
-      q.pa = (int)o.p[0] | (o.p[1] != o.p[0] + 1 ? kWrap : 0);
-      q.pb = (int)o.p[2] | (o.p[3] != o.p[2] + 1 ? kWrap : 0);
-      q.fa = from_double<float2>(wa > 0.0 ? o.w[1] / wa : 0.0);
-      q.fb = from_double<float2>(wb > 0.0 ? o.w[3] / wb : 0.0);
-      q.w = from_double<float2>(wb);
+      const double wr[2] = {o.w[0] + o.w[1], o.w[2] + o.w[3]};
+      const int near = wr[1] > wr[0] ? 1 : 0;
+      auto ring = [&](int r, int* p) {
+        const double w0 = o.w[2 * r], w1 = o.w[2 * r + 1];
+        const bool back = w1 > w0;
+        *p = (back ? (int)o.p[2 * r + 1] | kBack : (int)o.p[2 * r]) | (o.p[2 * r + 1] != o.p[2 * r] + 1 ? kWrap : 0);
+        return from_double<float2>(wr[r] > 0.0 ? (back ? w0 : w1) / wr[r] : 0.0);
+      };
+      q.fa = ring(near, &q.pa);
+      q.fb = ring(1 - near, &q.pb);
+      q.w = from_double<float2>(wr[1 - near]);
     }
     reinterpret_cast<PlanFF*>(w)[pos] = q;
     return;
@@ -248,17 +260,27 @@ __global__ void k_split_ff(const double* __restrict__ src, float2* __restrict__ 
     dst[k] = from_double<float2>(src[k]);
 }
 
+// The neighbour across longitude zero of the pixel of an entry with kWrap: the
+// first pixel of its ring, or (kBack) the last.
+__device__ __forceinline__ int wrapped_pixel(int nside, int e) {
+  int64_t j;
+  const int i = pix2ring(nside, e & kIndex, &j);
+  return (e & kBack) ? (e & kIndex) + 4 * min(min(i, 4 * nside - i), nside) - 1 : (e & kIndex) - (int)j;
+}
+
 // Plan interpolation of kRows positions in float-float arithmetic (FP32 pipe):
 // all entries, then all pixels are in flight before the first use (one position
 // after the other, each behind the branch to the FP64 form, waits twice for
-// memory per position); entries with pa < 0 in FP64 at the end.  Bound by
+// memory per position); polar entries in FP64 at the end.  Bound by
 // instructions in flight (IPC 1.9, a quarter of the warps): two positions at a
 // time leave more warps than four and wait less than one (defect 3033, 3616,
-// 3451 us at Nside 1024, 201M cells), and sums with one two-sum, accurate
-// relative to their terms, take a third of the instructions out.  Base and
-// defect: 2500 + 3039 us with 48-byte entries of four weights, full sums and
-// one position at a time, 2097 + 2790 us now.
-template <int kRows>
+// 3451 us at Nside 1024, 201M cells).  kLite: the weighted sums by one two-sum
+// (differences always), for the smooth potential, whose rms error relative to the
+// terms is 2^-49.20 so (2^-49.00 with four weights); 2^-49.00 on a lognormal map,
+// where full sums reach 2^-49.14 (four weights 2^-49.07), which kappa gets.
+// Base and defect: 2502 + 3038 us with 48-byte entries of four weights, full sums
+// and one position at a time, 2080 + 2935 now (2202 + 2932 with full sums in both).
+template <int kRows, bool kLite>
 __device__ __forceinline__ void apply_plan_ff(const float2* __restrict__ map_ff, const double* __restrict__ map,
                                               int nside, const double* __restrict__ ring_th,
                                               const PlanFF* __restrict__ plan, const size_t pos[kRows],
@@ -270,11 +292,12 @@ __device__ __forceinline__ void apply_plan_ff(const float2* __restrict__ map_ff,
     r[k] = ok[k] ? reinterpret_cast<const double4_32a*>(plan)[pos[k]] : double4_32a{0.0, 0.0, 0.0, 0.0};
 #pragma unroll
   for (int k = 0; k < kRows; ++k) {
-    int pa = max(__double2loint(r[k].w), 0), pb = __double2hiint(r[k].w), pa1 = pa + 1, pb1 = pb + 1;
-    if ((pa | pb) & kWrap) {
-      int64_t ja, jb;
-      if (pa & kWrap) { pa ^= kWrap; pix2ring(nside, pa, &ja); pa1 = pa - (int)ja; }
-      if (pb & kWrap) { pb ^= kWrap; pix2ring(nside, pb, &jb); pb1 = pb - (int)jb; }
+    const int ea = __double2loint(r[k].w), eb = __double2hiint(r[k].w);
+    const int pa = ea & kIndex, pb = eb & kIndex;
+    int pa1 = pa + 1 - ((ea >> 29) & 2), pb1 = pb + 1 - ((eb >> 29) & 2);
+    if ((ea | eb) < 0) {   // (polar entries: pixel 0, not used)
+      if (ea < 0) pa1 = wrapped_pixel(nside, ea);
+      if (eb < 0) pb1 = wrapped_pixel(nside, eb);
     }
     m[k][0] = map_ff[pa];
     m[k][1] = map_ff[pa1];
@@ -282,18 +305,19 @@ __device__ __forceinline__ void apply_plan_ff(const float2* __restrict__ map_ff,
     m[k][3] = map_ff[pb1];
   }
   auto ff = [](double x) { return make_float2(__int_as_float(__double2loint(x)), __int_as_float(__double2hiint(x))); };
+  auto add = [](float2 a, float2 b) { return kLite ? ff_add_lite(a, b) : ff_add(a, b); };
   bool general = false;
 #pragma unroll
   for (int k = 0; k < kRows; ++k) {
-    const float2 a = ff_add_lite(m[k][0], ff_mul(ff(r[k].x), ff_add_lite(m[k][1], ff_neg(m[k][0]))));
-    const float2 b = ff_add_lite(m[k][2], ff_mul(ff(r[k].y), ff_add_lite(m[k][3], ff_neg(m[k][2]))));
-    v[k] = ff_add_lite(a, ff_mul(ff(r[k].z), ff_add_lite(b, ff_neg(a))));
-    general |= __double2loint(r[k].w) < 0;
+    const float2 a = add(m[k][0], ff_mul(ff(r[k].x), ff_add_lite(m[k][1], ff_neg(m[k][0]))));
+    const float2 b = add(m[k][2], ff_mul(ff(r[k].y), ff_add_lite(m[k][3], ff_neg(m[k][2]))));
+    v[k] = add(a, ff_mul(ff(r[k].z), ff_add_lite(b, ff_neg(a))));
+    general |= __double2loint(r[k].w) == kPolar;
   }
   if (general) {
 #pragma unroll
     for (int k = 0; k < kRows; ++k)
-      if (__double2loint(r[k].w) < 0) v[k] = from_double<float2>(interp_map_tab(map, nside, ring_th, r[k].x, r[k].y));
+      if (__double2loint(r[k].w) == kPolar) v[k] = from_double<float2>(interp_map_tab(map, nside, ring_th, r[k].x, r[k].y));
   }
 }
 
@@ -315,7 +339,7 @@ __global__ void k_mg_setup_base_ff(int n, const PlanFF* __restrict__ plan, const
     ok[k] = k0 + k < side && k2 < side;
     pos[k] = (size_t)b * side * side + (size_t)(k0 + k) * side + k2;
   }
-  apply_plan_ff<kPlanRows>(psi_ff, psi, ns, ring_th, plan, pos, ok, v);
+  apply_plan_ff<kPlanRows, true>(psi_ff, psi, ns, ring_th, plan, pos, ok, v);
 #pragma unroll
   for (int k = 0; k < kPlanRows; ++k) {
     if (!ok[k]) continue;
@@ -349,7 +373,7 @@ __global__ void k_mg_setup_defect_ff(int n, const PlanFF* __restrict__ plan, con
         ok[k] = i0 + c + k < n;
         pos[k] = (size_t)b * n * n + (size_t)(i0 + c + k) * n + j;
       }
-      apply_plan_ff<kPlanRows>(kap_ff, kappa, nf, ring_th, plan, pos, ok, src);
+      apply_plan_ff<kPlanRows, false>(kap_ff, kappa, nf, ring_th, plan, pos, ok, src);
 #pragma unroll
       for (int k = 0; k < kPlanRows; ++k) {
         if (!ok[k]) continue;
