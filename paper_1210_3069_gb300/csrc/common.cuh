@@ -374,6 +374,7 @@ __device__ __forceinline__ int ring_above(int nside, double z, double s) {
 struct Interp8 {
   int64_t p[8];
   double w[8];
+  double f[3];   // without the polar stencil: fractions between the rings and along each of them
 };
 
 // Two pixels of ring r bracketing phi and the weight of the second
@@ -402,6 +403,7 @@ __device__ __forceinline__ Interp8 interp_weights_tab(int nside, const double* _
   while (i1 + 1 <= nr && ring_th[i1] <= theta) ++i1;
 #pragma unroll
   for (int k = 0; k < 8; ++k) { o.p[k] = 0; o.w[k] = 0.0; }
+  o.f[0] = o.f[2] = 0.0;
   if (i1 == 0 || i1 == nr) {
     const int ir = (i1 == 0) ? 1 : nr;
     const double tr = ring_th[ir - 1];
@@ -411,6 +413,7 @@ __device__ __forceinline__ Interp8 interp_weights_tab(int nside, const double* _
     ring_pair(nside, ir, phi, &a0, &a1, &fa);
     o.p[0] = a0; o.w[0] = w * (1.0 - fa);
     o.p[1] = a1; o.w[1] = w * fa;
+    o.f[1] = fa;   // (all there is on the last ring itself)
     const Ring r = ring_geom(nside, ir);
 #pragma unroll
     for (int k = 0; k < 4; ++k) { o.p[4 + k] = r.first + k; o.w[4 + k] = (1.0 - w) * 0.25; }
@@ -426,6 +429,9 @@ __device__ __forceinline__ Interp8 interp_weights_tab(int nside, const double* _
   o.p[1] = a1; o.w[1] = (1.0 - w) * fa;
   o.p[2] = b0; o.w[2] = w * (1.0 - fb);
   o.p[3] = b1; o.w[3] = w * fb;
+  o.f[0] = w;
+  o.f[1] = fa;
+  o.f[2] = fb;
   return o;
 }
 

@@ -206,8 +206,9 @@ constexpr int kPolar = kWrap;   // (pixel 0 is the first of its ring: wrapped on
 
 // Interpolation plan of one map for the positions of a patch level: either
 // all (n+2)^2 positions (ring = 1) or the n^2 interior cells (ring = 0).  Four
-// indices and FP64 weights, or (idx null) PlanFF entries in w.  Entries that
+// indices and FP64 weights, or (kFF) PlanFF entries in w.  Entries that
 // need the 8-pixel polar stencil keep (theta, phi) in FP64 with index -1.
+template <bool kFF>
 __global__ void k_mg_plan(int n, int ring, const double* __restrict__ rot, const double* __restrict__ pvec, int nside,
                           const double* __restrict__ ring_th, int4* __restrict__ idx,
                           double4_32a* __restrict__ w) {
@@ -222,25 +223,26 @@ __global__ void k_mg_plan(int n, int ring, const double* __restrict__ rot, const
   const Interp8 o = interp_weights_tab(nside, ring_th, th, ph);
   const size_t pos = (size_t)b * m * m + (size_t)k1 * m + k2;
   const bool polar = o.w[4] != 0.0 || o.w[5] != 0.0;
-  if (!idx) {
+  if constexpr (kFF) {
     PlanFF q{};
     q.pa = kPolar;
     if (polar) {
       *reinterpret_cast<double*>(&q.fa) = th;
       *reinterpret_cast<double*>(&q.fb) = ph;
     } else {
-      // fractions back from the weights (1 - w)(1 - fa), (1 - w) fa, w (1 - fb), w fb
-      const double wr[2] = {o.w[0] + o.w[1], o.w[2] + o.w[3]};
-      const int near = wr[1] > wr[0] ? 1 : 0;
+      // FP64-pipe bound: 1 - f (exact for f >= 1/2) instead of quotients of the
+      // weights, 152 instead of 171 ms for the 405M positions of nside 1024
+      auto half = [](double f) { return __double2hiint(f) >= 0x3fe00000; };   // f >= 1/2, off the FP64 pipe
+      const int near = half(o.f[0]) ? 1 : 0;
       auto ring = [&](int r, int* p) {
-        const double w0 = o.w[2 * r], w1 = o.w[2 * r + 1];
-        const bool back = w1 > w0;
+        const double f = o.f[1 + r];
+        const bool back = half(f);
         *p = (back ? (int)o.p[2 * r + 1] | kBack : (int)o.p[2 * r]) | (o.p[2 * r + 1] != o.p[2 * r] + 1 ? kWrap : 0);
-        return from_double<float2>(wr[r] > 0.0 ? (back ? w0 : w1) / wr[r] : 0.0);
+        return from_double<float2>(back ? 1.0 - f : f);
       };
       q.fa = ring(near, &q.pa);
       q.fb = ring(1 - near, &q.pb);
-      q.w = from_double<float2>(wr[1 - near]);
+      q.w = from_double<float2>(near ? 1.0 - o.f[0] : o.f[0]);
     }
     reinterpret_cast<PlanFF*>(w)[pos] = q;
     return;
@@ -3148,12 +3150,13 @@ static int solution_create(clc_ctx* ctx, int nf, const clc_mg_params* p, const i
         (!mx || (alloc(s->base_ff, pr * sizeof(float2)) && alloc(s->psi_ff, ns2 * sizeof(float2)) &&
                  alloc(s->kap_ff, nf2 * sizeof(float2))))) {
       const dim3 blk(kBX, kBY);
-      CLC_LAUNCH(ctx, "k_mg_plan", k_mg_plan, grid3(n0 + 2, n0 + 2, s->npatch), blk, 0, (int)n0, 1,
-                 (const double*)s->rot.p, (const double*)s->pvec.p, p->nside_sht, (const double*)s->ring_th_sht.p,
-                 (int4*)s->plan_psi_idx.p, (double4_32a*)s->plan_psi_w.p);
-      CLC_LAUNCH(ctx, "k_mg_plan", k_mg_plan, grid3(n0, n0, s->npatch), blk, 0, (int)n0, 0, (const double*)s->rot.p,
-                 (const double*)s->pvec.p, nf, (const double*)s->ring_th_fine.p, (int4*)s->plan_kap_idx.p,
-                 (double4_32a*)s->plan_kap_w.p);
+      auto plan = [&](int m, int ring, const clc::Buffer& th, int nside, clc::Buffer& idx, clc::Buffer& w) {
+        CLC_LAUNCH(ctx, "k_mg_plan", (mx ? k_mg_plan<true> : k_mg_plan<false>), grid3(m, m, s->npatch), blk, 0, (int)n0, ring,
+                   (const double*)s->rot.p, (const double*)s->pvec.p, nside, (const double*)th.p, (int4*)idx.p,
+                   (double4_32a*)w.p);
+      };
+      plan((int)n0 + 2, 1, s->ring_th_sht, p->nside_sht, s->plan_psi_idx, s->plan_psi_w);
+      plan((int)n0, 0, s->ring_th_fine, nf, s->plan_kap_idx, s->plan_kap_w);
       s->plan = true;
     }
   }
