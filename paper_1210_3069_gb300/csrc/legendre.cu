@@ -1036,6 +1036,97 @@ static DigArgs dig_args(const LegendreTable& T, const __half* op, const int* col
   return a;
 }
 
+// The analysis of one map at low band limits, straight in FP64 on the values the
+// digits stand for: a warp per (l, m), its lanes over eight neighbouring rings of
+// a row (one 16-byte word per digit plane).  Packing, the contraction's pipeline and
+// its walk over the rings take 27 us at nside 128 and 64 at nside 512 however small
+// lmax is (the FP64 sums before: 10 and 20 at lmax 16); this way 9.6 and 19.  It is
+// FP64 bound (three instructions per value) and grows with lmax^2: it saves 7, 14
+// and 20 us at nside 128, 256 and 512 with lmax 100, and loses 5 at the first two
+// with lmax 128.
+constexpr int kRowsLmax = 112;
+constexpr int kRowsChunk = 1024;   // rings held at a time
+
+// place of ring t of a chunk: lanes read eight rings each, from different banks
+__device__ __forceinline__ int rows_at(int t) { return (t & ~7) | ((t ^ (t >> 3)) & 7); }
+
+__global__ void __launch_bounds__(256) k_legendre_rows(DigArgs a, const double2* __restrict__ Fm, int ldf) {
+  __shared__ double2 V[2][kRowsChunk];   // north + (-1)^p south, times 2^(-31 - cexp)
+  const int ml = blockIdx.y, m = a.m0 + ml, lane = threadIdx.x & 31;
+  const int l = m + blockIdx.x * 8 + (threadIdx.x >> 5), p = (l - m) & 1, row = ((l - m) >> 1) & 63;
+  const bool on = l <= a.ltop;
+  int first = a.nkb, er = 0;
+  const __half* base = nullptr;
+  if (on) {
+    const int blk = a.gidx[2 * ml + p] + ((l - m) >> 7);
+    first = a.rb0[blk];
+    base = a.abase[blk];
+    er = a.rexp[(size_t)blk * 64 + row];
+  }
+  const double2* F = Fm + (size_t)m * ldf;
+  const int8_t* cx = a.cexp + (size_t)ml * a.nkb * 64;
+  double sx = 0.0, sy = 0.0;
+  for (int r0 = 0; r0 < a.R; r0 += kRowsChunk) {
+    const int n = min(kRowsChunk, a.R - r0);
+    __syncthreads();   // the previous chunk is consumed
+    for (int t = threadIdx.x; t < n; t += 256) {
+      const int r = r0 + t;
+      const double2 u = F[r];
+      double2 v = make_double2(0.0, 0.0);
+      if (r + 1 != 2 * a.nside) v = F[4 * a.nside - r - 2];
+      const double w = __longlong_as_double((long long)(1023 - 31 - (int)cx[r]) << 52);
+      V[0][rows_at(t)] = make_double2((u.x + v.x) * w, (u.y + v.y) * w);
+      V[1][rows_at(t)] = make_double2((u.x - v.x) * w, (u.y - v.y) * w);
+    }
+    __syncthreads();
+    if (!on) continue;
+    for (int c = 8 * lane; c < n; c += 256) {
+      const int rb = (r0 + c) >> 6;
+      unsigned long long y[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) y[q] = rb < first ? 0x8080808080808080ull : 0;
+      if (rb >= first) {
+        const __half* atom = base + (size_t)(rb - first) * kDigits * kAtom + dig_off(row, c & 63);
+#pragma unroll
+        for (int s = 0; s < kDigits; ++s) {
+          const uint4 d = *reinterpret_cast<const uint4*>(atom + s * kAtom);
+          const unsigned w[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {   // digit + 1152 has digit + 128 as its low byte
+            const __half2 h = __hadd2(*reinterpret_cast<const __half2*>(&w[j]), __half2half2(__ushort_as_half(0x6480)));
+            const unsigned b = *reinterpret_cast<const unsigned*>(&h);
+            y[2 * j] |= (unsigned long long)(b & 255u) << 8 * (kDigits - 1 - s);
+            y[2 * j + 1] |= (unsigned long long)((b >> 16) & 255u) << 8 * (kDigits - 1 - s);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        if (c + q >= n) break;
+        const double lam = (double)(long long)(y[q] - 0x8080808080808080ull);
+        const double2 v = V[p][rows_at(c + q)];
+        sx = fma(lam, v.x, sx);   // (also where lambda is zero: a NaN is not hidden)
+        sy = fma(lam, v.y, sy);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sx += __shfl_xor_sync(0xffffffffu, sx, o);
+    sy += __shfl_xor_sync(0xffffffffu, sy, o);
+  }
+  if (on && lane == 0)
+    a.out[0][alm_idx(a.ltop, l, m)] = make_double2(times_pow2(sx, er - 31), times_pow2(sy, er - 31));
+}
+
+static int analysis_rows(clc_ctx* ctx, const LegendreTable& T, const double2* F, int ldf, double2* out, int ltop) {
+  DigArgs a = dig_args(T, nullptr, nullptr);
+  a.out[0] = out;
+  a.ltop = ltop;
+  CLC_LAUNCH(ctx, "k_legendre_analysis", k_legendre_rows, dim3((ltop - T.m0) / 8 + 1, T.m1 - T.m0), 256, 0, a, F, ldf);
+  return launch_check(ctx, "k_legendre_rows");
+}
+
 template <int NC>
 static int analysis_cols(clc_ctx* ctx, const LegendreTable& T, const AnaCols& c, int ldf, double2* const* out, int ltop) {
   const int nm = T.m1 - T.m0;
@@ -1056,6 +1147,7 @@ static int analysis_cols(clc_ctx* ctx, const LegendreTable& T, const AnaCols& c,
 int legendre_analysis_cols(clc_ctx* ctx, const LegendreTable& T, int nv, const double2* const* F, const int* kind,
                            int ldf, double2* const* out, int ltop) {
   if (ltop < 0) ltop = T.lmax;
+  if (nv == 1 && !kind && T.lmax <= kRowsLmax) return analysis_rows(ctx, T, F[0], ldf, out[0], ltop);
   AnaCols c{};
   c.nv = nv;
   for (int v = 0; v < nv; ++v) {
