@@ -231,8 +231,12 @@ int ring_analysis_t(clc_ctx* ctx, const FftPlan& plan, int n, const double* cons
   RingMaps a{};
   for (int k = 0; k < n; ++k) a.map[k] = maps[k];
   cudaFuncSetAttribute(k_ring_analysis<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // A single map's blocks do not fill the SMs at the longest rings: twice the
+  // threads from 2048 points on (nside 512: 404 -> 365 us; at nside 128 49 -> 56, at
+  // 256 116 -> 127, and two maps at 256 lose 20)
+  const int threads = std::max(n == 1 && plan.mmax_fft >= 2048 ? 256 : 128, ring_fft_threads(plan.mmax_fft));
   CLC_LAUNCH(ctx, "k_ring_analysis", (k_ring_analysis<T>), dim3(4 * nside - 1, n),
-             std::max(128, ring_fft_threads(plan.mmax_fft)), smem, a, nside, lmax, weight, F, fstride, ldf,
+             threads, smem, a, nside, lmax, weight, F, fstride, ldf,
              plan_dev<T>(plan));
   return launch_check(ctx, "k_ring_analysis");
 }
