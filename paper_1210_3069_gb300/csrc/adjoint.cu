@@ -33,7 +33,6 @@ namespace clc {
 
 // the dual-number overloads below must not hide the FP64 math functions
 using ::atan2;
-using ::sincos;
 using ::sqrt;
 
 // ---------------------------------------------------------------------------
@@ -136,18 +135,6 @@ __device__ __forceinline__ Dual<K> sqrt(const Dual<K>& a) {
 #pragma unroll
   for (int k = 0; k < K; ++k) r.d[k] = a.d[k] * h;
   return r;
-}
-template <int K>
-__device__ __forceinline__ void sincos(const Dual<K>& a, Dual<K>* s, Dual<K>* c) {
-  double sv, cv;
-  ::sincos(a.v, &sv, &cv);
-  s->v = sv;
-  c->v = cv;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    s->d[k] = cv * a.d[k];
-    c->d[k] = -sv * a.d[k];
-  }
 }
 template <int K>
 __device__ __forceinline__ Dual<K> atan2(const Dual<K>& y, const Dual<K>& x) {

@@ -16,10 +16,17 @@
 // that FP16 holds exactly.  Digit products are at most 2^14, so an FP32
 // accumulator adds the up to 8 digit pairs i + j = g of 128 terms without
 // rounding (8 * 128 * 2^14 = 2^24); the sums of each g <= 7 are collected in
-// 64-bit integers and rounded once.  Digit pairs with g > 7 lie below 2^-62 of
-// the largest term and are left out.  The result does not depend on the order
-// of summation.  Rings where lambda_lm is small for every l (towards the
-// poles) are scaled up by 2^cexp <= 2^24 first.
+// 64-bit integers and rounded once.  Digit pairs with g > 7 are left out: at most
+// seven of a term reach 2^-62 of the product of the scales, so a term loses less
+// than 2^-59 of it.  The result does not depend on the order of summation.  Rings
+// where lambda_lm is small for every l (towards the poles) are scaled up by
+// 2^cexp <= 2^24 first.
+//   The error is thus relative to the scales, the largest |lambda_lm| 2^cexp of the
+// row and the largest |value| 2^-cexp of the column, not to each term: as small as
+// that of FP64 sums (2^-53 of the largest term) while the rings (or degrees) of a
+// column differ by less than about 2^33 where lambda_lm is small, which sources,
+// shears and their coefficients do; a column with larger contrasts keeps fewer
+// bits in the sums that its largest values hardly enter.
 //
 // Eight digits, not seven: the scale is the largest value of a row or column,
 // while the FP64 sums this replaces keep every term's own 53 bits.  Near the
@@ -34,8 +41,9 @@
 // 0.42e12 values per second) a value serves up to 16 columns at once, so both
 // directions are bound by the table traffic.  At nside 512, lmax 1024 the
 // FP64 kernels took 2.2 ms (analysis), 11.8 ms (synthesis of the three sums)
-// and 53.4 ms (spin-2 sums of two fields); the solve went from 19.2 to 7.8 ms
-// and the four spectra from 63.2 to 7.1 ms.
+// and 53.4 ms (spin-2 sums of two fields); with them the solve took 19.2 ms and
+// the four spectra 63.2, with the digits 7.8 and 7.1 (6.05 and 4.02 with the ring
+// FFTs of now).
 #include <algorithm>
 #include <cmath>
 

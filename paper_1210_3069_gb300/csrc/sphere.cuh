@@ -1,6 +1,6 @@
-// Vectors and tangent frames on the unit sphere shared by the ray recursion
-// and the image search: the (theta-hat, phi-hat) basis, Rodrigues rotation
-// and the parallel transport of Appendix B.
+// Vectors and tangent frames on the unit sphere shared by the ray recursion,
+// the image search and the spectra: products, the (theta-hat, phi-hat) basis and
+// the change of basis of a 2x2 matrix.
 #pragma once
 
 #include <cuda_runtime.h>
