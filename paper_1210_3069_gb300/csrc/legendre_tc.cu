@@ -27,6 +27,8 @@
 #include <algorithm>
 #include <map>
 
+#include <cuda_pipeline.h>
+
 #include "legendre_tc.cuh"
 #include "ring_fft.cuh"
 #include "legendre.cuh"
@@ -267,12 +269,14 @@ __global__ void __launch_bounds__(kRingThreads, 2) k_tc_ring_synthesis(TcBatchDe
 // (sin theta < 0.29) need them.
 //
 // lambda of the two orders on those rings is kept with the batch (it depends on
-// neither plane nor map), so the sums have no recurrence and split over l: a
-// block takes one (plane, order) on 32 northern rings (and their mirrors by the
-// parity of l + m), its eight warps every eighth l, the l-dependent factors
-// staged once.  One thread per (plane, ring) running the recurrence through
-// every l took 1.33 ms of the 2.25 ms of a batch of 12 small planes (now 0.04)
-// and 2.67 of the 12.4 ms of 21 planes at nside 512 (now 0.12).
+// neither plane nor map), so the sums have no recurrence: a block takes one
+// quantity of one (plane, order) on 32 northern rings, a warp each the real and the
+// imaginary part (0 for m = 0) on these rings and on their mirrors, the l-dependent
+// factors staged once.  The sums run through l in order: split over l (119 us) they
+// differ in the last FP64 bit, which in one batch of five turned the FP32 rounding
+// of a ring coefficient (5e-8 of the largest value of one field of one plane).
+// FP64 bound, one FMA per term and hemisphere, a warp's in 64 clocks: 68 us for
+// one plane at nside 512, 165 for 21 (with the recurrence in every thread 2670).
 
 // the unscaled recurrence is safe for m <= 1
 __global__ void k_tc_lam01(int nside, int L, int ncap, const double* __restrict__ co01, double* __restrict__ lam01) {
@@ -303,20 +307,22 @@ int tc_build_lam01(clc_ctx* ctx, const TcClass& C, double* lam01) {
   return launch_check(ctx, "k_tc_lam01");
 }
 
-constexpr int kLowChunk = 512;   // degrees staged at a time
-constexpr int kLowWarps = 8;
+constexpr int kLowChunk = 1024;  // degrees whose factors are staged at a time (a multiple of kLowTile)
+constexpr int kLowThreads = 128;
+constexpr int kLowTile = 32;     // degrees of lambda copied at a time, one tile ahead
 
-__global__ void __launch_bounds__(32 * kLowWarps) k_tc_low_orders(TcBatchDev b) {
-  __shared__ double cf[kLowChunk][6];   // psi, b, kappa_bl (re, im) of a degree
-  __shared__ double red[kLowWarps][12][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(kLowThreads) k_tc_low_orders(TcBatchDev b) {
+  __shared__ double cf[2][kLowChunk];   // re, im of the quantity's coefficients
+  __shared__ __align__(16) double tile[2][kLowTile][32];
+  const int comp = (threadIdx.x >> 5) & 1, lane = threadIdx.x & 31;
+  const bool mirror = threadIdx.x >= 64;   // warps 2, 3: the southern rings
   for (long long it = blockIdx.x; it < b.n_low; it += gridDim.x) {
     const TcClass& C = b.cls[find_class(b, it, &TcClass::low0)];
     const int ld = tc_cap_pad(C.ncap), nc = ld / 32, L = C.lmax, ns = C.nside;
-    const int loc = (int)(it - C.low0), ch = loc % nc, m = (loc / nc) & 1, pl = loc / (2 * nc);
+    const int loc = (int)(it - C.low0), q = loc % 3, ch = loc / 3 % nc, m = (loc / (3 * nc)) & 1, pl = loc / (6 * nc);
     const float2* a = C.alm + pl * C.astride;
     const double* co = C.co01 + (size_t)m * (L + 3) * 4;
-    const double* lam = C.lam01 + (size_t)m * (L + 2) * ld + ch * 32 + lane;
+    const double* lam = C.lam01 + (size_t)m * (L + 2) * ld + ch * 32;
     auto kap = [&](int l) -> double2 {
       if (l < m || l > L || l < 1) return make_double2(0.0, 0.0);
       const float2 v = a[alm_idx(L, l, m)];
@@ -327,58 +333,61 @@ __global__ void __launch_bounds__(32 * kLowWarps) k_tc_low_orders(TcBatchDev b) 
       const double d = (l >= 1 && l <= L) ? co[4 * l + 3] : 0.0;
       return make_double2(k.x * d, k.y * d);
     };
-    double acc[2][6];   // parity of l + m
-#pragma unroll
-    for (int i = 0; i < 6; ++i) acc[0][i] = acc[1][i] = 0.0;
+    double sum = 0.0;
     for (int l0 = m; l0 <= L + 1; l0 += kLowChunk) {
       const int n = min(kLowChunk, L + 2 - l0);
       __syncthreads();
-      for (int t = threadIdx.x; t < n; t += blockDim.x) {
+#pragma unroll 4
+      for (int t = threadIdx.x; t < n; t += kLowThreads) {
         const int l = l0 + t;
-        const double2 p0 = psi(l), pm = psi(l - 1), pp = psi(l + 1), kb = kap(l);
-        const double c1 = (l - 1.0) * co[4 * l + 2], c2 = (l + 2.0) * co[4 * (l + 1) + 2];
-        cf[t][0] = p0.x;
-        cf[t][1] = p0.y;
-        cf[t][2] = c1 * pm.x - c2 * pp.x;
-        cf[t][3] = c1 * pm.y - c2 * pp.y;
-        cf[t][4] = kb.x;
-        cf[t][5] = kb.y;
-      }
-      __syncthreads();
-      // l + m = 2 m + (l - m): even and odd terms alternate from l0 = m + multiples of kLowChunk on
-      for (int t = 2 * warp; t < n; t += 2 * kLowWarps) {
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          if (t + p >= n) break;
-          const double x = lam[(size_t)(l0 + t + p) * ld];
-#pragma unroll
-          for (int i = 0; i < 6; ++i) acc[p][i] = fma(cf[t + p][i], x, acc[p][i]);
+        double2 v;
+        if (q == 0) {
+          v = psi(l);
+        } else if (q == 1) {
+          const double2 pm = psi(l - 1), pp = psi(l + 1);
+          const double c1 = (l - 1.0) * co[4 * l + 2], c2 = (l + 2.0) * co[4 * (l + 1) + 2];
+          v = make_double2(c1 * pm.x - c2 * pp.x, c1 * pm.y - c2 * pp.y);
+        } else {
+          v = kap(l);
         }
+        cf[0][t] = v.x;
+        cf[1][t] = v.y;
+      }
+      auto copy = [&](int t0) {
+        for (int u = threadIdx.x; u < min(kLowTile, n - t0) * 16; u += kLowThreads)
+          __pipeline_memcpy_async(&tile[(t0 / kLowTile) & 1][u >> 4][2 * (u & 15)],
+                                  lam + (size_t)(l0 + t0 + (u >> 4)) * ld + 2 * (u & 15), 16);
+        __pipeline_commit();
+      };
+      copy(0);
+      for (int t0 = 0; t0 < n; t0 += kLowTile) {
+        copy(t0 + kLowTile);
+        __pipeline_wait_prior(1);
+        __syncthreads();   // (the first also completes the factors)
+        if (comp <= m) {   // the imaginary parts of m = 0 stay zero
+          // lambda_l changes sign in the mirror ring for odd l + m = 2 m + (l - m); l0 + t0 - m is even
+          const double* v = cf[comp] + t0;
+          const double(*x)[32] = tile[(t0 / kLowTile) & 1];
+          const int flip = mirror ? (int)0x80000000 : 0;
+          auto add = [&](int k) {
+            const double y = x[k][lane];
+            sum = fma(v[k], (k & 1) ? __hiloint2double(__double2hiint(y) ^ flip, __double2loint(y)) : y, sum);
+          };
+          if (n - t0 >= kLowTile) {
+#pragma unroll
+            for (int k = 0; k < kLowTile; ++k) add(k);
+          } else {
+            for (int k = 0; k < n - t0; ++k) add(k);
+          }
+        }
+        __syncthreads();   // the tile is consumed
       }
     }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      red[warp][i][lane] = acc[0][i];
-      red[warp][6 + i][lane] = acc[1][i];
-    }
-    __syncthreads();
-    double2* out = C.G01 + (size_t)pl * C.nq * 2 * C.ldf;
-    const size_t qs = 2 * (size_t)C.ldf, mo = (size_t)m * C.ldf;
-    if (warp < 3) {   // quantity q = warp
-      double e[2], o[2];
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        e[c] = o[c] = 0.0;
-        for (int w = 0; w < kLowWarps; ++w) {
-          e[c] += red[w][2 * warp + c][lane];
-          o[c] += red[w][6 + 2 * warp + c][lane];
-        }
-      }
-      const int i = ch * 32 + lane + 1;
-      if (i <= C.ncap) {
-        out[warp * qs + mo + i - 1] = make_double2(e[0] + o[0], e[1] + o[1]);
-        if (i != 2 * ns) out[warp * qs + mo + 4 * ns - i - 1] = make_double2(e[0] - o[0], e[1] - o[1]);
-      }
+    const int i = ch * 32 + lane + 1;
+    if (i <= C.ncap) {
+      double* out = reinterpret_cast<double*>(C.G01 + ((size_t)pl * C.nq + q) * 2 * C.ldf + (size_t)m * C.ldf) + comp;
+      if (!mirror) out[2 * (i - 1)] = sum;
+      else if (i != 2 * ns) out[2 * (4 * ns - i - 1)] = sum;
     }
   }
 }
@@ -890,8 +899,8 @@ int tc_run_stage(clc_ctx* ctx, const TcBatchDev& b, const TcItems& it, const TcL
     }
     case 3: {
       if (b.mode && b.n_low > 0) {
-        const int g = (int)std::min<long long>(b.n_low, (long long)num_sms(ctx) * 4);
-        CLC_LAUNCH(ctx, "k_tc_low_orders", k_tc_low_orders, g, 32 * kLowWarps, 0, b);
+        const int g = (int)std::min<long long>(b.n_low, (long long)num_sms(ctx) * 16);
+        CLC_LAUNCH(ctx, "k_tc_low_orders", k_tc_low_orders, g, kLowThreads, 0, b);
         const int rc = launch_check(ctx, "k_tc_low_orders");
         if (rc) return rc;
       }

@@ -171,7 +171,7 @@ static int tc_batch_build(clc_ctx* ctx, int nplanes, const int* nside, const int
     ring0 += (long long)P * (4 * ns - 1);
     pa0 += L + 1;
     ps0 += G;
-    low0 += (long long)P * 2 * (tc_cap_pad(C.ncap) / 32);
+    low0 += (long long)P * 6 * (tc_cap_pad(C.ncap) / 32);
   }
   d.n_ring = ring0;
   d.n_pa = pa0;
