@@ -1051,7 +1051,9 @@ static DigArgs dig_args(const LegendreTable& T, const __half* op, const int* col
 // lmax is (the FP64 sums before: 10 and 20 at lmax 16); this way 9.6 and 19.  It is
 // FP64 bound (three instructions per value) and grows with lmax^2: it saves 7, 14
 // and 20 us at nside 128, 256 and 512 with lmax 100, and loses 5 at the first two
-// with lmax 128.
+// with lmax 128.  For sht_analysis alone: a_lm are off by 1.5e-16 here (1.9e-16 with
+// the FP64 table), where the contraction rounds them once, and a solve, which the
+// difference would reach through its synthesis, gains nothing it needs.
 constexpr int kRowsLmax = 112;
 constexpr int kRowsChunk = 1024;   // rings held at a time
 
@@ -1127,14 +1129,6 @@ __global__ void __launch_bounds__(256) k_legendre_rows(DigArgs a, const double2*
     a.out[0][alm_idx(a.ltop, l, m)] = make_double2(times_pow2(sx, er - 31), times_pow2(sy, er - 31));
 }
 
-static int analysis_rows(clc_ctx* ctx, const LegendreTable& T, const double2* F, int ldf, double2* out, int ltop) {
-  DigArgs a = dig_args(T, nullptr, nullptr);
-  a.out[0] = out;
-  a.ltop = ltop;
-  CLC_LAUNCH(ctx, "k_legendre_analysis", k_legendre_rows, dim3((ltop - T.m0) / 8 + 1, T.m1 - T.m0), 256, 0, a, F, ldf);
-  return launch_check(ctx, "k_legendre_rows");
-}
-
 template <int NC>
 static int analysis_cols(clc_ctx* ctx, const LegendreTable& T, const AnaCols& c, int ldf, double2* const* out, int ltop) {
   const int nm = T.m1 - T.m0;
@@ -1152,10 +1146,18 @@ static int analysis_cols(clc_ctx* ctx, const LegendreTable& T, const AnaCols& c,
   return run_gemm<false, NC>(ctx, "k_legendre_analysis", a, T.an, T.n_an);
 }
 
+int legendre_analysis_map(clc_ctx* ctx, const LegendreTable& T, const double2* F, int ldf, double2* alm) {
+  if (T.lmax > kRowsLmax) return legendre_analysis(ctx, T, F, ldf, alm);
+  DigArgs a = dig_args(T, nullptr, nullptr);
+  a.out[0] = alm;
+  a.ltop = T.lmax;
+  CLC_LAUNCH(ctx, "k_legendre_analysis", k_legendre_rows, dim3((T.lmax - T.m0) / 8 + 1, T.m1 - T.m0), 256, 0, a, F, ldf);
+  return launch_check(ctx, "k_legendre_rows");
+}
+
 int legendre_analysis_cols(clc_ctx* ctx, const LegendreTable& T, int nv, const double2* const* F, const int* kind,
                            int ldf, double2* const* out, int ltop) {
   if (ltop < 0) ltop = T.lmax;
-  if (nv == 1 && !kind && T.lmax <= kRowsLmax) return analysis_rows(ctx, T, F[0], ldf, out[0], ltop);
   AnaCols c{};
   c.nv = nv;
   for (int v = 0; v < nv; ++v) {

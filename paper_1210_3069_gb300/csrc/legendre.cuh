@@ -75,6 +75,9 @@ inline int legendre_analysis(clc_ctx* ctx, const LegendreTable& T, const double2
   return legendre_analysis_cols(ctx, T, 1, &F, nullptr, ldf, &alm, ltop);
 }
 
+// The same of one map up to lmax, summed directly at low band limits.
+int legendre_analysis_map(clc_ctx* ctx, const LegendreTable& T, const double2* F, int ldf, double2* alm);
+
 // G_q[m][ring] = sum_l lambda_lm(ring) rhs_q[idx'(l, m)] for q < nq <= 4, where
 // rhs_q is packed with band limit lmax + 1 (idx' = alm_idx(lmax + 1, l, m)) and
 // lq[q] is the highest l used by rhs q.  G_q lives at G + q * ld * (lmax + 2).

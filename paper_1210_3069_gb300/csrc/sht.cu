@@ -45,7 +45,7 @@ int sht_analysis(clc_ctx* ctx, const double* map, int nside, int lmax, double2* 
   if (!F) return CLC_ENOMEM;
   const double w = 4.0 * kPi / (12.0 * (double)nside * nside);
   if ((rc = ring_analysis(ctx, *plan, map, lmax, w, F, ldf))) return rc;
-  return for_each_table(ctx, nside, lmax, [&](const LegendreTable& T) { return legendre_analysis(ctx, T, F, ldf, alm); });
+  return for_each_table(ctx, nside, lmax, [&](const LegendreTable& T) { return legendre_analysis_map(ctx, T, F, ldf, alm); });
 }
 
 // synthesis of nq right-hand sides (lmax + 1 packing) and the ring FFTs
