@@ -19,7 +19,7 @@
 // the blocks of the longest rings took a quarter of the whole launch each.
 // Six fields, FP64: 4.39 -> 3.02 ms at nside 512 (FP64 pipe 55 -> 80 % busy),
 // 229 -> 78 us at nside 64, where the serial alias sums of the rings next to
-// the poles had set the time; one map, analysis: 0.73 -> 0.50 ms.  Batch of 21
+// the poles had set the time; one map, analysis, lmax 1024: 0.73 -> 0.48 ms.  Batch of 21
 // planes at nside 512, FP32: 16.5 -> 12.5 ms for the whole solve, bit for bit.
 #pragma once
 
